@@ -421,8 +421,8 @@ __global__ void __launch_bounds__(256) adj_push_kernel(GridParams g, const DirIn
     retarded_delay(di.dcoef, di.dcoef_lo, nv_idx, m, f);
     const int L0 = n - m, L1 = n - m - 1;
     const float xo = mu * di.ds;
-    const float T = expf(-xo);
-    const float b0 = ray_b0(xo, T);
+    float T = expf(-xo), b0 = ray_b0(xo, T), b0l;
+    if (g.fine) ray_weights_fine(mu, di.ds, di.ds_lo, T, b0, b0l);
     const float db0 = ray_db0(xo, T);
     float Iup = 0.0f, Sup = 0.0f;
     if (kind == 0) {

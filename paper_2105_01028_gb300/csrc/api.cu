@@ -48,6 +48,10 @@ struct trinity_ctx {
   float* d_rcorr32 = nullptr;
   float* P32 = nullptr;
   uint16_t* Pbf = nullptr;
+  // FP32 iteration on the tensor cores: one buffer holds the split phase matrix and tables
+  bool split = false;
+  uint8_t* d_split = nullptr;
+  SplitTables sp{};
   DirInfo* d_dirs = nullptr;
   int8_t* d_offs = nullptr;
   int *d_det_vox = nullptr, *d_det_dir = nullptr, *d_det_id = nullptr;
@@ -358,6 +362,8 @@ int lock_inputs(trinity_ctx* ctx) {
   CK(cudaMemset(ctx->d_det, 0, ndet * sizeof(double)));
   CK(cudaMemcpy(ctx->d_dirs, ctx->hdirs.data(), ctx->hdirs.size() * sizeof(DirInfo),
                 cudaMemcpyHostToDevice));
+  // the exact solve's operators hold b1 in FP64, the BF16 iteration is coarser than these weights
+  ctx->g.fine = ctx->g_s.fine = ctx->desc.precision == TRINITY_FP32 && !ctx->exact ? 1 : 0;
   // the photon balance starts from the energy of the state held before step 0
   ctx->energy_init = 0.0;
   if (ctx->has_init) {
@@ -375,6 +381,42 @@ int lock_inputs(trinity_ctx* ctx) {
   }
   CK(cudaMemcpy(ctx->d_balance, &ctx->energy_init, sizeof(double), cudaMemcpyHostToDevice));
   ctx->locked = true;
+  return TRINITY_OK;
+}
+
+// Device bytes of the split phase matrix: the two operand images, diagonals and roots.
+size_t split_bytes(int na) {
+  return 2 * static_cast<size_t>((na + 63) / 64) * na * 128 + 3 * static_cast<size_t>(na) * 4 + 64 * 4;
+}
+
+// Build the split of the phase matrix for the tensor-core iteration and upload it.
+int upload_split(trinity_ctx* ctx, const std::vector<double>& P, int na, double g) {
+  const SplitImage im = scatter_split_image(P, na, g);
+  std::vector<uint8_t> buf(split_bytes(na));
+  uint8_t* p = buf.data();
+  const size_t op = im.ph.size() * 2, dg = im.diag.size() * 4, cw = im.cw.size() * 4;
+  std::memcpy(p, im.ph.data(), op);
+  std::memcpy(p + op, im.pl.data(), op);
+  std::memcpy(p + 2 * op, im.diag.data(), dg);
+  std::memcpy(p + 2 * op + dg, im.cw.data(), cw);
+  CK(cudaMemcpy(ctx->d_split, p, buf.size(), cudaMemcpyHostToDevice));
+  SplitTables t = ctx->sp;
+  t.ph = ctx->d_split;
+  t.pl = ctx->d_split + op;
+  t.diag = reinterpret_cast<const float*>(ctx->d_split + 2 * op);
+  t.cw = reinterpret_cast<const float*>(ctx->d_split + 2 * op + dg);
+  t.unit = im.unit;
+  t.cycle = im.cycle;
+  t.max_inner = im.max_inner;
+  t.lam = im.lam;
+  t.lo = im.lo;
+  if (ctx->graph && std::memcmp(&t, &ctx->sp, sizeof(t)) != 0) {
+    // captured launches carry the scalars by value (another g needs a new capture)
+    CK(cudaStreamSynchronize(ctx->stream));
+    cudaGraphExecDestroy(ctx->graph);
+    ctx->graph = nullptr;
+  }
+  ctx->sp = t;
   return TRINITY_OK;
 }
 
@@ -581,6 +623,9 @@ int enqueue_scatter(trinity_ctx* ctx, const RunState& rs) {
     CK(launch_scatter_bf16(gs, bf_tables(ctx), ctx->Pbf, ctx->Qc, ctx->mut, ctx->eps, ctx->nidx, ctx->Ic,
                            ctx->S, static_cast<float>(ctx->desc.tol), ctx->desc.max_iters, rs,
                            ctx->stream));
+  } else if (ctx->split) {
+    CK(launch_scatter_split(gs, ctx->sp, bf_tables(ctx), ctx->Qc, ctx->mut, ctx->eps, ctx->nidx, ctx->Ic, ctx->S,
+                            static_cast<float>(ctx->desc.tol), ctx->desc.max_iters, rs, ctx->stream));
   } else {
     CK(launch_scatter_fp32(gs, ctx->d_b1ds, ctx->nch, ctx->P32, ctx->d_rcorr32, ctx->Qc, ctx->mut, ctx->eps,
                            ctx->nidx, ctx->Ic, ctx->S, static_cast<float>(ctx->desc.tol), ctx->desc.max_iters,
@@ -806,6 +851,7 @@ int trinity_create_grid(const trinity_grid_desc* desc, void* cuda_stream, trinit
     di.a0 = ax[0];
     di.a1 = ax[1];
     di.ds = static_cast<float>(ctx->lat.ds[d]);
+    di.ds_lo = static_cast<float>(ctx->lat.ds[d] - static_cast<double>(di.ds));
     const double dc = ctx->lat.ds[d] / (kC0 * ctx->dt);
     di.dcoef = static_cast<float>(dc);
     di.dcoef_lo = static_cast<float>(dc - static_cast<double>(di.dcoef));
@@ -876,7 +922,7 @@ int trinity_create_grid(const trinity_grid_desc* desc, void* cuda_stream, trinit
     ctx->Qc = ctx->Q;  // one grid: the scatter reads Q and writes I directly
     ctx->Ic = ctx->I;
   }
-  if (desc->precision == TRINITY_BF16) {
+  if (desc->precision == TRINITY_BF16 || na_s >= 48) {
     ctx->tma_out = make_scatter_out_maps(ctx->g_s, ctx->Ic, ctx->S, ctx->out_maps) == cudaSuccess;
     if (!ctx->tma_out) cudaGetLastError();  // plain stores
   }
@@ -925,6 +971,12 @@ int trinity_create_grid(const trinity_grid_desc* desc, void* cuda_stream, trinit
     }
     ctx->ncls = static_cast<int>(cds.size());
     if (desc->precision == TRINITY_BF16 && ctx->ncls > 16) return bail(TRINITY_E_UNSUPPORTED);
+    // FP32 on the tensor cores: 48 or 192 directions whose spacings fall into 16 classes
+    ctx->split = desc->precision == TRINITY_FP32 && scatter_split_supported(static_cast<int>(na_s), ctx->ncls);
+    if (ctx->split && dalloc(&ctx->d_split, split_bytes(static_cast<int>(na_s))) != cudaSuccess) {
+      cudaGetLastError();
+      return bail(TRINITY_E_OOM);
+    }
     std::vector<float> flat(16 * static_cast<size_t>(nch), 0.0f);
     for (size_t k = 0; k < cds.size() && k < 16; ++k)
       std::copy(cds[k].begin(), cds[k].end(), flat.begin() + k * nch);
@@ -1039,6 +1091,10 @@ int trinity_set_optics(trinity_ctx* ctx, const float* mua, const float* mus, con
   CK(cudaMemcpy(ctx->nidx, r.data(), nv * 4, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(ctx->P32, P32.data(), P32.size() * 4, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(ctx->Pbf, Pb.data(), Pb.size() * 2, cudaMemcpyHostToDevice));
+  if (ctx->split) {
+    const int rc4 = upload_split(ctx, P, na, g);
+    if (rc4 != TRINITY_OK) return rc4;
+  }
   ctx->g_aniso = g;
   ctx->optics_set = true;
   // A uniform mu_t or n lets the sweeps take exp, b0, b1 and the retarded delay once per
@@ -1830,7 +1886,7 @@ void trinity_destroy(trinity_ctx* ctx) {
                   ctx->d_det_vox, ctx->d_det_dir,  ctx->d_det_id,    ctx->d_det_w,   ctx->d_det,
                   ctx->d_step,    ctx->d_smax,     ctx->d_nonconv,   ctx->d_error,   ctx->d_iters_max,
                   ctx->d_iters_sum, ctx->d_energy, ctx->d_escaped,   ctx->d_bins, ctx->d_tile_iters,
-                  ctx->d_tile_ctr, ctx->d_rcorr,   ctx->d_cls,       ctx->d_cls_ds,
+                  ctx->d_tile_ctr, ctx->d_rcorr,   ctx->d_cls,       ctx->d_cls_ds,   ctx->d_split,
                   ctx->d_rcorr32, ctx->d_absorbed, ctx->d_residual,  ctx->d_balance, ctx->d_refl};
   for (void* p : bufs)
     if (p) cudaFree(p);

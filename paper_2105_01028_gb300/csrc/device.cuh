@@ -13,6 +13,7 @@ struct DirInfo {
   int sgn;        // travel sign along dom
   int a0, a1;     // transverse axes (increasing order)
   float ds;       // ray-sample spacing h / |Omega_dom| (mm)
+  float ds_lo;    // its rounding remainder
   float dcoef;    // ds / (c0 dt): retarded delay in steps per unit refractive index (hi part)
   float dcoef_lo; // ds / (c0 dt) - dcoef (lo part: the delay's fraction is exact to FP32)
   float src_amp;  // inflow intensity while the pulse is on (0: not a source direction)
@@ -27,6 +28,7 @@ struct GridParams {
   int periodic;
   int mirror;       // mirror faces: a ghost upwind sample reads its image (see sweep.cu)
   int hist_from;    // first valid time level: 0, or -4 with an initial state
+  int fine;         // sweep weights by ray_weights_fine: the FP32 source iteration
   int warm;         // initial guess of the source iteration: 0 S(n-1), 1 2 S(n-1) - S(n-2)
   int src_voxel;    // flat voxel index of the source spot, -1 if none
   int pulse_steps;
@@ -134,6 +136,31 @@ __device__ __forceinline__ float ray_b1(float x, float T) {
   return (x - 1.0f + T) / x;
 }
 
+// Sweep weights T = e^-x and b0 of a segment x = mu ds, as the FP32 source iteration needs
+// them (lo: remainder of b0):
+//  - the rounding error of x = fl(mu fl(ds)) is carried into T to first order (15 mean free
+//    paths multiply it by 15 in the light that crosses the source cell: 1e-6 of every curve);
+//  - for x >= 1 b0 is the complement (1 - b1) - T of the FP32 b1 that the iteration applies
+//    (T < 1 - b1 there, so both differences are exact with their error terms).  With b0 and
+//    b1 rounded on their own T + b0 + b1 is off by up to 3e-8, which the scattering
+//    multiplies by 1 / (1 - a b1) ~ 14 in every segment, always to the same side in a
+//    uniform medium: up to 1.5e-5 of the field after 100 steps at 16^3 voxels, 48 directions.
+__device__ __forceinline__ void ray_weights_fine(float mu, float ds, float ds_lo, float& T, float& b0, float& lo) {
+  const float x = mu * ds;
+  const float e = fmaf(mu, ds_lo, fmaf(mu, ds, -x));
+  const float T0 = expf(-x);
+  T = fmaf(-e, T0, T0);
+  lo = 0.0f;
+  if (x < 1.0f) {
+    b0 = ray_b0(x, T0);
+  } else {
+    const float b1 = ray_b1(x, T0);
+    const float h = 1.0f - b1;
+    b0 = h - T;
+    lo = ((1.0f - h) - b1) + ((h - b0) - T);
+  }
+}
+
 // Kernel launchers (defined in kernels.cu / scatter_tc.cu).
 cudaError_t launch_sweep(const GridParams& g, const DirInfo* dirs, const int8_t* offs,
                          const float* Iring, const float* Sring, const float* mut,
@@ -165,6 +192,27 @@ cudaError_t launch_energy_density(const GridParams& g, const float* I, const flo
                                   cudaStream_t st);
 cudaError_t launch_interface(int nvox, int na, const int* vox, const int* rowptr, const int* src,
                              const float* w, const uint8_t* keep, float* Q, int nv, cudaStream_t st);
+// FP32 source iteration on the tensor cores (scatter_split.cu): the phase matrix split into
+// FP16 operands, on the host and on the device.
+struct SplitImage {
+  std::vector<uint16_t> ph, pl;  // operand images
+  std::vector<float> diag;       // [3][na] diagonal: high, low; of the inner operator
+  std::vector<float> cw;         // [64] Chebyshev roots of the inner iteration
+  int cycle, max_inner;
+  float unit, lam, lo;
+};
+struct SplitTables {
+  const uint8_t *ph, *pl;
+  const float *diag, *cw;
+  int cycle, max_inner;
+  float unit;     // one unit of Ph
+  float lam, lo;  // spectrum of the rebalanced iteration: rho lam [lo, 1]
+};
+bool scatter_split_supported(int na, int ncls);
+SplitImage scatter_split_image(const std::vector<double>& P, int na, double g_aniso);
+cudaError_t launch_scatter_split(const GridParams& g, const SplitTables& sp, const BfTables& t, const float* Q,
+                                 const float* mut, const float* eps, const float* nidx, float* Iring, float* Sring,
+                                 float tol, int max_iters, RunState rs, cudaStream_t st);
 bool scatter_bf16_supported(int na);
 cudaError_t launch_scatter_bf16(const GridParams& g, const BfTables& t, const uint16_t* Pbf,
                                 const float* Q, const float* mut, const float* eps,

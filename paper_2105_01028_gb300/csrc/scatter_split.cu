@@ -1,0 +1,950 @@
+// FP32 source iteration on the 5th-generation tensor cores (tcgen05): FP32-accurate
+// residuals from split FP16 operands, corrections from single FP16 products.
+//
+// Per voxel the source function is the fixed point of S = a P (Q + b1 o S) (Eq. 12 with
+// Eq. 10).  The plain iteration applies an FP32 product P X some 40 times per voxel and
+// step; on the CUDA cores that is bound by the FP32 pipe.  Here the fixed point is reached
+// by iterative refinement:
+//
+//   outer: r = a P~ (Q + b1 S) - S with an FP32-accurate product (below): the plain
+//          iteration's change, on which its stop test is taken (at a quarter of the
+//          tolerance: the recursion has no noise floor that would hold it above);
+//   inner: the error equation (1 - a P B1) e = r is solved to the relative accuracy of one
+//          FP16 product per iteration, S += e, and r follows by recursion.
+//
+// The result carries the accuracy of the outer residual: what an inner product rounds is a
+// part of 2^-11 of the correction it makes, and an outer residual follows until that part
+// is below the tolerance (two outers per voxel and step on a developed slab).
+//
+// FP32-accurate product.  The diagonal of P~ is applied in FP32 (it holds half a row's
+// weight at g = 0.9); the off-diagonal part, in units of about 2^-t, is split as Ph + Pl with
+// Ph whole numbers of at most 11 bits and Pl multiples of 2^-12, X, scaled per voxel by a
+// power of two, as Xh + Xl likewise (Xh below 2^10).  t is chosen so that every partial sum
+// of Xh Ph stays below 2^24: the FP32 accumulator in TMEM then holds it exactly, whatever
+// the order, and its truncation (the tensor core does not round an accumulation to
+// nearest: three TF32 products summed in one accumulator are 1.7e-6 off, one-sided) has
+// nothing to act on.  Xl Ph + Xh Pl + Xl Pl goes to a second accumulator, 2^-10 of the
+// first in size, where the truncation is below 2^-32 of the result.  Each row of
+// Ph + Pl + diag sums to one (the diagonal is a float pair), so photons are conserved.
+// Measured against FP64 on the 96x96x64 slab: 2.1e-7 in 2-norm of I and S after two steps;
+// the sum of 192 FP32 products on the CUDA cores that it replaces: 2.2e-7.
+//
+// Inner iteration.  Isotropic rebalance as in the other kernels: c = a sum_j b1_j r_j /
+// sum_j (1 - a b1_j) is added to every direction of r; the two-grid iteration that this
+// makes has its spectrum in about [0, rho |g|], and Chebyshev weights over that interval
+// (roots in an order that keeps the partial products bounded) damp it by 0.43 an
+// iteration instead of 0.8:  d = r + c,  S += w d,  r <- r - w d + w a P B1 d.
+// P B1 d is one chain of K = 16 MMAs of FP16 x (b1 d, scaled by a power of two per voxel)
+// and Ph, its diagonal again FP32.
+//
+// Layout: as the BF16 kernel's (scatter_tc.cu): persistent CTAs, tiles of 8 x 4 x 4 voxels
+// (M = 128), operands K-major with the 128-byte swizzle, one voxel row per thread, four
+// column groups of 48 directions (three of 16 at 48 directions).  TMEM: D / first
+// accumulator in [0, N_a), r / second accumulator in [256, 256 + N_a) and, at 192
+// directions, two thirds of Q in the columns left over; S stays in registers.  Shared
+// memory at 192 directions: Ph 72 KB, Xh and Xl 48 KB each; Pl (72 KB) does not fit beside
+// them and is streamed from L2 in six 12 KB blocks through a ring of three.
+#include <cuda.h>
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+#include <cstring>
+#include <vector>
+
+#include "device.cuh"
+#include "tcgen05.cuh"
+
+namespace trinity {
+
+namespace {
+
+constexpr int kSplitCycle = 64;                // longest Chebyshev cycle
+constexpr float kTolShare = 0.25f;             // share of the tolerance the stop test leaves to the change
+constexpr float kInnerError = 4.8828125e-04f;  // 2^-11: error of an inner correction, relative to it
+constexpr float kInnerDrop = 9.765625e-04f;    // 2^-10: an inner solve reduces its residual this far at most
+constexpr int kMaxOuter = 8;
+
+template <int NA>
+struct Sp {
+  static constexpr int KB = (NA + 63) / 64;        // 128-byte K blocks
+  static constexpr int KSTEPS = NA / 16;           // MMAs per operand pair (K = 16 each)
+  static constexpr int kGroups = NA >= 192 ? 4 : 3;
+  static constexpr int kThreads = 128 * kGroups;
+  static constexpr int HALF = NA / kGroups;        // columns per thread
+  static constexpr int CH = 8;                     // columns per TMEM load
+  static constexpr int NCH = HALF / CH;
+  static constexpr int QT = NA >= 192 ? 32 : 0;    // Q columns per thread kept in TMEM
+  static constexpr int QR = HALF - QT;             // ... and in registers
+  static constexpr int NCT = QT / CH;
+  static constexpr int POW2 = NA <= 64 ? 64 : 256;
+  static constexpr int TCOLS = 2 * POW2;
+  static constexpr int ROFF = POW2;                // residual / second accumulator
+  static constexpr bool kRing = NA >= 192;         // Pl streamed through a ring
+  static constexpr int kBlkRows = 96;
+  static constexpr int kBlkBytes = kBlkRows * 128;
+  static constexpr int kNblk = kRing ? KB * (NA / kBlkRows) : 1;
+  static constexpr int kSlots = 3;
+  static constexpr int P_BYTES = KB * NA * 128;
+  static constexpr int A_BYTES = KB * kM * 128;
+  static constexpr int OFF_PH = 0;
+  static constexpr int OFF_XH = (P_BYTES + 1023) / 1024 * 1024;
+  static constexpr int OFF_XL = OFF_XH + A_BYTES;
+  static constexpr int OFF_PL = OFF_XL + A_BYTES;
+  static constexpr int PL_BYTES = kRing ? kSlots * kBlkBytes : (P_BYTES + 1023) / 1024 * 1024;
+  static constexpr int OFF_B1T = OFF_PL + PL_BYTES;                // [kMaxClasses][kM] f32
+  static constexpr int OFF_DI = OFF_B1T + kMaxClasses * kM * 4;    // [3][NA] f32: diagonals
+  static constexpr int OFF_B1C = OFF_DI + 3 * NA * 4;              // [NA] f32 (uniform mu_t)
+  static constexpr int OFF_CLS = OFF_B1C + NA * 4;                 // [NA] u8
+  static constexpr int SMEM = OFF_CLS + ((NA + 15) / 16) * 16 + 1024;
+  static constexpr uint32_t IDESC_ANY = (1u << 4) | (static_cast<uint32_t>(kM >> 4) << 24);  // FP16 x FP16 -> FP32
+  static constexpr uint32_t IDESC = IDESC_ANY | (static_cast<uint32_t>(NA >> 3) << 17);
+  static constexpr uint32_t IDESC_BLK = IDESC_ANY | (static_cast<uint32_t>(kBlkRows >> 3) << 17);
+};
+
+__device__ __forceinline__ float pow2f(int e) { return __uint_as_float(static_cast<uint32_t>(127 + e) << 23); }
+__device__ __forceinline__ int exponent(float x) { return static_cast<int>((__float_as_uint(x) >> 23) & 0xffu) - 127; }
+
+// Power-of-two scale 2^e that brings a row whose largest element is m to [2^top, 2^(top+1)),
+// kept within the range where 2^-(e + 24) is a normal float.
+__device__ __forceinline__ int scale_exponent(float m, int top) {
+  const int e = m > 0.0f ? top - exponent(m) : 0;
+  return e > 100 ? 100 : (e < -100 ? -100 : e);
+}
+
+__device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi) {
+  const __half2 h = __floats2half2_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// u (|u| < 2^11) = h + l: h the nearest whole number, l the rest to multiples of 2^-12.
+// The magic additions round to nearest even at bit 0 and bit -12; every step is exact.
+__device__ __forceinline__ void split_u(float u, float& h, float& l) {
+  h = (u + 12582912.0f) - 12582912.0f;
+  const float d = u - h;
+  l = (d + 3072.0f) - 3072.0f;
+}
+
+__device__ __forceinline__ void bulk_to_smem(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+
+// kUniB1: mu_t is the same in every voxel, so b1 depends on the column's ray spacing only.
+template <int NA, bool kUniB1>
+__global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
+    scatter_split_kernel(GridParams g, SplitTables t, const uint8_t* __restrict__ cls,
+                         const float* __restrict__ cls_ds, int ncls, int nch, const float* __restrict__ Q,
+                         const float* __restrict__ mut, const float* __restrict__ eps,
+                         const float* __restrict__ nidx, float* __restrict__ Iring, float* __restrict__ Sring,
+                         float tol, int max_iters, const __grid_constant__ CUtensorMap tmOutI,
+                         const __grid_constant__ CUtensorMap tmOutS, int tma_out, RunState rs) {
+  using C = Sp<NA>;
+  constexpr int CH = C::CH, NCH = C::NCH, NCT = C::NCT;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sPh = smem + C::OFF_PH;
+  uint8_t* sXh = smem + C::OFF_XH;
+  uint8_t* sXl = smem + C::OFF_XL;
+  uint8_t* sPl = smem + C::OFF_PL;
+  float* b1t = reinterpret_cast<float*>(smem + C::OFF_B1T);
+  float* sDi = reinterpret_cast<float*>(smem + C::OFF_DI);  // diagonal of P~ (hi), (lo); of the inner operator
+  float* sB1c = reinterpret_cast<float*>(smem + C::OFF_B1C);
+  uint8_t* sCls = smem + C::OFF_CLS;
+
+  __shared__ uint64_t mbar;
+  __shared__ uint64_t pl_full[C::kSlots], pl_empty[C::kSlots];
+  __shared__ uint32_t tmem_base_s;
+  __shared__ int tile_s, next_s;
+  __shared__ int abort_s;
+  __shared__ float e_s[kM], rho_s[kM], den_s[kM];
+  __shared__ int ccnt_s[kMaxClasses];
+  __shared__ float clsb1_s[kMaxClasses];
+  __shared__ float sumb1_s;
+  __shared__ float cw_s[kSplitCycle];
+  constexpr int kGroups = C::kGroups;
+  __shared__ float red_d[kGroups][kM], red_s[kGroups][kM], red_c[kGroups][kM];
+  __shared__ double esum_s[C::kThreads / 32];
+  __shared__ double asum_sh;
+  __shared__ float smax_s[C::kThreads / 32];
+
+  const int tid = threadIdx.x;
+  const int warp = tid >> 5, lane = tid & 31;
+  const int row = ((warp & 3) << 5) + lane;
+  const int grp = warp >> 2;  // column group
+  const int cb = grp * C::HALF;
+  const int n = *rs.step;
+  const size_t plane = static_cast<size_t>(g.nv);
+  const float s_glob = __uint_as_float(rs.smax[(n - 1) & 1]);
+  const bool has_prev = (n - 1) >= g.hist_from;
+  const bool has_prev2 = g.warm != 0 && (n - 2) >= g.hist_from;  // linear extrapolation in time
+  const size_t prev_base = static_cast<size_t>(ring_slot(n - 1)) * g.na * plane;
+  const size_t prev2_base = static_cast<size_t>(ring_slot(n - 2)) * g.na * plane;
+  const size_t cur_base = static_cast<size_t>(ring_slot(n)) * g.na * plane;
+  const int bxn = (g.nx + 7) >> 3, byn = (g.ny + 3) >> 2;
+  const int ntiles = brick_tiles(g.nx, g.ny, g.nz);
+
+  // ---- one-time set-up: TMEM, barriers, operand images, diagonals, class tables
+  if (warp == 0) tmem_alloc(&tmem_base_s, C::TCOLS);
+  uint32_t pl_issued = 0, pl_used = 0;  // thread 0: Pl blocks loaded and consumed so far
+  const auto pl_load = [&]() {
+    const uint32_t s = pl_issued % C::kSlots;
+    bulk_to_smem(smem_u32(sPl) + s * C::kBlkBytes,
+                 t.pl + static_cast<size_t>(pl_issued % C::kNblk) * C::kBlkBytes, C::kBlkBytes, &pl_full[s]);
+    ++pl_issued;
+  };
+  if (tid == 0) {
+    mbar_init(&mbar);
+    for (int s = 0; s < C::kSlots; ++s) {
+      mbar_init(&pl_full[s]);
+      mbar_init(&pl_empty[s]);
+    }
+    abort_s = 0;
+    asum_sh = 0.0;
+    if constexpr (C::kRing) {
+      for (int s = 0; s < C::kSlots; ++s) pl_load();
+    }
+  }
+  for (int u = tid; u < C::P_BYTES / 16; u += blockDim.x)
+    reinterpret_cast<uint4*>(sPh)[u] = __ldg(reinterpret_cast<const uint4*>(t.ph) + u);
+  if constexpr (!C::kRing) {
+    for (int u = tid; u < C::P_BYTES / 16; u += blockDim.x)
+      reinterpret_cast<uint4*>(sPl)[u] = __ldg(reinterpret_cast<const uint4*>(t.pl) + u);
+  }
+  if (tid < kMaxClasses) ccnt_s[tid] = 0;
+  if (tid < kSplitCycle) cw_s[tid] = t.cw[tid];
+  __syncthreads();
+  for (int i = tid; i < NA; i += blockDim.x) {
+    atomicAdd(&ccnt_s[cls[i]], 1);
+    sDi[i] = t.diag[i];
+    sDi[NA + i] = t.diag[NA + i];
+    sDi[2 * NA + i] = t.diag[2 * NA + i];
+    sCls[i] = cls[i];
+    if (kUniB1) {  // the same operations as the per-row table below, on the same mu_t
+      const int k = cls[i];
+      float bs = 0.0f;
+      for (int j = 0; j < nch; ++j) {
+        const float x = g.mut_u * cls_ds[k * nch + j];
+        bs += ray_b1(x, expf(-x));
+      }
+      sB1c[i] = bs * (1.0f / static_cast<float>(nch));
+    }
+  }
+  fence_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (kUniB1) {
+    // the denominators' sum_j b1_j, in the order the general form sums it (per class; all
+    // directions of a class hold the same b1, so concurrent writes store the same value)
+    for (int i = tid; i < NA; i += blockDim.x) clsb1_s[sCls[i]] = sB1c[i];
+    __syncthreads();
+    if (tid == 0) {
+      float sb = 0.0f;
+      for (int k2 = 0; k2 < ncls; ++k2) sb = fmaf(static_cast<float>(ccnt_s[k2]), clsb1_s[k2], sb);
+      sumb1_s = sb;
+    }
+    __syncthreads();
+  }
+  const uint32_t tmem = tmem_base_s;
+  const uint32_t t_row = tmem + (static_cast<uint32_t>((warp & 3) << 5) << 16);
+  // this thread's Q columns in TMEM (column group h: N_a + 32 h for h < 2, ROFF + N_a + 32 (h - 2))
+  const uint32_t t_q = t_row + static_cast<uint32_t>(grp < 2 ? NA + C::QT * grp : C::ROFF + NA + C::QT * (grp - 2));
+  const uint32_t aXh = smem_u32(sXh), aXl = smem_u32(sXl), aPh = smem_u32(sPh), aPl = smem_u32(sPl);
+  uint32_t phase = 0;
+  bool aborted = false;
+  double esum = 0.0;
+  float smax_loc = 0.0f;
+  float S[C::HALF];                       // S of the thread's row and columns
+  float qr[C::QR > 0 ? C::QR : 1];        // Q of the thread's last QR columns
+  const float tscale = t.unit;            // one unit of Ph
+  bool first_tile = true;
+
+  // b1 of 8 columns from c0 on (volatile or asm loads: hoisted out of the iterations these
+  // tables would cost more registers than there are)
+  const auto load_b1 = [&](int c0, float (&bv)[8]) {
+    if (kUniB1) {
+      lds_vec<8>(sB1c + c0, bv);
+    } else {
+      const volatile float* vb = b1t;
+      uint32_t cv[2];
+      lds_bytes<8>(sCls + c0, cv);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) bv[j] = vb[((cv[j >> 2] >> (8 * (j & 3))) & 0xffu) * kM + row];
+    }
+  };
+  // Q of chunk ch (issued before tmem_wait_ld where it lives in TMEM)
+  const auto load_q = [&](int ch, float (&qv)[CH]) {
+    if (ch < NCT) tmem_ld<CH>(t_q + ch * CH, qv);
+  };
+  const auto reg_q = [&](int ch, float (&qv)[CH]) {
+    if (ch >= NCT) {
+#pragma unroll
+      for (int j = 0; j < CH; ++j) qv[j] = qr[(ch - NCT) * CH + j];
+    }
+  };
+  // max over the row's column groups of red_d, red_s, sum of red_c
+  const auto row_max = [&](const float (&red)[kGroups][kM]) {
+    float m = red[0][row];
+#pragma unroll
+    for (int gi = 1; gi < kGroups; ++gi) m = fmaxf(m, red[gi][row]);
+    return m;
+  };
+  const auto row_sum = [&](const float (&red)[kGroups][kM]) {
+    float s = red[0][row];
+#pragma unroll
+    for (int gi = 1; gi < kGroups; ++gi) s += red[gi][row];
+    return s;
+  };
+  // wait for the MMAs committed to mbar; false for the whole warp if the wait ran out
+  const auto wait_mma = [&]() {
+    const bool ok = mbar_wait_bounded(&mbar, phase);
+    phase ^= 1u;
+    if (!ok) abort_s = 1;
+    const bool to = __any_sync(0xffffffffu, !ok);
+    tc_fence_after();
+    return !to;
+  };
+  // thread 0: the two accumulators of an FP32-accurate product
+  const auto issue_product = [&]() {
+    tc_fence_after();
+#pragma unroll
+    for (int s = 0; s < C::KSTEPS; ++s) {
+      const uint32_t ko = static_cast<uint32_t>((s & 3) * 32), kb = static_cast<uint32_t>(s >> 2);
+      mma_f16(tmem, sw128_desc(aXh + kb * kM * 128 + ko), sw128_desc(aPh + kb * NA * 128 + ko), C::IDESC, s > 0);
+    }
+#pragma unroll
+    for (int s = 0; s < C::KSTEPS; ++s) {
+      const uint32_t ko = static_cast<uint32_t>((s & 3) * 32), kb = static_cast<uint32_t>(s >> 2);
+      mma_f16(tmem + C::ROFF, sw128_desc(aXl + kb * kM * 128 + ko), sw128_desc(aPh + kb * NA * 128 + ko), C::IDESC,
+              s > 0);
+    }
+    if constexpr (!C::kRing) {
+#pragma unroll
+      for (int s = 0; s < C::KSTEPS; ++s) {
+        const uint32_t ko = static_cast<uint32_t>(s * 32);
+        mma_f16(tmem + C::ROFF, sw128_desc(aXh + ko), sw128_desc(aPl + ko), C::IDESC, 1u);
+        mma_f16(tmem + C::ROFF, sw128_desc(aXl + ko), sw128_desc(aPl + ko), C::IDESC, 1u);
+      }
+      mma_commit(&mbar);
+    } else {
+      // blocks b: K block b / 2, output directions 96 (b & 1) .. + 95; the first three are
+      // resident or in flight
+      static_assert(C::kNblk == 2 * C::kSlots, "the second half of the blocks refills the ring once");
+      bool ok = true;
+#pragma unroll 1
+      for (int b = 0; b < C::kNblk; ++b) {
+        if (b == C::kSlots) {  // as the first blocks' MMAs complete, the others take their slots
+          for (uint32_t q = pl_used; ok && q < pl_used + C::kSlots; ++q) {
+            ok = mbar_wait_bounded(&pl_empty[q % C::kSlots], ((q / C::kSlots) & 1u) ^ 1u);
+            if (ok) pl_load();
+          }
+        }
+        const uint32_t s = pl_used % C::kSlots;
+        if (ok) ok = mbar_wait_bounded(&pl_full[s], (pl_used / C::kSlots) & 1u);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t kb = static_cast<uint32_t>(b >> 1), d = tmem + C::ROFF + (b & 1) * C::kBlkRows;
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+          const uint64_t pd = sw128_desc(aPl + s * C::kBlkBytes + ks * 32);
+          mma_f16(d, sw128_desc(aXh + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, 1u);
+          mma_f16(d, sw128_desc(aXl + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, 1u);
+        }
+        mma_commit(&pl_empty[s]);
+        ++pl_used;
+      }
+      mma_commit(&mbar);
+      if (!ok) abort_s = 1;
+    }
+  };
+
+  while (true) {
+    // the previous tile's TMA stores must have read the staging area (the X operands)
+    // before X is written again
+    if (tid == 0) {
+      if (tma_out) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      tile_s = first_tile ? atomicAdd(rs.tile_ctr + (n & 1), 1) : next_s;
+      next_s = atomicAdd(rs.tile_ctr + (n & 1), 1);
+    }
+    first_tile = false;
+    __syncthreads();
+    const int tile = tile_s;
+    if (tile >= ntiles) break;
+    const int vb = brick_voxel(g, bxn, byn, tile, row);
+    const bool vin = vb >= 0;
+    const int v = vin ? vb : 0;
+
+    // per-row constants and the b1 table over ds classes
+    if (tid < kM) {
+      const int vv = brick_voxel(g, bxn, byn, tile, tid);
+      float ev = 1.0f, rho = 0.0f;
+      if (vv >= 0) {
+        ev = eps[vv];
+        const float xm = mut[vv] * g.ds_max;
+        rho = (1.0f - ev) * ray_b1(xm, expf(-xm));
+      }
+      e_s[tid] = ev;
+      rho_s[tid] = rho;
+    }
+    for (int u = tid; u < (kUniB1 ? 0 : ncls * kM); u += blockDim.x) {
+      const int k = u / kM, r = u % kM;
+      const int vv = brick_voxel(g, bxn, byn, tile, r);
+      float bs = 0.0f;
+      if (vv >= 0) {
+        const float mu = mut[vv];
+        for (int j = 0; j < nch; ++j) {
+          const float x = mu * cls_ds[k * nch + j];
+          bs += ray_b1(x, expf(-x));
+        }
+      }
+      b1t[k * kM + r] = bs * (1.0f / static_cast<float>(nch));
+    }
+    __syncthreads();
+    // rebalance denominator sum_j (1 - a b1_j) of each row
+    if (tid < kM) {
+      float sb;
+      if (kUniB1) {
+        sb = sumb1_s;
+      } else {
+        sb = 0.0f;
+        for (int k2 = 0; k2 < ncls; ++k2) sb = fmaf(static_cast<float>(ccnt_s[k2]), b1t[k2 * kM + tid], sb);
+      }
+      den_s[tid] = static_cast<float>(NA) - (1.0f - e_s[tid]) * sb;
+    }
+
+    // ---- warm start S(n-1), or 2 S(n-1) - S(n-2), into registers; Q (read once) into TMEM
+    // or registers; max |X| of the row.  Loads go two chunks (48 per thread) at a time.
+    float xmax = 0.0f;
+    {
+      static_assert(NCH % 2 == 0 && NCT % 2 == 0, "chunks go in pairs");
+#pragma unroll
+      for (int c2 = 0; c2 < NCH; c2 += 2) {
+        float s1[2][CH], s2[2][CH], qc[2][CH];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int j = 0; j < CH; ++j) {
+            const size_t col = static_cast<size_t>(cb + (c2 + u) * CH + j) * plane + v;
+            s1[u][j] = (vin && has_prev) ? __ldg(Sring + prev_base + col) : 0.0f;
+            s2[u][j] = (vin && has_prev2) ? __ldg(Sring + prev2_base + col) : 0.0f;
+            qc[u][j] = vin ? __ldg(Q + col) : 0.0f;
+          }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int ch = c2 + u;
+          float bv[8];
+          load_b1(cb + ch * CH, bv);
+#pragma unroll
+          for (int j = 0; j < CH; ++j) {
+            const float s0 = (vin && has_prev2) ? fmaf(2.0f, s1[u][j], -s2[u][j]) : s1[u][j];
+            S[ch * CH + j] = s0;
+            xmax = fmaxf(xmax, fabsf(fmaf(bv[j], s0, qc[u][j])));
+            if (ch >= NCT) qr[(ch - NCT) * CH + j] = qc[u][j];
+          }
+          if (ch < NCT) tmem_st<CH>(t_q + ch * CH, qc[u]);
+        }
+      }
+    }
+    red_d[grp][row] = xmax;
+    tmem_wait_st();
+    __syncthreads();
+
+    const float ev = e_s[row], al = 1.0f - ev, rho = rho_s[row];
+    const float amp = rho / (1.0f - rho);           // error bound per unit change
+    const float span = rho * t.lam;                 // Chebyshev interval [t.lo span, span]
+    const float eta = kInnerError * fmaxf(1.0f, 0.08f * amp);
+    bool live = vin;       // the row takes part in this outer iteration
+    bool hitmax = false, bad = false;
+    float thr = 0.0f, prevr = 3.0e38f;
+    int iters = 0;
+    int outer = 0;
+    while (true) {
+      // ---- X = Q + b1 S, split
+      const int ex = scale_exponent(row_max(red_d), 9);
+      const float sx = pow2f(ex);
+#pragma unroll
+      for (int ch = 0; ch < NCH; ++ch) {
+        const int c0 = cb + ch * CH;
+        float qv[CH], bv[8];
+        load_q(ch, qv);
+        load_b1(c0, bv);
+        if (ch < NCT) tmem_wait_ld();
+        reg_q(ch, qv);
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int j = 0; j < CH; j += 2) {
+          float h0, l0, h1, l1;
+          split_u(fmaf(bv[j], S[ch * CH + j], qv[j]) * sx, h0, l0);
+          split_u(fmaf(bv[j + 1], S[ch * CH + j + 1], qv[j + 1]) * sx, h1, l1);
+          hi[j / 2] = pack_f16x2(h0, h1);
+          lo[j / 2] = pack_f16x2(l0, l1);
+        }
+        const uint32_t off = sw128_chunk_off(kM, row, c0);
+        *reinterpret_cast<uint4*>(sXh + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        *reinterpret_cast<uint4*>(sXl + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+      }
+      fence_async_smem();
+      tc_fence_before();
+      __syncthreads();
+      if (tid == 0) issue_product();
+      bool mma_ok = wait_mma();
+      if (tid == 0 && C::kRing && mma_ok) {
+        // the next product's first blocks (its slots' MMAs have completed)
+        while (pl_issued < pl_used + C::kSlots) pl_load();
+      }
+      // ---- residual r = a P~ X - S -> TMEM
+      float rm = 0.0f, sm = 0.0f, cs = 0.0f;
+      const float ky = tscale * pow2f(-ex);
+      if (mma_ok) {
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) {
+          const int c0 = cb + ch * CH;
+          float a0[CH], a1[CH], qv[CH], bv[8], dv[8], dl[8];
+          tmem_ld<CH>(t_row + c0, a0);
+          tmem_ld<CH>(t_row + C::ROFF + c0, a1);
+          load_q(ch, qv);
+          load_b1(c0, bv);
+          lds_vec<8>(sDi + c0, dv);
+          lds_vec<8>(sDi + NA + c0, dl);
+          tmem_wait_ld();
+          reg_q(ch, qv);
+#pragma unroll
+          for (int j = 0; j < CH; ++j) {
+            const float s = S[ch * CH + j];
+            const float x = fmaf(bv[j], s, qv[j]);
+            float y = fmaf(dl[j], x, (a0[j] + a1[j]) * ky);
+            y = fmaf(dv[j], x, y);
+            const float sh = fmaf(-ev, y, y);
+            const float r = sh - s;
+            a0[j] = r;
+            rm = fmaxf(rm, fabsf(r));
+            sm = fmaxf(sm, fabsf(sh));
+            cs = fmaf(bv[j], r, cs);
+          }
+          tmem_st<CH>(t_row + C::ROFF + c0, a0);
+        }
+        tmem_wait_st();
+      }
+      red_d[grp][row] = rm;
+      red_s[grp][row] = sm;
+      red_c[grp][row] = cs;
+      __syncthreads();
+      if (abort_s) {
+        aborted = true;
+        break;
+      }
+      bool inner = false, fin = !live;  // fin: S has taken its last r of this outer
+      bool stalled = false;
+      float target = 0.0f, es = 0.0f, crow = 0.0f;
+      rm = row_max(red_d);
+      if (live) {
+        ++iters;
+        thr = kTolShare * tol * fmaxf(row_max(red_s), 1e-6f * s_glob);
+        stalled = rm > 0.25f * prevr;
+        prevr = rm;
+        target = fmaxf(thr, amp * rm * kInnerDrop);
+        const bool conv = amp * rm <= thr;
+        inner = !conv && iters < max_iters && rm <= 3.0e38f;
+        hitmax = !conv && !inner;
+        if (inner) crow = al * row_sum(red_c) / den_s[row];
+      }
+      // ---- inner iterations on the error equation
+      int k = 0;
+      while (true) {
+        const float half = 0.5f * (span - t.lo * span), mid = 0.5f * (span + t.lo * span);
+        const float om = 1.0f / (1.0f - fmaf(half, cw_s[k % t.cycle], mid));
+        const float w = inner ? om : (fin ? 0.0f : 1.0f);
+        const int er = scale_exponent(rm + fabsf(crow), 13);
+        const float sc = inner ? pow2f(er) : 0.0f;
+        if (__any_sync(0xffffffffu, w != 0.0f)) {
+#pragma unroll
+          for (int ch = 0; ch < NCH; ++ch) {
+            const int c0 = cb + ch * CH;
+            float rv[CH], bv[8];
+            tmem_ld<CH>(t_row + C::ROFF + c0, rv);
+            load_b1(c0, bv);
+            tmem_wait_ld();
+            uint32_t hi[4];
+#pragma unroll
+            for (int j = 0; j < CH; j += 2) {
+              const float d0 = rv[j] + crow, d1 = rv[j + 1] + crow;
+              S[ch * CH + j] = fmaf(w, d0, S[ch * CH + j]);
+              S[ch * CH + j + 1] = fmaf(w, d1, S[ch * CH + j + 1]);
+              hi[j / 2] = pack_f16x2(bv[j] * d0 * sc, bv[j + 1] * d1 * sc);
+            }
+            *reinterpret_cast<uint4*>(sXh + sw128_chunk_off(kM, row, c0)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+          }
+        }
+        if (inner) es += om * (rm + fabsf(crow));
+        if (!inner) fin = true;
+        fence_async_smem();
+        tc_fence_before();
+        if (!__syncthreads_or(inner ? 1 : 0)) break;
+        if (tid == 0) {
+          tc_fence_after();
+#pragma unroll
+          for (int s = 0; s < C::KSTEPS; ++s) {
+            const uint32_t ko = static_cast<uint32_t>((s & 3) * 32), kb = static_cast<uint32_t>(s >> 2);
+            mma_f16(tmem, sw128_desc(aXh + kb * kM * 128 + ko), sw128_desc(aPh + kb * NA * 128 + ko), C::IDESC, s > 0);
+          }
+          mma_commit(&mbar);
+        }
+        mma_ok = wait_mma();
+        float rmx = 0.0f, csx = 0.0f;
+        if (mma_ok && __any_sync(0xffffffffu, inner)) {
+          const float kd = tscale * pow2f(-er), wa = w * al;
+#pragma unroll
+          for (int ch = 0; ch < NCH; ++ch) {
+            const int c0 = cb + ch * CH;
+            float rv[CH], dd[CH], bv[8], di[8];
+            tmem_ld<CH>(t_row + c0, dd);
+            tmem_ld<CH>(t_row + C::ROFF + c0, rv);
+            load_b1(c0, bv);
+            lds_vec<8>(sDi + 2 * NA + c0, di);
+            tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < CH; ++j) {
+              const float d = rv[j] + crow;
+              const float y = fmaf(di[j], bv[j] * d, dd[j] * kd);  // P B1 d
+              const float rn = fmaf(wa, y, fmaf(-w, d, rv[j]));
+              rv[j] = inner ? rn : rv[j];
+              rmx = fmaxf(rmx, fabsf(rv[j]));
+              csx = fmaf(bv[j], rv[j], csx);
+            }
+            tmem_st<CH>(t_row + C::ROFF + c0, rv);
+          }
+          tmem_wait_st();
+        }
+        red_d[grp][row] = rmx;
+        red_c[grp][row] = csx;
+        __syncthreads();
+        if (abort_s) {
+          aborted = true;
+          break;
+        }
+        ++k;
+        if (inner) {
+          rm = row_max(red_d);
+          ++iters;
+          const bool conv = amp * rm <= target;
+          if (conv || iters >= max_iters || k >= t.max_inner || !(rm <= 3.0e38f)) {
+            inner = false;
+            if (!conv && iters >= max_iters) hitmax = true;
+            crow = 0.0f;
+          } else {
+            crow = al * row_sum(red_c) / den_s[row];
+          }
+        }
+      }
+      if (aborted) break;
+      ++outer;
+      // another accurate residual where the inner products' error may exceed the tolerance
+      bool more = live && !hitmax && !stalled && iters < max_iters && outer < kMaxOuter &&
+                  (amp * rm > thr || eta * es > thr);
+      if (live && amp * rm > thr && iters >= max_iters) bad = true;
+      live = more;
+      // (the barrier also separates the reads of red_d above from the writes below)
+      if (!__syncthreads_or(more ? 1 : 0)) break;
+      xmax = 0.0f;
+#pragma unroll
+      for (int ch = 0; ch < NCH; ++ch) {
+        float qv[CH], bv[8];
+        load_q(ch, qv);
+        load_b1(cb + ch * CH, bv);
+        if (ch < NCT) tmem_wait_ld();
+        reg_q(ch, qv);
+#pragma unroll
+        for (int j = 0; j < CH; ++j) xmax = fmaxf(xmax, fabsf(fmaf(bv[j], S[ch * CH + j], qv[j])));
+      }
+      red_d[grp][row] = xmax;
+      __syncthreads();
+    }
+    if (aborted) break;
+    if (bad && grp == 0) atomicAdd(rs.nonconv, 1);
+
+    // ---- write-out: I = Q + b1 S and S of every voxel
+    const float nv_v = vin ? nidx[v] : 0.0f;
+    const float mu_v = vin ? mut[v] : 0.0f;
+    float esum_row = 0.0f;
+    if (C::KB * 64 == NA && tma_out) {
+      // staged: I and then S of the tile go to the X operand area as 8-direction boxes of
+      // the brick ([direction][row], conflict-free) and one thread stores them with TMA
+      float* stg = reinterpret_cast<float*>(sXh);
+      const int bx = tile % bxn, t2 = tile / bxn;
+      const int ox = bx << 3, oy = (t2 % byn) << 2, oz = (t2 / byn) << 2;
+      const int pbase = ring_slot(n) * NA;
+#pragma unroll
+      for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) {
+          const int c0 = cb + ch * CH;
+          float qv[CH], bv[8];
+          if (pass == 0) {
+            load_q(ch, qv);
+            load_b1(c0, bv);
+            if (ch < NCT) tmem_wait_ld();
+            reg_q(ch, qv);
+          }
+#pragma unroll
+          for (int j = 0; j < CH; ++j) {
+            const int col = c0 + j;
+            float val = S[ch * CH + j];
+            if (pass == 0) {
+              val = fmaf(bv[j], S[ch * CH + j], qv[j]);
+              if (vin) {
+                esum_row += val;
+                smax_loc = fmaxf(smax_loc, fabsf(S[ch * CH + j]));
+              }
+            }
+            stg[(col >> 3) * 1024 + (col & 7) * 128 + row] = val;
+          }
+        }
+        fence_async_smem();
+        __syncthreads();
+        if (tid == 0) {
+          const uint64_t map = reinterpret_cast<uint64_t>(pass == 0 ? &tmOutI : &tmOutS);
+#pragma unroll 1
+          for (int bb = 0; bb < NA / 8; ++bb)
+            asm volatile(
+                "cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(map),
+                "r"(ox), "r"(oy), "r"(oz), "r"(pbase + bb * 8), "r"(smem_u32(stg + bb * 1024))
+                : "memory");
+          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          if (pass == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        }
+        if (pass == 0) __syncthreads();
+      }
+    } else {
+      float* pI = Iring + cur_base + static_cast<size_t>(cb) * plane + v;
+      float* pS = Sring + cur_base + static_cast<size_t>(cb) * plane + v;
+#pragma unroll
+      for (int ch = 0; ch < NCH; ++ch) {
+        float qv[CH], bv[8];
+        load_q(ch, qv);
+        load_b1(cb + ch * CH, bv);
+        if (ch < NCT) tmem_wait_ld();
+        reg_q(ch, qv);
+        if (vin) {
+#pragma unroll
+          for (int j = 0; j < CH; ++j) {
+            const float s = S[ch * CH + j];
+            const float Iv = fmaf(bv[j], s, qv[j]);
+            pI[static_cast<size_t>(ch * CH + j) * plane] = Iv;
+            pS[static_cast<size_t>(ch * CH + j) * plane] = s;
+            esum_row += Iv;
+            smax_loc = fmaxf(smax_loc, fabsf(s));
+          }
+        }
+      }
+    }
+    if (vin) esum += static_cast<double>(esum_row) * static_cast<double>(nv_v);
+    float ab = vin ? esum_row * (ev * mu_v) : 0.0f;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) ab += __shfl_xor_sync(0xffffffffu, ab, o);
+    if (lane == 0) atomicAdd(&asum_sh, static_cast<double>(ab));
+    // iteration statistics of this tile (group-0 threads hold one row each)
+    if (warp < 4) {
+      int im = vin ? iters : 0;
+      unsigned long long is = static_cast<unsigned long long>(im);
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) {
+        im = max(im, __shfl_xor_sync(0xffffffffu, im, o));
+        is += __shfl_xor_sync(0xffffffffu, is, o);
+      }
+      if (lane == 0) {
+        atomicMax(rs.iters_max + n, im);
+        atomicAdd(rs.iters_sum + n, is);
+      }
+    }
+    __syncthreads();
+  }
+
+  if (aborted && tid == 0) atomicExch(rs.error, 7);
+  if (tid == 0) {
+    if (tma_out) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    // the Pl blocks loaded ahead have landed before the shared memory is given back
+    if constexpr (C::kRing) {
+      for (uint32_t q = pl_used; q < pl_issued; ++q) mbar_wait_bounded(&pl_full[q % C::kSlots], (q / C::kSlots) & 1u);
+    }
+  }
+  // energy and max |S| of this CTA's voxels
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    esum += __shfl_xor_sync(0xffffffffu, esum, o);
+    smax_loc = fmaxf(smax_loc, __shfl_xor_sync(0xffffffffu, smax_loc, o));
+  }
+  if (lane == 0) {
+    esum_s[warp] = esum;
+    smax_s[warp] = smax_loc;
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0) {
+    double e = 0.0;
+    float sm = 0.0f;
+    for (int w = 0; w < C::kThreads / 32; ++w) {
+      e += esum_s[w];
+      sm = fmaxf(sm, smax_s[w]);
+    }
+    atomicAdd(rs.energy + n, e * static_cast<double>(g.e_scale));
+    atomicAdd(rs.absorbed + n, asum_sh * g.a_scale);
+    atomicMax(rs.smax + (n & 1), __float_as_uint(sm));
+  }
+  if (warp == 0) {
+    tc_fence_after();
+    tmem_dealloc(tmem, C::TCOLS);
+  }
+}
+
+int g_split_sms = 0;
+
+template <int NA>
+cudaError_t configure_split() {
+  cudaError_t e = cudaFuncSetAttribute(scatter_split_kernel<NA, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       Sp<NA>::SMEM);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(scatter_split_kernel<NA, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              Sp<NA>::SMEM);
+}
+
+uint16_t half_bits(double x) {  // x is an FP16 number
+  const __half h = __float2half(static_cast<float>(x));
+  uint16_t u;
+  std::memcpy(&u, &h, 2);
+  return u;
+}
+
+}  // namespace
+
+bool scatter_split_supported(int na, int ncls) {
+  if ((na != 48 && na != 192) || ncls > kMaxClasses) return false;
+  if (g_split_sms == 0) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        configure_split<48>() != cudaSuccess || configure_split<192>() != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    g_split_sms = sms;
+  }
+  return true;
+}
+
+// Off-diagonal part of the FP64 phase matrix P split as (Ph + Pl) unit, in the kernel's operand layout: Ph
+// [K block][na rows][128 B], Pl likewise at 48 directions and as six blocks (K block, half
+// of the rows) of 96 rows at 192; diag: the FP32 pair that makes each row of Ph + Pl + diag
+// sum to one, and the diagonal that does so with Ph alone.
+SplitImage scatter_split_image(const std::vector<double>& P, int na, double g_aniso) {
+  SplitImage im;
+  const int kb = (na + 63) / 64;
+  double pmax = 0.0, rmax = 0.0;
+  for (int i = 0; i < na; ++i) {
+    double s = 0.0;
+    for (int j = 0; j < na; ++j)
+      if (j != i) {
+        const double p = std::fabs(P[static_cast<size_t>(i) * na + j]);
+        pmax = std::max(pmax, p);
+        s += p;
+      }
+    rmax = std::max(rmax, s);
+  }
+  // Ph of at most 11 bits; |sum Xh Ph| <= 2^10 sum |Ph| <= 2^10 (2^t rmax + na / 2) < 2^24, with room for
+  // the unit's rounding
+  int t = 0;
+  while (t < 20 && std::ldexp(pmax, t + 1) <= 2046.0 && std::ldexp(rmax, t + 1) + na / 2 <= 16128.0) ++t;
+  // one unit of Ph: 2^-t made so that the largest entry is a whole number of units (an
+  // isotropic P is then split exactly; its equal entries would else all err to one side)
+  const double whole = std::floor(std::ldexp(pmax, t));
+  im.unit = static_cast<float>(whole >= 1.0 ? pmax / whole : std::ldexp(1.0, -t));
+  const double unit = im.unit;
+  im.ph.assign(static_cast<size_t>(kb) * na * 64, 0);
+  im.pl.assign(static_cast<size_t>(kb) * na * 64, 0);
+  im.diag.assign(static_cast<size_t>(3) * na, 0.0f);
+  const int blk = 96;
+  for (int i = 0; i < na; ++i) {
+    double sh = 0.0, sl = 0.0;
+    for (int j = 0; j < na; ++j) {
+      if (j == i) continue;
+      const double u = P[static_cast<size_t>(i) * na + j] / unit;
+      const double h = std::nearbyint(u);
+      const double l = std::nearbyint((u - h) * 4096.0) / 4096.0;
+      sh += h;
+      sl += l;
+      const int k = j >> 6, ch = (j & 63) >> 3;
+      const size_t in_row = static_cast<size_t>(((ch ^ (i & 7)) << 3) + (j & 7));
+      im.ph[(static_cast<size_t>(k) * na + i) * 64 + in_row] = half_bits(h);
+      // 96 is a multiple of 8, so a block's rows keep the swizzle phase i & 7
+      const size_t prow = na >= 192 ? static_cast<size_t>(k * (na / blk) + i / blk) * blk + i % blk
+                                    : static_cast<size_t>(k) * na + i;
+      im.pl[prow * 64 + in_row] = half_bits(l);
+    }
+    const double d = 1.0 - (sh + sl) * unit;
+    im.diag[i] = static_cast<float>(d);
+    im.diag[na + i] = static_cast<float>(d - static_cast<double>(im.diag[i]));
+    im.diag[2 * na + i] = static_cast<float>(1.0 - sh * unit);
+  }
+  // Chebyshev interval of the rebalanced iteration, in units of rho: the eigenvalues of P
+  // but the constant vector's lie in [0, |g| + 0.013] for g >= 0 (checked for g from 0 to
+  // 0.99 at 12, 48 and 192 directions) and in +- that for g < 0
+  const double a = std::fabs(g_aniso);
+  im.lam = static_cast<float>(std::min(a + 0.015, 0.5 * (a + 1.0)));
+  im.lo = g_aniso >= 0.0 ? 0.0f : -1.0f;
+  // cycle length: long enough to damp by ~50 (sigma^m, sigma of kappa = 1 / (1 - lam))
+  const double kap = std::sqrt((1.0 - im.lo * im.lam) / (1.0 - im.lam));
+  int m = 8;
+  while (m < kSplitCycle && std::pow((kap - 1.0) / (kap + 1.0), m) > 0.02) m *= 2;
+  im.cycle = m;
+  im.max_inner = 8 * m;
+  // roots in the order that keeps every partial product bounded (Lebedev and Finogenov 1971)
+  std::vector<int> th(1, 1);
+  while (static_cast<int>(th.size()) < m) {
+    const int n2 = 2 * static_cast<int>(th.size());
+    std::vector<int> nx;
+    for (int a2 : th) {
+      nx.push_back(a2);
+      nx.push_back(2 * n2 - a2);
+    }
+    th = nx;
+  }
+  im.cw.assign(kSplitCycle, 0.0f);
+  for (int k = 0; k < m; ++k)  // damping of the large eigenvalues of 1 - T first
+    im.cw[k] = static_cast<float>(std::cos((2 * m - th[k]) * 3.14159265358979323846 / (2.0 * m)));
+  return im;
+}
+
+cudaError_t launch_scatter_split(const GridParams& g, const SplitTables& sp, const BfTables& t, const float* Q,
+                                 const float* mut, const float* eps, const float* nidx, float* Iring, float* Sring,
+                                 float tol, int max_iters, RunState rs, cudaStream_t st) {
+  CUtensorMap mI, mS;
+  std::memset(&mI, 0, sizeof(mI));
+  std::memset(&mS, 0, sizeof(mS));
+  const int tma_out = (t.out_maps && g.na % 64 == 0) ? 1 : 0;
+  if (tma_out) {
+    std::memcpy(&mI, t.out_maps, sizeof(CUtensorMap));
+    std::memcpy(&mS, static_cast<const unsigned char*>(t.out_maps) + 128, sizeof(CUtensorMap));
+  }
+  const int ntiles = brick_tiles(g.nx, g.ny, g.nz);
+  const int grid = ntiles < g_split_sms ? ntiles : g_split_sms;
+  const bool uni = g.mut_u >= 0.0f;
+  if (g_split_sms == 0) return cudaErrorInvalidValue;
+  if (g.na == 48) {
+    auto k = uni ? scatter_split_kernel<48, true> : scatter_split_kernel<48, false>;
+    k<<<grid, Sp<48>::kThreads, Sp<48>::SMEM, st>>>(g, sp, t.cls, t.cls_ds, t.ncls, t.nch, Q, mut, eps, nidx, Iring,
+                                                    Sring, tol, max_iters, mI, mS, tma_out, rs);
+  } else if (g.na == 192) {
+    auto k = uni ? scatter_split_kernel<192, true> : scatter_split_kernel<192, false>;
+    k<<<grid, Sp<192>::kThreads, Sp<192>::SMEM, st>>>(g, sp, t.cls, t.cls_ds, t.ncls, t.nch, Q, mut, eps, nidx,
+                                                      Iring, Sring, tol, max_iters, mI, mS, tma_out, rs);
+  } else {
+    return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace trinity

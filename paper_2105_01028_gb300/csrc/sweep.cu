@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(256) sweep_kernel(GridParams g, const DirInfo*
                                                     float* __restrict__ Q, RunState rs) {
   __shared__ DirInfo di_s;
   __shared__ int n_s, m_s;
-  __shared__ float f_s, T_s, b0_s;
+  __shared__ float f_s, T_s, b0_s, b0l_s;
   __shared__ const float* ilev_s[5];  // plane d of I at level n - m, null before the history
   __shared__ const float* slev_s[5];
   const int d = blockIdx.y;
@@ -83,9 +83,11 @@ __global__ void __launch_bounds__(256) sweep_kernel(GridParams g, const DirInfo*
     }
     if (kUniMu) {
       const float xo = g.mut_u * di.ds;
-      const float T = expf(-xo);
+      float T = expf(-xo), b0 = ray_b0(xo, T), lo = 0.0f;
+      if (g.fine) ray_weights_fine(g.mut_u, di.ds, di.ds_lo, T, b0, lo);
       T_s = T;
-      b0_s = ray_b0(xo, T);
+      b0_s = b0;
+      b0l_s = lo;
     }
   }
   __syncthreads();
@@ -99,7 +101,7 @@ __global__ void __launch_bounds__(256) sweep_kernel(GridParams g, const DirInfo*
   const int nrows = g.ny * g.nz;
   const int n = n_s;
   const int dom = di_s.dom, sgn = di_s.sgn, a0 = di_s.a0, a1 = di_s.a1;
-  const float ds = di_s.ds, dc_hi = di_s.dcoef, dc_lo = di_s.dcoef_lo, src_amp = di_s.src_amp;
+  const float ds = di_s.ds, ds_lo = di_s.ds_lo, dc_hi = di_s.dcoef, dc_lo = di_s.dcoef_lo, src_amp = di_s.src_amp;
   const size_t plane = static_cast<size_t>(g.nv);
   const int8_t* off0 = offs + (static_cast<size_t>(d) * 2 + 0) * g.nmax;
   const int8_t* off1 = offs + (static_cast<size_t>(d) * 2 + 1) * g.nmax;
@@ -112,7 +114,7 @@ __global__ void __launch_bounds__(256) sweep_kernel(GridParams g, const DirInfo*
   const size_t lev0 = static_cast<size_t>(d) * plane;
   const int m_u = kUniN ? m_s : 0;
   const float f_u = kUniN ? f_s : 0.0f;
-  const float T_u = kUniMu ? T_s : 0.0f, b0_u = kUniMu ? b0_s : 0.0f;
+  const float T_u = kUniMu ? T_s : 0.0f, b0_u = kUniMu ? b0_s : 0.0f, b0l_u = kUniMu ? b0l_s : 0.0f;
 
   // Q of voxel v from its upwind sample u (kind 0), the inflow face (kind 1) or a side face
   // (kind 2: nothing enters, or with mirror faces the image); (qd, q0, q1) are the upwind
@@ -166,16 +168,22 @@ __global__ void __launch_bounds__(256) sweep_kernel(GridParams g, const DirInfo*
       const float on1 = (L1 >= 0 && L1 < g.pulse_steps) ? 1.0f : 0.0f;
       Iup = src_amp * fmaf(f, on1, (1.0f - f) * on0);
     }
-    float T, b0;
+    float T, b0, b0l = 0.0f;
     if (kUniMu) {
       T = T_u;
       b0 = b0_u;
+      b0l = b0l_u;
     } else {
-      const float xo = __ldg(mut + v) * ds;
-      T = expf(-xo);
-      b0 = ray_b0(xo, T);
+      const float mu = __ldg(mut + v);
+      if (g.fine) {
+        ray_weights_fine(mu, ds, ds_lo, T, b0, b0l);
+      } else {
+        const float xo = mu * ds;
+        T = expf(-xo);
+        b0 = ray_b0(xo, T);
+      }
     }
-    Q[lev0 + v] = fmaf(Sup, b0, Iup * T);
+    Q[lev0 + v] = fmaf(Sup, b0, fmaf(Sup, b0l, Iup * T));
   };
 
   for (int row = blockIdx.x * blockDim.y + threadIdx.y; row < nrows; row += gridDim.x * blockDim.y) {

@@ -98,7 +98,7 @@ struct Box {
 // Per-direction constants of the current step (same for all of its items).
 struct DirStep {
   int d, sgn, m;
-  float f, T, b0, src_amp;
+  float f, T, b0, b0l, src_amp;  // per-voxel weights: b0, b0l hold the spacing and its remainder
   int p0, p1;       // plane coordinates of levels n - m and n - m - 1 in the ring tensor
   bool h0, h1;      // the level lies in the stored history (else it reads as zero)
 };
@@ -166,13 +166,16 @@ __global__ void __launch_bounds__(256) sweep_tma_kernel(GridParams g, const DirI
     s.m = m < 1 ? 1 : (m > 3 ? 3 : m);
     s.f = f;
     s.src_amp = di.src_amp;
+    s.b0l = 0.0f;
     if (kUniMu) {
       const float xo = g.mut_u * di.ds;
       s.T = expf(-xo);
       s.b0 = ray_b0(xo, s.T);
+      if (g.fine) ray_weights_fine(g.mut_u, di.ds, di.ds_lo, s.T, s.b0, s.b0l);
     } else {
       s.T = 0.0f;
-      s.b0 = di.ds;  // the spacing, for the per-voxel weights
+      s.b0 = di.ds;
+      s.b0l = di.ds_lo;
     }
     const int L0 = n - s.m, L1 = n - s.m - 1;
     s.h0 = L0 >= g.hist_from;
@@ -279,16 +282,22 @@ __global__ void __launch_bounds__(256) sweep_tma_kernel(GridParams g, const DirI
         Iup = fmaf(w1, i1, w0 * i0);
         Sup = fmaf(w1, s1v, w0 * s0v);
       }
-      float T, b0;
+      float T, b0, b0l = 0.0f;
       if (kUniMu) {
         T = s.T;
         b0 = s.b0;
+        b0l = s.b0l;
       } else {
-        const float xo = __ldg(mut + v) * s.b0;
-        T = expf(-xo);
-        b0 = ray_b0(xo, T);
+        const float mu = __ldg(mut + v);
+        if (g.fine) {
+          ray_weights_fine(mu, s.b0, s.b0l, T, b0, b0l);
+        } else {
+          const float xo = mu * s.b0;
+          T = expf(-xo);
+          b0 = ray_b0(xo, T);
+        }
       }
-      Qd[v] = fmaf(Sup, b0, Iup * T);
+      Qd[v] = fmaf(Sup, b0, fmaf(Sup, b0l, Iup * T));
     };
     if (DOM == 2 || DOM == 1) {
       // warps over the item's rows, lanes along x

@@ -28,7 +28,7 @@ struct Child {
   const int8_t* off1;
   float* qf;             // plane d of Q_f
   int dom, sgn, a0, a1, nd, n0, n1, sd, s0, s1;
-  float ds, dc_hi, dc_lo, src_amp;
+  float ds, ds_lo, dc_hi, dc_lo, src_amp;
   int m;                 // uniform refractive index: the delay's whole part ...
   float f, T, b0;        // ... and fraction; uniform mu_t: exp(-x) and b0(x)
 };
@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(256, 5) sweep2_kernel(GridParams g, const DirI
     ch.s0 = di.a0 == 0 ? 1 : (di.a0 == 1 ? g.nx : g.nx * g.ny);
     ch.s1 = di.a1 == 0 ? 1 : (di.a1 == 1 ? g.nx : g.nx * g.ny);
     ch.ds = di.ds;
+    ch.ds_lo = di.ds_lo;
     ch.dc_hi = di.dcoef;
     ch.dc_lo = di.dcoef_lo;
     ch.src_amp = di.src_amp;
@@ -107,9 +108,10 @@ __global__ void __launch_bounds__(256, 5) sweep2_kernel(GridParams g, const DirI
     }
     if (kUniMu) {
       const float xo = g.mut_u * di.ds;
-      const float T = expf(-xo);
-      ch.T = T;
-      ch.b0 = ray_b0(xo, T);
+      float lo;
+      ch.T = expf(-xo);
+      ch.b0 = ray_b0(xo, ch.T);
+      if (g.fine) ray_weights_fine(g.mut_u, di.ds, di.ds_lo, ch.T, ch.b0, lo);
     }
     cs[k] = ch;
   }
@@ -202,8 +204,10 @@ __global__ void __launch_bounds__(256, 5) sweep2_kernel(GridParams g, const DirI
             b0 = ch.b0;
           } else {
             const float xo = mu * ch.ds;
+            float lo;
             T = expf(-xo);
             b0 = ray_b0(xo, T);
+            if (g.fine) ray_weights_fine(mu, ch.ds, ch.ds_lo, T, b0, lo);
           }
           const float q = Iup * T + Sup * b0;
           ch.qf[v] = q;
