@@ -407,8 +407,8 @@ void trinity_serve_destroy(trinity_server* srv);
  * the code runs where allocation is forbidden).  It runs the per-voxel source iteration
  * S = (1 - eps) P (Q + b1 o S) of the FP32 mode (same arithmetic and stop rule as
  * trinity_step) on caller-owned device buffers and allocates no device memory: its
- * scratch (per-voxel contraction bounds, a max-reduction cell, iteration counters) is a
- * static device array of 4 MiB + 16 B that every GPU loading the library holds until the
+ * scratch (per-voxel contraction bounds, a max-reduction cell, iteration counters, the
+ * phase matrix split for the tensor cores) is a static device array of 4.2 MiB that every GPU loading the library holds until the
  * process exits.
  *   na       12, 48 or 192 directions; nvox voxels, 1 <= nvox <= 1048576 (the scratch
  *            limit: larger sizes return TRINITY_E_INVALID without running).

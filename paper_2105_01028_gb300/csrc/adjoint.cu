@@ -28,24 +28,6 @@ __device__ __forceinline__ int pick(int axis, int x, int y, int z) {
   return axis == 0 ? x : (axis == 1 ? y : z);
 }
 
-// db1/dx = b0(x) / x.  Below x = 1 the series of b0 divided by x (summed to x^10).
-__device__ __forceinline__ float ray_b0_over_x(float x, float T) {
-  if (x < 1.0f) {
-    float p = 1.0f / 43545600.0f;
-    p = fmaf(p, x, -1.0f / 3991680.0f);
-    p = fmaf(p, x, 1.0f / 403200.0f);
-    p = fmaf(p, x, -1.0f / 45360.0f);
-    p = fmaf(p, x, 1.0f / 5760.0f);
-    p = fmaf(p, x, -1.0f / 840.0f);
-    p = fmaf(p, x, 1.0f / 144.0f);
-    p = fmaf(p, x, -1.0f / 30.0f);
-    p = fmaf(p, x, 1.0f / 8.0f);
-    p = fmaf(p, x, -1.0f / 3.0f);
-    return fmaf(p, x, 0.5f);
-  }
-  return (1.0f - (1.0f + x) * T) / (x * x);
-}
-
 // db0/dx = [T (1 + x + x^2) - 1] / x^2.  Below x = 1 its Taylor series
 // sum_{j>=1} (-1)^(j+1) j^2 / (j+1)! x^(j-1), summed to j = 13.
 __device__ __forceinline__ float ray_db0(float x, float T) {
@@ -112,7 +94,8 @@ __global__ void adj_inject_kernel(const int* __restrict__ det_vox, const int* __
 }
 
 // ----------------------------------------------------------------------------------------
-// Transposed scattering solve, FP32 on CUDA cores.  Same tiling and iteration as the
+// Transposed scattering solve, FP32 on CUDA cores (12 directions; more run on the tensor
+// cores, scatter_split.cu, mode kAdjoint).  Same tiling and iteration as the
 // forward FP32 kernel (a CTA owns 16 voxels, thread i owns direction i, blocked sums of
 // P X with the diagonal row-sum correction r_i, y = (1 - eps) (P X + r X), the same stop
 // rule with a stall exit, the same isotropic rebalance after each plain update) with
@@ -507,21 +490,10 @@ cudaError_t launch_adj_scatter_fp32(const GridParams& g, const DirInfo* dirs, co
                                     int max_iters, const unsigned* yglob_prev, unsigned* ymax_cur,
                                     int* nonconv, unsigned long long* iters_sum, cudaStream_t st) {
   const int tiles = (g.nv + kTile - 1) / kTile;
-#define TRINITY_ADJ_CASE(NA)                                                                   \
-  case NA:                                                                                     \
-    adj_scatter_fp32_kernel<NA><<<tiles, AdjCfg<NA>::kThreads, 0, st>>>(                       \
-        g.nv, dirs, g.ds_max, P, rcorr, mut, eps, Ib_n, Sb_n, I_n, S_n, Y, Y2, extrap, Qb, gA,  \
-        gmut, tol,                                                                             \
-        max_iters, yglob_prev, ymax_cur, nonconv, iters_sum);                                  \
-    break;
-  switch (g.na) {
-    TRINITY_ADJ_CASE(12)
-    TRINITY_ADJ_CASE(48)
-    TRINITY_ADJ_CASE(192)
-    default:
-      return cudaErrorInvalidValue;
-  }
-#undef TRINITY_ADJ_CASE
+  if (g.na != 12) return cudaErrorInvalidValue;  // 48 and 192 directions: scatter_split.cu
+  adj_scatter_fp32_kernel<12><<<tiles, AdjCfg<12>::kThreads, 0, st>>>(
+      g.nv, dirs, g.ds_max, P, rcorr, mut, eps, Ib_n, Sb_n, I_n, S_n, Y, Y2, extrap, Qb, gA, gmut, tol, max_iters,
+      yglob_prev, ymax_cur, nonconv, iters_sum);
   return cudaGetLastError();
 }
 

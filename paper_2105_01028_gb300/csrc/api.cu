@@ -49,7 +49,8 @@ struct trinity_ctx {
   float* P32 = nullptr;
   uint16_t* Pbf = nullptr;
   // FP32 iteration on the tensor cores: one buffer holds the split phase matrix and tables
-  bool split = false;
+  bool split = false;        // forward steps use it (FP32, 48 or 192 directions)
+  bool split_ready = false;  // d_split holds the current phase matrix
   uint8_t* d_split = nullptr;
   SplitTables sp{};
   DirInfo* d_dirs = nullptr;
@@ -391,6 +392,7 @@ size_t split_bytes(int na) {
 
 // Build the split of the phase matrix for the tensor-core iteration and upload it.
 int upload_split(trinity_ctx* ctx, const std::vector<double>& P, int na, double g) {
+  if (!ctx->d_split) CK(dalloc(&ctx->d_split, split_bytes(na)));
   const SplitImage im = scatter_split_image(P, na, g);
   std::vector<uint8_t> buf(split_bytes(na));
   uint8_t* p = buf.data();
@@ -417,6 +419,7 @@ int upload_split(trinity_ctx* ctx, const std::vector<double>& P, int na, double 
     ctx->graph = nullptr;
   }
   ctx->sp = t;
+  ctx->split_ready = true;
   return TRINITY_OK;
 }
 
@@ -971,12 +974,11 @@ int trinity_create_grid(const trinity_grid_desc* desc, void* cuda_stream, trinit
     }
     ctx->ncls = static_cast<int>(cds.size());
     if (desc->precision == TRINITY_BF16 && ctx->ncls > 16) return bail(TRINITY_E_UNSUPPORTED);
-    // FP32 on the tensor cores: 48 or 192 directions whose spacings fall into 16 classes
-    ctx->split = desc->precision == TRINITY_FP32 && scatter_split_supported(static_cast<int>(na_s), ctx->ncls);
-    if (ctx->split && dalloc(&ctx->d_split, split_bytes(static_cast<int>(na_s))) != cudaSuccess) {
-      cudaGetLastError();
-      return bail(TRINITY_E_OOM);
-    }
+    // FP32 on the tensor cores from 48 directions on (their spacings fall into 5 classes, 15
+    // at 192, also as the children's lists of a two-level grid)
+    ctx->split = desc->precision == TRINITY_FP32 && na_s >= 48;
+    if (ctx->split && !scatter_split_supported(static_cast<int>(na_s), ctx->ncls))
+      return bail(TRINITY_E_UNSUPPORTED);
     std::vector<float> flat(16 * static_cast<size_t>(nch), 0.0f);
     for (size_t k = 0; k < cds.size() && k < 16; ++k)
       std::copy(cds[k].begin(), cds[k].end(), flat.begin() + k * nch);
@@ -1091,6 +1093,7 @@ int trinity_set_optics(trinity_ctx* ctx, const float* mua, const float* mus, con
   CK(cudaMemcpy(ctx->nidx, r.data(), nv * 4, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(ctx->P32, P32.data(), P32.size() * 4, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(ctx->Pbf, Pb.data(), Pb.size() * 2, cudaMemcpyHostToDevice));
+  ctx->split_ready = false;
   if (ctx->split) {
     const int rc4 = upload_split(ctx, P, na, g);
     if (rc4 != TRINITY_OK) return rc4;
@@ -1452,6 +1455,12 @@ int trinity_run_checkpointed(trinity_ctx* ctx, int nsteps, int every) {
     return fail(ctx, TRINITY_E_STATE, "a checkpointed run starts at step 0 (call trinity_reset)");
   int rc = lock_inputs(ctx);
   if (rc != TRINITY_OK) return rc;
+  if (ctx->na_s >= 48 && !ctx->split_ready) {  // BF16 forward: the reverse sweep is FP32
+    if (!scatter_split_supported(ctx->na_s, ctx->ncls))
+      return fail(ctx, TRINITY_E_UNSUPPORTED, "the transposed solve does not fit this device");
+    rc = upload_split(ctx, std::vector<double>(ctx->h_P32.begin(), ctx->h_P32.end()), ctx->na_s, ctx->g_aniso);
+    if (rc != TRINITY_OK) return rc;
+  }
   rc = ensure_capacity(ctx, nsteps);
   if (rc != TRINITY_OK) return rc;
   free_adjoint(ctx);
@@ -1600,13 +1609,34 @@ int adjoint_impl(trinity_ctx* ctx, const double* dL_dE, size_t n, double* grad_m
       CK(mark(3, true));
       CK(launch_adj_inject(ctx->d_det_vox, ctx->d_det_dir, ctx->d_det_w, ctx->d_det_id, ctx->n_det_entries,
                            ctx->d_G, ctx->nbins, bin, aI_n, g.nv, ctx->d_ymax + (lev & 1), ctx->stream));
-      CK(launch_adj_scatter_fp32(g, ctx->d_dirs, ctx->P32, ctx->d_rcorr32, ctx->mut, ctx->eps, aI_n, aS_n,
-                                 ctx->d_stI + here, ctx->d_stS + here, ctx->d_Y,
-                                 ctx->g.warm ? ctx->d_Y + lvl : nullptr, ctx->g.warm && lev <= N - 3 ? 1 : 0,
-                                 ctx->d_Qb, ctx->d_gA,
-                                 ctx->d_gmut, tol, ctx->desc.max_iters, ctx->d_ymax + ((lev + 1) & 1),
-                                 ctx->d_ymax + (lev & 1), ctx->d_adj_nonconv, ctx->d_adj_iters,
-                                 ctx->stream));
+      const int extrap = ctx->g.warm && lev <= N - 3 ? 1 : 0;
+      if (ctx->split_ready) {
+        SplitIo io{};
+        io.q = io.sb = aS_n;
+        io.ib = aI_n;
+        io.s1 = io.y = ctx->d_Y;
+        io.y2 = ctx->g.warm ? ctx->d_Y + lvl : nullptr;
+        io.s2 = extrap ? ctx->d_Y + lvl : nullptr;
+        io.eps = ctx->eps;
+        io.mut = ctx->mut;
+        io.i_n = ctx->d_stI + here;
+        io.s_n = ctx->d_stS + here;
+        io.qb = ctx->d_Qb;
+        io.gA = ctx->d_gA;
+        io.gmut = ctx->d_gmut;
+        io.s_glob = ctx->d_ymax + ((lev + 1) & 1);
+        CK(launch_adj_scatter_split(ctx->g_s, ctx->sp, bf_tables(ctx), io, tol, ctx->desc.max_iters,
+                                    ctx->d_ymax + (lev & 1), ctx->d_adj_nonconv, ctx->d_adj_iters, ctx->d_error,
+                                    ctx->stream));
+      } else {
+        CK(launch_adj_scatter_fp32(g, ctx->d_dirs, ctx->P32, ctx->d_rcorr32, ctx->mut, ctx->eps, aI_n, aS_n,
+                                   ctx->d_stI + here, ctx->d_stS + here, ctx->d_Y,
+                                   ctx->g.warm ? ctx->d_Y + lvl : nullptr, extrap,
+                                   ctx->d_Qb, ctx->d_gA,
+                                   ctx->d_gmut, tol, ctx->desc.max_iters, ctx->d_ymax + ((lev + 1) & 1),
+                                   ctx->d_ymax + (lev & 1), ctx->d_adj_nonconv, ctx->d_adj_iters,
+                                   ctx->stream));
+      }
       CK(mark(3, false));
       CK(mark(4, true));
       CK(launch_interface(ctx->n_iface, g.na, ctx->d_if_vox, ctx->d_ift_rowptr, ctx->d_ift_src,

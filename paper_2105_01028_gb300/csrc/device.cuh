@@ -136,6 +136,24 @@ __device__ __forceinline__ float ray_b1(float x, float T) {
   return (x - 1.0f + T) / x;
 }
 
+// db1/dx = b0(x) / x.  Below x = 1 the series of b0 divided by x (summed to x^10).
+__device__ __forceinline__ float ray_b0_over_x(float x, float T) {
+  if (x < 1.0f) {
+    float p = 1.0f / 43545600.0f;
+    p = fmaf(p, x, -1.0f / 3991680.0f);
+    p = fmaf(p, x, 1.0f / 403200.0f);
+    p = fmaf(p, x, -1.0f / 45360.0f);
+    p = fmaf(p, x, 1.0f / 5760.0f);
+    p = fmaf(p, x, -1.0f / 840.0f);
+    p = fmaf(p, x, 1.0f / 144.0f);
+    p = fmaf(p, x, -1.0f / 30.0f);
+    p = fmaf(p, x, 1.0f / 8.0f);
+    p = fmaf(p, x, -1.0f / 3.0f);
+    return fmaf(p, x, 0.5f);
+  }
+  return (1.0f - (1.0f + x) * T) / (x * x);
+}
+
 // Sweep weights T = e^-x and b0 of a segment x = mu ds, as the FP32 source iteration needs
 // them (lo: remainder of b0):
 //  - the rounding error of x = fl(mu fl(ds)) is carried into T to first order (15 mean free
@@ -204,11 +222,29 @@ struct SplitImage {
 struct SplitTables {
   const uint8_t *ph, *pl;
   const float *diag, *cw;
+  const float* dyn;  // unit, lam, lo on the device, or null: the values below
   int cycle, max_inner;
   float unit;     // one unit of Ph
   float lam, lo;  // spectrum of the rebalanced iteration: rho lam [lo, 1]
 };
+// Buffers of one launch (see SplitMode in scatter_split.cu).
+struct SplitIo {
+  const float *q, *s1, *s2;      // Q (adjoint: Sbar), start of the iteration and level before it
+  const float *eps, *mut, *nidx;
+  const float* b1;               // buffers: b1 per (direction, voxel)
+  const unsigned* s_glob;        // buffers, adjoint: max of the level before, as float bits
+  float *I, *S;                  // step: rings; buffers: outputs
+  float *ib, *sb;                // adjoint: Ibar, Sbar of the level (cleared)
+  const float *i_n, *s_n;        // adjoint: I and S of the level
+  float *y, *y2, *qb;            // adjoint: y(n+1) -> y(n), y(n+2) -> y(n+1) or null, Qbar
+  double *gA, *gmut;             // adjoint: gradient sums per voxel
+};
 bool scatter_split_supported(int na, int ncls);
+cudaError_t launch_adj_scatter_split(const GridParams& g, const SplitTables& sp, const BfTables& t, const SplitIo& io,
+                                     float tol, int max_iters, unsigned* ymax_cur, int* nonconv,
+                                     unsigned long long* iters_sum, int* error, cudaStream_t st);
+cudaError_t launch_scatter_split_buffers(int na, int nvox, const SplitTables& sp, const SplitIo& io, float tol,
+                                         int max_iters, int* iters_max, int* nonconv, int* error, cudaStream_t st);
 SplitImage scatter_split_image(const std::vector<double>& P, int na, double g_aniso);
 cudaError_t launch_scatter_split(const GridParams& g, const SplitTables& sp, const BfTables& t, const float* Q,
                                  const float* mut, const float* eps, const float* nidx, float* Iring, float* Sring,

@@ -15,7 +15,8 @@ __device__ __forceinline__ int pick(int axis, int x, int y, int z) {
 }
 
 // ----------------------------------------------------------------------------------------
-// Source iteration on CUDA cores (plain FP32 mode).
+// Source iteration on CUDA cores (FP32 mode at 12 directions; more run on the tensor
+// cores, scatter_split.cu, whose operand rows 12 directions would not fill).
 // A CTA owns a tile of kTile voxels; thread i < NA owns outgoing direction i of all of them.
 // Isotropic rebalance (angular two-grid correction): after each plain update S_half of
 // S_k, the voxel's isotropic error component is removed.  The error of S_half,
@@ -464,22 +465,9 @@ cudaError_t launch_scatter_fp32(const GridParams& g, const float* b1ds, int nch,
                                 const float* eps, const float* nidx, float* Iring, float* Sring,
                                 float tol, int max_iters, RunState rs, cudaStream_t st) {
   const int tiles = (g.nv + kTile - 1) / kTile;
-  switch (g.na) {
-    case 12:
-      scatter_fp32_kernel<12><<<tiles, ScatterCfg<12>::kThreads, 0, st>>>(
-          g, b1ds, nch, P, rcorr, Q, mut, eps, nidx, Iring, Sring, tol, max_iters, rs);
-      break;
-    case 48:
-      scatter_fp32_kernel<48><<<tiles, ScatterCfg<48>::kThreads, 0, st>>>(
-          g, b1ds, nch, P, rcorr, Q, mut, eps, nidx, Iring, Sring, tol, max_iters, rs);
-      break;
-    case 192:
-      scatter_fp32_kernel<192><<<tiles, ScatterCfg<192>::kThreads, 0, st>>>(
-          g, b1ds, nch, P, rcorr, Q, mut, eps, nidx, Iring, Sring, tol, max_iters, rs);
-      break;
-    default:
-      return cudaErrorInvalidValue;
-  }
+  if (g.na != 12) return cudaErrorInvalidValue;  // 48 and 192 directions: scatter_split.cu
+  scatter_fp32_kernel<12><<<tiles, ScatterCfg<12>::kThreads, 0, st>>>(g, b1ds, nch, P, rcorr, Q, mut, eps, nidx, Iring,
+                                                                      Sring, tol, max_iters, rs);
   return cudaGetLastError();
 }
 

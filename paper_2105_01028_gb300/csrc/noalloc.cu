@@ -9,6 +9,7 @@
 // contraction bounds, a max-reduction cell and iteration counters) lives in a
 // file-scope static device array of fixed size, which every GPU that loads the library
 // holds until the process exits.  Inputs and outputs are still the caller's.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <cstddef>
@@ -29,8 +30,14 @@ struct NoAllocScratch {
   unsigned smax;       // max |S_prev| as float bits (the stop rule's floor scale)
   int iters_max;       // largest iteration count of the call
   int nonconv;         // voxels that reached max_iters
-  int pad;
+  int error;           // device error word (a bounded wait ran out)
   float rho[kNoAllocMaxVoxels];  // per-voxel contraction bound (1 - eps) max_d b1
+  // the caller's P, split for the tensor cores (48 and 192 directions; see scatter_split.cu)
+  alignas(128) uint16_t ph[3 * 192 * 64];
+  alignas(128) uint16_t pl[3 * 192 * 64];
+  float diag[3 * 192];
+  float cw[64];
+  float dyn[4];        // unit, Chebyshev interval
 };
 
 static __device__ __align__(256) NoAllocScratch g_noalloc_scratch;
@@ -53,22 +60,150 @@ int scratch_for_current_device(NoAllocScratch** out) {
   return TRINITY_OK;
 }
 
-// Per voxel: rho = (1 - eps) max_d b1; and max |S_prev| over everything.
+// Max |S_prev| over everything and (b1 given: 12 directions) per voxel rho = (1 - eps) max_d b1.
 __global__ void noalloc_prepass(int na, int nvox, const float* __restrict__ b1, const float* __restrict__ eps,
                                 const float* __restrict__ S_prev, NoAllocScratch* sc) {
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   float sm = 0.0f;
   if (v < nvox) {
     float bmax = 0.0f;
+#pragma unroll 8
     for (int d = 0; d < na; ++d) {
-      bmax = fmaxf(bmax, b1[static_cast<size_t>(d) * nvox + v]);
+      if (b1) bmax = fmaxf(bmax, b1[static_cast<size_t>(d) * nvox + v]);
       sm = fmaxf(sm, fabsf(S_prev[static_cast<size_t>(d) * nvox + v]));
     }
-    sc->rho[v] = (1.0f - eps[v]) * bmax;
+    if (b1) sc->rho[v] = (1.0f - eps[v]) * bmax;
   }
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) sm = fmaxf(sm, __shfl_xor_sync(0xffffffffu, sm, o));
   if ((threadIdx.x & 31) == 0) atomicMax(&sc->smax, __float_as_uint(sm));
+}
+
+// Split of the caller's P on the device (the host form is scatter_split_image): one CTA.
+// The spectrum of P without the constant vector is estimated by power iteration (the
+// context path knows it from g): it sets the interval of the Chebyshev weights only, and an
+// eigenvalue above the estimate is still damped, as in the plain iteration.
+template <int NA>
+__global__ void __launch_bounds__(1024) noalloc_split_prep(const float* __restrict__ P, NoAllocScratch* sc) {
+  __shared__ float x_s[NA], y_s[NA];
+  __shared__ float red_s[32], red2_s[32];
+  __shared__ float pm_s, rm_s;
+  constexpr int kRows = 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // largest off-diagonal entry and row weight
+  float pm = 0.0f, rm = 0.0f;
+  for (int i = warp; i < NA; i += kRows) {
+    float s = 0.0f;
+    for (int j = lane; j < NA; j += 32)
+      if (j != i) {
+        const float p = fabsf(P[static_cast<size_t>(j) * NA + i]);
+        pm = fmaxf(pm, p);
+        s += p;
+      }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    rm = fmaxf(rm, s);
+  }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
+  if (lane == 0) {
+    red_s[warp] = pm;
+    red2_s[warp] = rm;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < kRows; ++w) {
+      pm = fmaxf(pm, red_s[w]);
+      rm = fmaxf(rm, red2_s[w]);
+    }
+    pm_s = pm;
+    rm_s = rm;
+  }
+  __syncthreads();
+  int t = 0;
+  while (t < 20 && ldexpf(pm_s, t + 1) <= 2046.0f && ldexpf(rm_s, t + 1) + NA / 2 <= 16128.0f) ++t;
+  const float whole = floorf(ldexpf(pm_s, t));
+  const float unit_f = whole >= 1.0f ? static_cast<float>(static_cast<double>(pm_s) / whole) : ldexpf(1.0f, -t);
+  const double unit = unit_f;
+  for (int i = warp; i < NA; i += kRows) {
+    double sh = 0.0, sl = 0.0;
+    for (int j = lane; j < NA; j += 32) {
+      double h = 0.0, l = 0.0;
+      if (j != i) {
+        const double u = static_cast<double>(P[static_cast<size_t>(j) * NA + i]) / unit;
+        h = rint(u);
+        l = rint((u - h) * 4096.0) / 4096.0;
+      }
+      sh += h;
+      sl += l;
+      const int k = j >> 6, ch = (j & 63) >> 3;
+      const int in_row = ((ch ^ (i & 7)) << 3) + (j & 7);
+      const int prow = NA >= 192 ? (k * (NA / 96) + i / 96) * 96 + i % 96 : k * NA + i;
+      sc->ph[(k * NA + i) * 64 + in_row] = __half_as_ushort(__float2half_rn(static_cast<float>(h)));
+      sc->pl[prow * 64 + in_row] = __half_as_ushort(__float2half_rn(static_cast<float>(l)));
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+      sh += __shfl_xor_sync(0xffffffffu, sh, o);
+      sl += __shfl_xor_sync(0xffffffffu, sl, o);
+    }
+    if (lane == 0) {
+      const double d = 1.0 - (sh + sl) * unit;
+      sc->diag[i] = static_cast<float>(d);
+      sc->diag[NA + i] = static_cast<float>(d - static_cast<double>(static_cast<float>(d)));
+      sc->diag[2 * NA + i] = static_cast<float>(1.0 - sh * unit);
+    }
+  }
+  // power iterations: the largest |eigenvalue| besides the constant vector's, then the
+  // largest of (that - eigenvalue), which tells how far the spectrum reaches below zero
+  float lam = 0.0f, low = 0.0f;
+#pragma unroll 1
+  for (int stage = 0; stage < 2; ++stage) {
+    for (int i = tid; i < NA; i += blockDim.x) {
+      unsigned h = (i + 1) * 2654435761u;
+      h ^= h >> 15;
+      x_s[i] = static_cast<float>(h & 0xffffu) / 65536.0f - 0.5f;
+    }
+    __syncthreads();
+    float norm0 = 1.0f;
+#pragma unroll 1
+    for (int it = 0; it < (stage == 0 ? 48 : 24); ++it) {
+      for (int i = warp; i < NA; i += kRows) {
+        float s = 0.0f;
+        for (int j = lane; j < NA; j += 32) s = fmaf(P[static_cast<size_t>(i) * NA + j], x_s[j], s);
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) y_s[i] = stage == 0 ? s : fmaf(lam, x_s[i], -s);
+      }
+      __syncthreads();
+      float m = 0.0f;  // every warp the same sums, in the same order
+      for (int j = lane; j < NA; j += 32) m += y_s[j];
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+      m /= NA;
+      float q = 0.0f;
+      for (int j = lane; j < NA; j += 32) q = fmaf(y_s[j] - m, y_s[j] - m, q);
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+      norm0 = sqrtf(q);
+      const float inv = norm0 > 1e-30f ? 1.0f / norm0 : 0.0f;
+      for (int j = tid; j < NA; j += blockDim.x) x_s[j] = (y_s[j] - m) * inv;
+      __syncthreads();
+    }
+    if (stage == 0)
+      lam = norm0;
+    else
+      low = lam - norm0;
+  }
+  if (tid == 0) {
+    const float l = fminf(fmaxf(lam, 0.0f) * 1.01f + 0.01f, 0.5f * (fminf(lam, 0.999f) + 1.0f));
+    sc->dyn[0] = unit_f;
+    sc->dyn[1] = l;
+    sc->dyn[2] = low < -0.02f ? -1.0f : 0.0f;
+    const int root[8] = {15, 1, 9, 7, 13, 3, 11, 5};  // as scatter_split_image orders them
+    for (int k = 0; k < 8; ++k) sc->cw[k] = cospif(root[k] / 16.0f);
+    for (int k = 8; k < 64; ++k) sc->cw[k] = 0.0f;
+  }
 }
 
 __device__ __forceinline__ float noalloc_transpose_max(float (&vals)[32], int lane) {
@@ -262,20 +397,43 @@ extern "C" int trinity_source_iteration_noalloc(int na, int nvox, const float* P
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the counters and the max cell start at zero on every call; rho is overwritten below
   if (cudaMemsetAsync(sc, 0, offsetof(NoAllocScratch, rho), st) != cudaSuccess) return TRINITY_E_CUDA;
-  noalloc_prepass<<<(nvox + 255) / 256, 256, 0, st>>>(na, nvox, b1, eps, S_prev, sc);
-  const int tiles = (nvox + kNaTile - 1) / kNaTile;
+  noalloc_prepass<<<(nvox + 255) / 256, 256, 0, st>>>(na, nvox, na == 12 ? b1 : nullptr, eps, S_prev, sc);
   const float ftol = static_cast<float>(tol);
-  if (na == 12)
+  if (na == 12) {
+    const int tiles = (nvox + kNaTile - 1) / kNaTile;
     noalloc_iteration<12><<<tiles, 32, 0, st>>>(nvox, P, Q, b1, eps, S_prev, S_out, I_out, ftol, max_iters, sc);
-  else if (na == 48)
-    noalloc_iteration<48><<<tiles, 64, 0, st>>>(nvox, P, Q, b1, eps, S_prev, S_out, I_out, ftol, max_iters, sc);
-  else
-    noalloc_iteration<192><<<tiles, 192, 0, st>>>(nvox, P, Q, b1, eps, S_prev, S_out, I_out, ftol, max_iters, sc);
+  } else {
+    if (!scatter_split_supported(na, 0)) return TRINITY_E_CUDA;
+    if (na == 48)
+      noalloc_split_prep<48><<<1, 1024, 0, st>>>(P, sc);
+    else
+      noalloc_split_prep<192><<<1, 1024, 0, st>>>(P, sc);
+    SplitTables sp{};
+    sp.ph = reinterpret_cast<const uint8_t*>(sc->ph);
+    sp.pl = reinterpret_cast<const uint8_t*>(sc->pl);
+    sp.diag = sc->diag;
+    sp.cw = sc->cw;
+    sp.dyn = sc->dyn;
+    sp.cycle = 8;
+    sp.max_inner = 256;
+    SplitIo io{};
+    io.q = Q;
+    io.s1 = S_prev;
+    io.eps = eps;
+    io.b1 = b1;
+    io.s_glob = &sc->smax;
+    io.I = I_out;
+    io.S = S_out;
+    if (launch_scatter_split_buffers(na, nvox, sp, io, ftol, max_iters, &sc->iters_max, &sc->nonconv, &sc->error, st) !=
+        cudaSuccess)
+      return TRINITY_E_CUDA;
+  }
   if (cudaGetLastError() != cudaSuccess) return TRINITY_E_CUDA;
-  int counters[2] = {0, 0};
+  int counters[3] = {0, 0, 0};
   if (cudaMemcpyAsync(counters, &sc->iters_max, sizeof(counters), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return TRINITY_E_CUDA;
+  if (counters[2] != 0) return TRINITY_E_TIMEOUT;
   if (iters_max) *iters_max = counters[0];
   return counters[1] > 0 ? TRINITY_W_NOT_CONVERGED : TRINITY_OK;
 }

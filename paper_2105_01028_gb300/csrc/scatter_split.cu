@@ -134,15 +134,21 @@ __device__ __forceinline__ void bulk_to_smem(uint32_t dst, const void* src, uint
                : "memory");
 }
 
+// What a launch solves for:
+//   kStep     S(n) of a forward step (Q and the S ring of a context; I and S written);
+//   kBuffers  the same on caller-owned buffers with b1 given per (direction, voxel);
+//   kAdjoint  the transposed solve y = a P (Sbar + b1 (Ibar + y)) of a reverse step: the
+//             same equation with Q = Sbar + b1 Ibar; the tile's end writes Qbar = Ibar + y,
+//             clears the consumed adjoint level and adds the gradient sums.
+enum SplitMode { kStep = 0, kBuffers = 1, kAdjoint = 2 };
+
 // kUniB1: mu_t is the same in every voxel, so b1 depends on the column's ray spacing only.
-template <int NA, bool kUniB1>
+template <int NA, bool kUniB1, int kMode>
 __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
     scatter_split_kernel(GridParams g, SplitTables t, const uint8_t* __restrict__ cls,
-                         const float* __restrict__ cls_ds, int ncls, int nch, const float* __restrict__ Q,
-                         const float* __restrict__ mut, const float* __restrict__ eps,
-                         const float* __restrict__ nidx, float* __restrict__ Iring, float* __restrict__ Sring,
-                         float tol, int max_iters, const __grid_constant__ CUtensorMap tmOutI,
-                         const __grid_constant__ CUtensorMap tmOutS, int tma_out, RunState rs) {
+                         const float* __restrict__ cls_ds, int ncls, int nch, SplitIo io, float tol, int max_iters,
+                         const __grid_constant__ CUtensorMap tmOutI, const __grid_constant__ CUtensorMap tmOutS,
+                         int tma_out, RunState rs) {
   using C = Sp<NA>;
   constexpr int CH = C::CH, NCH = C::NCH, NCT = C::NCT;
   extern __shared__ uint8_t smem_raw[];
@@ -177,16 +183,29 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
   const int row = ((warp & 3) << 5) + lane;
   const int grp = warp >> 2;  // column group
   const int cb = grp * C::HALF;
-  const int n = *rs.step;
+  const int n = kMode == kStep ? *rs.step : 0;
   const size_t plane = static_cast<size_t>(g.nv);
-  const float s_glob = __uint_as_float(rs.smax[(n - 1) & 1]);
-  const bool has_prev = (n - 1) >= g.hist_from;
-  const bool has_prev2 = g.warm != 0 && (n - 2) >= g.hist_from;  // linear extrapolation in time
-  const size_t prev_base = static_cast<size_t>(ring_slot(n - 1)) * g.na * plane;
-  const size_t prev2_base = static_cast<size_t>(ring_slot(n - 2)) * g.na * plane;
+  const float s_glob = __uint_as_float(kMode == kStep ? rs.smax[(n - 1) & 1] : *io.s_glob);
+  // start of the iteration: the previous level and, for the linear extrapolation in time,
+  // the one before it
+  const float* sp1 = io.s1;
+  const float* sp2 = io.s2;
+  if (kMode == kStep) {
+    sp1 = (n - 1) >= g.hist_from ? io.s1 + static_cast<size_t>(ring_slot(n - 1)) * g.na * plane : nullptr;
+    sp2 = g.warm != 0 && (n - 2) >= g.hist_from ? io.s1 + static_cast<size_t>(ring_slot(n - 2)) * g.na * plane
+                                                : nullptr;
+  }
   const size_t cur_base = static_cast<size_t>(ring_slot(n)) * g.na * plane;
   const int bxn = (g.nx + 7) >> 3, byn = (g.ny + 3) >> 2;
-  const int ntiles = brick_tiles(g.nx, g.ny, g.nz);
+  // flat tiles of 128 voxels where the voxels have no grid
+  const int ntiles = kMode == kBuffers ? (g.nv + kM - 1) / kM : brick_tiles(g.nx, g.ny, g.nz);
+  const auto tile_voxel = [&](int tl, int r) {
+    if (kMode == kBuffers) {
+      const int f = tl * kM + r;
+      return f < g.nv ? f : -1;
+    }
+    return brick_voxel(g, bxn, byn, tl, r);
+  };
 
   // ---- one-time set-up: TMEM, barriers, operand images, diagonals, class tables
   if (warp == 0) tmem_alloc(&tmem_base_s, C::TCOLS);
@@ -219,10 +238,11 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
   if (tid < kSplitCycle) cw_s[tid] = t.cw[tid];
   __syncthreads();
   for (int i = tid; i < NA; i += blockDim.x) {
-    atomicAdd(&ccnt_s[cls[i]], 1);
     sDi[i] = t.diag[i];
     sDi[NA + i] = t.diag[NA + i];
     sDi[2 * NA + i] = t.diag[2 * NA + i];
+    if (kMode == kBuffers) continue;
+    atomicAdd(&ccnt_s[cls[i]], 1);
     sCls[i] = cls[i];
     if (kUniB1) {  // the same operations as the per-row table below, on the same mu_t
       const int k = cls[i];
@@ -261,13 +281,29 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
   float smax_loc = 0.0f;
   float S[C::HALF];                       // S of the thread's row and columns
   float qr[C::QR > 0 ? C::QR : 1];        // Q of the thread's last QR columns
-  const float tscale = t.unit;            // one unit of Ph
+  // one unit of Ph and the Chebyshev interval (from the device where P came from there)
+  const float tscale = t.dyn ? t.dyn[0] : t.unit, lam = t.dyn ? t.dyn[1] : t.lam, lam_lo = t.dyn ? t.dyn[2] : t.lo;
   bool first_tile = true;
 
   // b1 of 8 columns from c0 on (volatile or asm loads: hoisted out of the iterations these
   // tables would cost more registers than there are)
-  const auto load_b1 = [&](int c0, float (&bv)[8]) {
-    if (kUniB1) {
+  // (kBuffers: from the caller's array; in the inner iterations as FP16, kept where Xl was)
+  int v = 0;
+  const auto load_b1 = [&](int c0, float (&bv)[8], bool inner_pass = false) {
+    if (kMode == kBuffers) {
+      if (inner_pass) {
+        const volatile __half* hb = reinterpret_cast<const volatile __half*>(sXl) + c0 * kM + row;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          __half_raw hr;
+          hr.x = reinterpret_cast<const volatile unsigned short*>(hb)[j * kM];
+          bv[j] = __half2float(__half(hr));
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) bv[j] = io.b1[static_cast<size_t>(c0 + j) * plane + v];
+      }
+    } else if (kUniB1) {
       lds_vec<8>(sB1c + c0, bv);
     } else {
       const volatile float* vb = b1t;
@@ -368,35 +404,41 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
     // before X is written again
     if (tid == 0) {
       if (tma_out) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-      tile_s = first_tile ? atomicAdd(rs.tile_ctr + (n & 1), 1) : next_s;
-      next_s = atomicAdd(rs.tile_ctr + (n & 1), 1);
+      if (kMode == kStep) {
+        tile_s = first_tile ? atomicAdd(rs.tile_ctr + (n & 1), 1) : next_s;
+        next_s = atomicAdd(rs.tile_ctr + (n & 1), 1);
+      } else {
+        tile_s = first_tile ? static_cast<int>(blockIdx.x) : tile_s + static_cast<int>(gridDim.x);
+      }
     }
     first_tile = false;
     __syncthreads();
     const int tile = tile_s;
     if (tile >= ntiles) break;
-    const int vb = brick_voxel(g, bxn, byn, tile, row);
+    const int vb = tile_voxel(tile, row);
     const bool vin = vb >= 0;
-    const int v = vin ? vb : 0;
+    v = vin ? vb : 0;
 
     // per-row constants and the b1 table over ds classes
     if (tid < kM) {
-      const int vv = brick_voxel(g, bxn, byn, tile, tid);
+      const int vv = tile_voxel(tile, tid);
       float ev = 1.0f, rho = 0.0f;
       if (vv >= 0) {
-        ev = eps[vv];
-        const float xm = mut[vv] * g.ds_max;
-        rho = (1.0f - ev) * ray_b1(xm, expf(-xm));
+        ev = io.eps[vv];
+        if (kMode != kBuffers) {
+          const float xm = io.mut[vv] * g.ds_max;
+          rho = (1.0f - ev) * ray_b1(xm, expf(-xm));
+        }
       }
       e_s[tid] = ev;
       rho_s[tid] = rho;
     }
-    for (int u = tid; u < (kUniB1 ? 0 : ncls * kM); u += blockDim.x) {
+    for (int u = tid; u < (kUniB1 || kMode == kBuffers ? 0 : ncls * kM); u += blockDim.x) {
       const int k = u / kM, r = u % kM;
-      const int vv = brick_voxel(g, bxn, byn, tile, r);
+      const int vv = tile_voxel(tile, r);
       float bs = 0.0f;
       if (vv >= 0) {
-        const float mu = mut[vv];
+        const float mu = io.mut[vv];
         for (int j = 0; j < nch; ++j) {
           const float x = mu * cls_ds[k * nch + j];
           bs += ray_b1(x, expf(-x));
@@ -406,7 +448,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
     }
     __syncthreads();
     // rebalance denominator sum_j (1 - a b1_j) of each row
-    if (tid < kM) {
+    if (tid < kM && kMode != kBuffers) {
       float sb;
       if (kUniB1) {
         sb = sumb1_s;
@@ -417,31 +459,39 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
       den_s[tid] = static_cast<float>(NA) - (1.0f - e_s[tid]) * sb;
     }
 
-    // ---- warm start S(n-1), or 2 S(n-1) - S(n-2), into registers; Q (read once) into TMEM
-    // or registers; max |X| of the row.  Loads go two chunks (48 per thread) at a time.
-    float xmax = 0.0f;
+    // ---- warm start (the previous level or its extrapolation in time) into registers; Q
+    // (read once) into TMEM or registers; max |X| of the row.  Loads go two chunks (48 per
+    // thread) at a time.
+    float xmax = 0.0f, bmax = 0.0f, bsum = 0.0f;
     {
       static_assert(NCH % 2 == 0 && NCT % 2 == 0, "chunks go in pairs");
+      constexpr int PR = kMode == kStep ? 2 : 1;
 #pragma unroll
-      for (int c2 = 0; c2 < NCH; c2 += 2) {
-        float s1[2][CH], s2[2][CH], qc[2][CH];
+      for (int c2 = 0; c2 < NCH; c2 += PR) {
+        float s1[PR][CH], s2[PR][CH], qc[PR][CH], qi[PR][CH];
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
+        for (int u = 0; u < PR; ++u)
 #pragma unroll
           for (int j = 0; j < CH; ++j) {
             const size_t col = static_cast<size_t>(cb + (c2 + u) * CH + j) * plane + v;
-            s1[u][j] = (vin && has_prev) ? __ldg(Sring + prev_base + col) : 0.0f;
-            s2[u][j] = (vin && has_prev2) ? __ldg(Sring + prev2_base + col) : 0.0f;
-            qc[u][j] = vin ? __ldg(Q + col) : 0.0f;
+            s1[u][j] = (vin && sp1) ? (kMode == kStep ? __ldg(sp1 + col) : sp1[col]) : 0.0f;
+            s2[u][j] = (vin && sp2) ? (kMode == kStep ? __ldg(sp2 + col) : sp2[col]) : 0.0f;
+            qc[u][j] = vin ? (kMode == kStep ? __ldg(io.q + col) : io.q[col]) : 0.0f;
+            qi[u][j] = (kMode == kAdjoint && vin) ? io.ib[col] : 0.0f;
           }
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < PR; ++u) {
           const int ch = c2 + u;
           float bv[8];
           load_b1(cb + ch * CH, bv);
 #pragma unroll
           for (int j = 0; j < CH; ++j) {
-            const float s0 = (vin && has_prev2) ? fmaf(2.0f, s1[u][j], -s2[u][j]) : s1[u][j];
+            if (kMode == kAdjoint) qc[u][j] = fmaf(bv[j], qi[u][j], qc[u][j]);  // Sbar + b1 Ibar
+            if (kMode == kBuffers) {
+              bmax = fmaxf(bmax, bv[j]);
+              bsum += bv[j];
+            }
+            const float s0 = (vin && sp2) ? fmaf(2.0f, s1[u][j], -s2[u][j]) : s1[u][j];
             S[ch * CH + j] = s0;
             xmax = fmaxf(xmax, fabsf(fmaf(bv[j], s0, qc[u][j])));
             if (ch >= NCT) qr[(ch - NCT) * CH + j] = qc[u][j];
@@ -451,12 +501,22 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
       }
     }
     red_d[grp][row] = xmax;
+    if (kMode == kBuffers) {
+      red_s[grp][row] = bmax;
+      red_c[grp][row] = bsum;
+    }
     tmem_wait_st();
     __syncthreads();
+    float den = den_s[row];
+    float rho = rho_s[row];
+    if (kMode == kBuffers) {
+      rho = (1.0f - e_s[row]) * row_max(red_s);
+      den = static_cast<float>(NA) - (1.0f - e_s[row]) * row_sum(red_c);
+    }
 
-    const float ev = e_s[row], al = 1.0f - ev, rho = rho_s[row];
+    const float ev = e_s[row], al = 1.0f - ev;
     const float amp = rho / (1.0f - rho);           // error bound per unit change
-    const float span = rho * t.lam;                 // Chebyshev interval [t.lo span, span]
+    const float span = rho * lam;                   // Chebyshev interval [lam_lo span, span]
     const float eta = kInnerError * fmaxf(1.0f, 0.08f * amp);
     bool live = vin;       // the row takes part in this outer iteration
     bool hitmax = false, bad = false;
@@ -520,8 +580,16 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
             float y = fmaf(dl[j], x, (a0[j] + a1[j]) * ky);
             y = fmaf(dv[j], x, y);
             const float sh = fmaf(-ev, y, y);
-            const float r = sh - s;
+            float r = sh - s;
+            if (kMode == kBuffers)
+              reinterpret_cast<__half*>(sXl)[(c0 + j) * kM + row] = __float2half_rn(bv[j]);
+            // adjoint, no scattering: y = 0 now; its P z goes where the residual would
             a0[j] = r;
+            if (kMode == kAdjoint && al == 0.0f) {
+              S[ch * CH + j] = 0.0f;
+              a0[j] = y;
+              r = 0.0f;
+            }
             rm = fmaxf(rm, fabsf(r));
             sm = fmaxf(sm, fabsf(sh));
             cs = fmaf(bv[j], r, cs);
@@ -538,25 +606,25 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
         aborted = true;
         break;
       }
-      bool inner = false, fin = !live;  // fin: S has taken its last r of this outer
+      bool inner = false, fin = !live || (kMode == kAdjoint && al == 0.0f);  // fin: S has taken its last r of this outer
       bool stalled = false;
       float target = 0.0f, es = 0.0f, crow = 0.0f;
       rm = row_max(red_d);
       if (live) {
         ++iters;
         thr = kTolShare * tol * fmaxf(row_max(red_s), 1e-6f * s_glob);
-        stalled = rm > 0.25f * prevr;
+        stalled = rm > 0.5f * prevr;
         prevr = rm;
         target = fmaxf(thr, amp * rm * kInnerDrop);
         const bool conv = amp * rm <= thr;
         inner = !conv && iters < max_iters && rm <= 3.0e38f;
         hitmax = !conv && !inner;
-        if (inner) crow = al * row_sum(red_c) / den_s[row];
+        if (inner) crow = al * row_sum(red_c) / den;
       }
       // ---- inner iterations on the error equation
       int k = 0;
       while (true) {
-        const float half = 0.5f * (span - t.lo * span), mid = 0.5f * (span + t.lo * span);
+        const float half = 0.5f * (span - lam_lo * span), mid = 0.5f * (span + lam_lo * span);
         const float om = 1.0f / (1.0f - fmaf(half, cw_s[k % t.cycle], mid));
         const float w = inner ? om : (fin ? 0.0f : 1.0f);
         const int er = scale_exponent(rm + fabsf(crow), 13);
@@ -567,7 +635,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
             const int c0 = cb + ch * CH;
             float rv[CH], bv[8];
             tmem_ld<CH>(t_row + C::ROFF + c0, rv);
-            load_b1(c0, bv);
+            load_b1(c0, bv, true);
             tmem_wait_ld();
             uint32_t hi[4];
 #pragma unroll
@@ -604,7 +672,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
             float rv[CH], dd[CH], bv[8], di[8];
             tmem_ld<CH>(t_row + c0, dd);
             tmem_ld<CH>(t_row + C::ROFF + c0, rv);
-            load_b1(c0, bv);
+            load_b1(c0, bv, true);
             lds_vec<8>(sDi + 2 * NA + c0, di);
             tmem_wait_ld();
 #pragma unroll
@@ -637,7 +705,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
             if (!conv && iters >= max_iters) hitmax = true;
             crow = 0.0f;
           } else {
-            crow = al * row_sum(red_c) / den_s[row];
+            crow = al * row_sum(red_c) / den;
           }
         }
       }
@@ -667,9 +735,62 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
     if (aborted) break;
     if (bad && grp == 0) atomicAdd(rs.nonconv, 1);
 
+    if constexpr (kMode == kAdjoint) {
+      // ---- Qbar, warm start of the next reverse step, cleared adjoint level, gradient sums
+      float ga = 0.0f, gm = 0.0f;
+      const float mu_v = vin ? io.mut[v] : 0.0f;
+      const float inv_al = al > 0.0f ? 1.0f / al : 0.0f;
+#pragma unroll
+      for (int ch = 0; ch < NCH; ++ch) {
+        const int c0 = cb + ch * CH;
+        float pz[CH];
+        if (__any_sync(0xffffffffu, al == 0.0f)) {
+          tmem_ld<CH>(t_row + C::ROFF + c0, pz);
+          tmem_wait_ld();
+        }
+        if (vin) {
+          float ib[CH], yo[CH], in[CH], sn[CH];
+#pragma unroll
+          for (int j = 0; j < CH; ++j) {
+            const size_t o = static_cast<size_t>(c0 + j) * plane + v;
+            ib[j] = io.ib[o];
+            yo[j] = io.y2 ? io.y[o] : 0.0f;
+            in[j] = __ldg(io.i_n + o);
+            sn[j] = __ldg(io.s_n + o);
+          }
+#pragma unroll
+          for (int j = 0; j < CH; ++j) {
+            const size_t o = static_cast<size_t>(c0 + j) * plane + v;
+            const float y = S[ch * CH + j], qbar = ib[j] + y;
+            io.qb[o] = qbar;
+            if (io.y2) io.y2[o] = yo[j];
+            io.y[o] = y;
+            io.ib[o] = 0.0f;
+            io.sb[o] = 0.0f;
+            smax_loc = fmaxf(smax_loc, fabsf(y));
+            ga = fmaf(in[j], al > 0.0f ? y * inv_al : pz[j], ga);  // I (P z)
+            const float ds = cls_ds[sCls[c0 + j]], x = mu_v * ds;
+            gm = fmaf(ds * sn[j] * qbar, ray_b0_over_x(x, expf(-x)), gm);
+          }
+        }
+      }
+      red_d[grp][row] = ga;
+      red_s[grp][row] = gm;
+      __syncthreads();
+      if (grp == 0 && vin) {
+        double sa = 0.0, sm = 0.0;
+#pragma unroll
+        for (int gi = 0; gi < kGroups; ++gi) {
+          sa += static_cast<double>(red_d[gi][row]);
+          sm += static_cast<double>(red_s[gi][row]);
+        }
+        io.gA[v] += sa;
+        io.gmut[v] += sm;
+      }
+    } else {
     // ---- write-out: I = Q + b1 S and S of every voxel
-    const float nv_v = vin ? nidx[v] : 0.0f;
-    const float mu_v = vin ? mut[v] : 0.0f;
+    const float nv_v = (kMode == kStep && vin) ? io.nidx[v] : 0.0f;
+    const float mu_v = (kMode == kStep && vin) ? io.mut[v] : 0.0f;
     float esum_row = 0.0f;
     if (C::KB * 64 == NA && tma_out) {
       // staged: I and then S of the tile go to the X operand area as 8-direction boxes of
@@ -720,8 +841,8 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
         if (pass == 0) __syncthreads();
       }
     } else {
-      float* pI = Iring + cur_base + static_cast<size_t>(cb) * plane + v;
-      float* pS = Sring + cur_base + static_cast<size_t>(cb) * plane + v;
+      float* pI = io.I + cur_base + static_cast<size_t>(cb) * plane + v;
+      float* pS = io.S + cur_base + static_cast<size_t>(cb) * plane + v;
 #pragma unroll
       for (int ch = 0; ch < NCH; ++ch) {
         float qv[CH], bv[8];
@@ -742,11 +863,14 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
         }
       }
     }
-    if (vin) esum += static_cast<double>(esum_row) * static_cast<double>(nv_v);
-    float ab = vin ? esum_row * (ev * mu_v) : 0.0f;
+    if (kMode == kStep) {
+      if (vin) esum += static_cast<double>(esum_row) * static_cast<double>(nv_v);
+      float ab = vin ? esum_row * (ev * mu_v) : 0.0f;
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) ab += __shfl_xor_sync(0xffffffffu, ab, o);
-    if (lane == 0) atomicAdd(&asum_sh, static_cast<double>(ab));
+      for (int o = 16; o >= 1; o >>= 1) ab += __shfl_xor_sync(0xffffffffu, ab, o);
+      if (lane == 0) atomicAdd(&asum_sh, static_cast<double>(ab));
+    }
+    }
     // iteration statistics of this tile (group-0 threads hold one row each)
     if (warp < 4) {
       int im = vin ? iters : 0;
@@ -757,8 +881,8 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
         is += __shfl_xor_sync(0xffffffffu, is, o);
       }
       if (lane == 0) {
-        atomicMax(rs.iters_max + n, im);
-        atomicAdd(rs.iters_sum + n, is);
+        if (rs.iters_max) atomicMax(rs.iters_max + n, im);
+        if (rs.iters_sum) atomicAdd(rs.iters_sum + n, is);
       }
     }
     __syncthreads();
@@ -791,9 +915,11 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
       e += esum_s[w];
       sm = fmaxf(sm, smax_s[w]);
     }
-    atomicAdd(rs.energy + n, e * static_cast<double>(g.e_scale));
-    atomicAdd(rs.absorbed + n, asum_sh * g.a_scale);
-    atomicMax(rs.smax + (n & 1), __float_as_uint(sm));
+    if (kMode == kStep) {
+      atomicAdd(rs.energy + n, e * static_cast<double>(g.e_scale));
+      atomicAdd(rs.absorbed + n, asum_sh * g.a_scale);
+    }
+    if (kMode != kBuffers) atomicMax(rs.smax + (n & 1), __float_as_uint(sm));
   }
   if (warp == 0) {
     tc_fence_after();
@@ -803,13 +929,36 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
 
 int g_split_sms = 0;
 
-template <int NA>
+template <int NA, int kMode>
 cudaError_t configure_split() {
-  cudaError_t e = cudaFuncSetAttribute(scatter_split_kernel<NA, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       Sp<NA>::SMEM);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(scatter_split_kernel<NA, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              Sp<NA>::SMEM);
+  cudaError_t e = cudaFuncSetAttribute(scatter_split_kernel<NA, false, kMode>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, Sp<NA>::SMEM);
+  if (e != cudaSuccess || kMode == kBuffers) return e;
+  return cudaFuncSetAttribute(scatter_split_kernel<NA, kMode != kBuffers, kMode>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, Sp<NA>::SMEM);
+}
+
+template <int kMode>
+cudaError_t launch_split(const GridParams& g, const SplitTables& sp, const BfTables& t, const SplitIo& io, float tol,
+                         int max_iters, const CUtensorMap& mI, const CUtensorMap& mS, int tma_out, const RunState& rs,
+                         cudaStream_t st) {
+  if (g_split_sms == 0) return cudaErrorInvalidValue;
+  const int ntiles = kMode == kBuffers ? (g.nv + kM - 1) / kM : brick_tiles(g.nx, g.ny, g.nz);
+  const int grid = ntiles < g_split_sms ? ntiles : g_split_sms;
+  constexpr bool kU = kMode != kBuffers;
+  const bool uni = kU && g.mut_u >= 0.0f;
+  if (g.na == 48) {
+    auto k = uni ? scatter_split_kernel<48, kU, kMode> : scatter_split_kernel<48, false, kMode>;
+    k<<<grid, Sp<48>::kThreads, Sp<48>::SMEM, st>>>(g, sp, t.cls, t.cls_ds, t.ncls, t.nch, io, tol, max_iters, mI, mS,
+                                                    tma_out, rs);
+  } else if (g.na == 192) {
+    auto k = uni ? scatter_split_kernel<192, kU, kMode> : scatter_split_kernel<192, false, kMode>;
+    k<<<grid, Sp<192>::kThreads, Sp<192>::SMEM, st>>>(g, sp, t.cls, t.cls_ds, t.ncls, t.nch, io, tol, max_iters, mI,
+                                                      mS, tma_out, rs);
+  } else {
+    return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
 }
 
 uint16_t half_bits(double x) {  // x is an FP16 number
@@ -827,7 +976,9 @@ bool scatter_split_supported(int na, int ncls) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        configure_split<48>() != cudaSuccess || configure_split<192>() != cudaSuccess) {
+        configure_split<48, kStep>() != cudaSuccess || configure_split<192, kStep>() != cudaSuccess ||
+        configure_split<48, kBuffers>() != cudaSuccess || configure_split<192, kBuffers>() != cudaSuccess ||
+        configure_split<48, kAdjoint>() != cudaSuccess || configure_split<192, kAdjoint>() != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
@@ -929,22 +1080,43 @@ cudaError_t launch_scatter_split(const GridParams& g, const SplitTables& sp, con
     std::memcpy(&mI, t.out_maps, sizeof(CUtensorMap));
     std::memcpy(&mS, static_cast<const unsigned char*>(t.out_maps) + 128, sizeof(CUtensorMap));
   }
-  const int ntiles = brick_tiles(g.nx, g.ny, g.nz);
-  const int grid = ntiles < g_split_sms ? ntiles : g_split_sms;
-  const bool uni = g.mut_u >= 0.0f;
-  if (g_split_sms == 0) return cudaErrorInvalidValue;
-  if (g.na == 48) {
-    auto k = uni ? scatter_split_kernel<48, true> : scatter_split_kernel<48, false>;
-    k<<<grid, Sp<48>::kThreads, Sp<48>::SMEM, st>>>(g, sp, t.cls, t.cls_ds, t.ncls, t.nch, Q, mut, eps, nidx, Iring,
-                                                    Sring, tol, max_iters, mI, mS, tma_out, rs);
-  } else if (g.na == 192) {
-    auto k = uni ? scatter_split_kernel<192, true> : scatter_split_kernel<192, false>;
-    k<<<grid, Sp<192>::kThreads, Sp<192>::SMEM, st>>>(g, sp, t.cls, t.cls_ds, t.ncls, t.nch, Q, mut, eps, nidx,
-                                                      Iring, Sring, tol, max_iters, mI, mS, tma_out, rs);
-  } else {
-    return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+  SplitIo io{};
+  io.q = Q;
+  io.s1 = Sring;
+  io.eps = eps;
+  io.mut = mut;
+  io.nidx = nidx;
+  io.I = Iring;
+  io.S = Sring;
+  return launch_split<kStep>(g, sp, t, io, tol, max_iters, mI, mS, tma_out, rs, st);
+}
+
+cudaError_t launch_adj_scatter_split(const GridParams& g, const SplitTables& sp, const BfTables& t, const SplitIo& io,
+                                     float tol, int max_iters, unsigned* ymax_cur, int* nonconv,
+                                     unsigned long long* iters_sum, int* error, cudaStream_t st) {
+  CUtensorMap m;
+  std::memset(&m, 0, sizeof(m));
+  RunState rs{};
+  rs.smax = ymax_cur;
+  rs.nonconv = nonconv;
+  rs.iters_sum = iters_sum;
+  rs.error = error;
+  return launch_split<kAdjoint>(g, sp, t, io, tol, max_iters, m, m, 0, rs, st);
+}
+
+cudaError_t launch_scatter_split_buffers(int na, int nvox, const SplitTables& sp, const SplitIo& io, float tol,
+                                         int max_iters, int* iters_max, int* nonconv, int* error, cudaStream_t st) {
+  CUtensorMap m;
+  std::memset(&m, 0, sizeof(m));
+  GridParams g{};
+  g.na = na;
+  g.nv = nvox;
+  g.mut_u = -1.0f;
+  RunState rs{};
+  rs.iters_max = iters_max;
+  rs.nonconv = nonconv;
+  rs.error = error;
+  return launch_split<kBuffers>(g, sp, BfTables{}, io, tol, max_iters, m, m, 0, rs, st);
 }
 
 }  // namespace trinity
