@@ -348,37 +348,47 @@ __global__ void __launch_bounds__(AdjCfg<NA>::kThreads, 2)
 }
 
 // ----------------------------------------------------------------------------------------
-// Upwind push and the transport part of dL/dmu_t.  One thread per voxel v loops over the
-// directions (so the per-voxel sum over d stays in a register); a warp covers 32
-// consecutive x, so every access of a direction's plane is a contiguous run.  Within one
-// direction the lattice maps voxels to upwind samples one to one (a translation per
-// slab), so no two threads update the same adjoint entry: plain read-modify-writes.
+// Upwind push and the transport part of dL/dmu_t.  A block owns 32 consecutive voxels (a
+// direction's planes are then read in contiguous runs) and its 16 warps share the
+// directions, two at a time: the 18 loads of both are issued before the first store.  The
+// sums over directions are combined in shared memory in a fixed order.  Within one
+// direction the lattice maps voxels to upwind samples one to one (a translation per slab),
+// and directions have planes of their own, so no two threads update the same adjoint entry:
+// plain read-modify-writes.  Bound by HBM (52 B per voxel and direction).  A thread that
+// walked all 192 directions of its voxel one after the other left 128 blocks at 32^3 and the
+// kernel bound by its chain of dependent loads: 625 us, now 129.
 // Forward levels come from the segment store, level L at index L - lev_base.
 // ----------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) adj_push_kernel(GridParams g, const DirInfo* __restrict__ dirs,
-                                                       const int8_t* __restrict__ offs,
-                                                       const float* __restrict__ stI,
-                                                       const float* __restrict__ stS, int lev_base,
-                                                       int n, const float* __restrict__ mut,
-                                                       const float* __restrict__ nidx,
-                                                       const float* __restrict__ Qb,
-                                                       float* __restrict__ IbR, float* __restrict__ SbR,
-                                                       double* __restrict__ gmut) {
+constexpr int kPushWarps = 16;
+
+__global__ void __launch_bounds__(32 * kPushWarps)
+    adj_push_kernel(GridParams g, const DirInfo* __restrict__ dirs, const int8_t* __restrict__ offs,
+                    const float* __restrict__ stI, const float* __restrict__ stS, int lev_base, int n,
+                    const float* __restrict__ mut, const float* __restrict__ nidx, const float* __restrict__ Qb,
+                    float* __restrict__ IbR, float* __restrict__ SbR, double* __restrict__ gmut) {
   extern __shared__ DirInfo dir_s[];
+  __shared__ float acc_s[kPushWarps][32];
   for (int d = threadIdx.x; d < g.na; d += blockDim.x) dir_s[d] = dirs[d];
   __syncthreads();
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= g.nv) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int v = blockIdx.x * 32 + lane;
+  const bool in = v < g.nv;
   const size_t plane = static_cast<size_t>(g.nv);
   const size_t lplane = plane * g.na;  // one time level of a field
   const int x = v % g.nx, y = (v / g.nx) % g.ny, z = v / (g.nx * g.ny);
-  const float mu = __ldg(mut + v);
-  const float nv_idx = __ldg(nidx + v);
-  float acc = 0.0f;
-#pragma unroll 1
-  for (int d = 0; d < g.na; ++d) {
-    const float qpre = __ldg(Qb + static_cast<size_t>(d) * plane + v);
-    if (qpre == 0.0f) continue;
+  const float mu = in ? __ldg(mut + v) : 0.0f;
+  const float nv_idx = in ? __ldg(nidx + v) : 1.0f;
+
+  struct Sample {
+    float q, f, i0, i1, s0, s1;      // Qbar; time weight; I and S of the upwind sample at both levels
+    float ib0, ib1, sb0, sb1;        // its adjoint entries
+    size_t o0, o1;                   // their places
+    int kind, L0;                    // 0 upwind sample, 1 inflow face, 2 side face, 3 nothing
+  };
+  const auto gather = [&](int d, Sample& s) {
+    s.kind = 3;
+    if (!in || d >= g.na) return;
+    s.q = __ldg(Qb + static_cast<size_t>(d) * plane + v);
     const DirInfo& di = dir_s[d];
     const int dom = di.dom, sgn = di.sgn, a0 = di.a0, a1 = di.a1;
     const int nd = pick(dom, g.nx, g.ny, g.nz);
@@ -389,65 +399,94 @@ __global__ void __launch_bounds__(256) adj_push_kernel(GridParams g, const DirIn
     int qd = pd - sgn;
     int q0 = p0 - offs[(static_cast<size_t>(d) * 2 + 0) * g.nmax + kp];
     int q1 = p1 - offs[(static_cast<size_t>(d) * 2 + 1) * g.nmax + kp];
-    int kind = 0;
+    s.kind = 0;
     if (g.periodic) {
       qd = (qd + nd) % nd;
       q0 = (q0 + n0) % n0;
       q1 = (q1 + n1) % n1;
     } else if (kp == 0) {
-      kind = 1;
+      s.kind = 1;
     } else if (q0 < 0 || q0 >= n0 || q1 < 0 || q1 >= n1) {
-      kind = 2;
+      s.kind = 2;
     }
     int m;
-    float f;
-    retarded_delay(di.dcoef, di.dcoef_lo, nv_idx, m, f);
-    const int L0 = n - m, L1 = n - m - 1;
+    retarded_delay(di.dcoef, di.dcoef_lo, nv_idx, m, s.f);
+    s.L0 = n - m;
+    const int L1 = s.L0 - 1;
+    s.i0 = s.i1 = s.s0 = s.s1 = s.ib0 = s.ib1 = s.sb0 = s.sb1 = 0.0f;
+    if (s.kind != 0) return;
+    const int sd = dom == 0 ? 1 : (dom == 1 ? g.nx : g.nx * g.ny);
+    const int s0 = a0 == 0 ? 1 : (a0 == 1 ? g.nx : g.nx * g.ny);
+    const int s1 = a1 == 0 ? 1 : (a1 == 1 ? g.nx : g.nx * g.ny);
+    const size_t du = static_cast<size_t>(d) * plane + static_cast<size_t>(qd) * sd + static_cast<size_t>(q0) * s0 +
+                      static_cast<size_t>(q1) * s1;
+    if (s.L0 >= g.hist_from) {
+      const size_t o = static_cast<size_t>(s.L0 - lev_base) * lplane + du;
+      s.i0 = __ldg(stI + o);
+      s.s0 = __ldg(stS + o);
+    }
+    if (L1 >= g.hist_from) {
+      const size_t o = static_cast<size_t>(L1 - lev_base) * lplane + du;
+      s.i1 = __ldg(stI + o);
+      s.s1 = __ldg(stS + o);
+    }
+    s.o0 = static_cast<size_t>(ring_slot(s.L0)) * lplane + du;
+    s.o1 = static_cast<size_t>(ring_slot(L1)) * lplane + du;
+    if (s.L0 >= 0) {  // levels before 0 are inputs, not parameters
+      s.ib0 = IbR[s.o0];
+      s.sb0 = SbR[s.o0];
+    }
+    if (L1 >= 0) {
+      s.ib1 = IbR[s.o1];
+      s.sb1 = SbR[s.o1];
+    }
+  };
+  float acc = 0.0f;
+  const auto push = [&](int d, const Sample& s) {
+    if (s.kind == 3 || s.q == 0.0f) return;
+    const DirInfo& di = dir_s[d];
+    const float f = s.f;
+    const int L0 = s.L0, L1 = s.L0 - 1;
     const float xo = mu * di.ds;
     float T = expf(-xo), b0 = ray_b0(xo, T), b0l;
     if (g.fine) ray_weights_fine(mu, di.ds, di.ds_lo, T, b0, b0l);
     const float db0 = ray_db0(xo, T);
     float Iup = 0.0f, Sup = 0.0f;
-    if (kind == 0) {
-      const int sd = dom == 0 ? 1 : (dom == 1 ? g.nx : g.nx * g.ny);
-      const int s0 = a0 == 0 ? 1 : (a0 == 1 ? g.nx : g.nx * g.ny);
-      const int s1 = a1 == 0 ? 1 : (a1 == 1 ? g.nx : g.nx * g.ny);
-      const size_t u = static_cast<size_t>(qd) * sd + static_cast<size_t>(q0) * s0 +
-                       static_cast<size_t>(q1) * s1;
-      const size_t du = static_cast<size_t>(d) * plane + u;
-      float i0 = 0.0f, i1 = 0.0f, s0v = 0.0f, s1v = 0.0f;
-      if (L0 >= g.hist_from) {
-        const size_t o = static_cast<size_t>(L0 - lev_base) * lplane + du;
-        i0 = __ldg(stI + o);
-        s0v = __ldg(stS + o);
-      }
-      if (L1 >= g.hist_from) {
-        const size_t o = static_cast<size_t>(L1 - lev_base) * lplane + du;
-        i1 = __ldg(stI + o);
-        s1v = __ldg(stS + o);
-      }
-      Iup = (1.0f - f) * i0 + f * i1;
-      Sup = (1.0f - f) * s0v + f * s1v;
-      // push to the upwind sample (levels before 0 are inputs, not parameters)
-      const float tq = T * qpre, bq = b0 * qpre;
+    if (s.kind == 0) {
+      Iup = (1.0f - f) * s.i0 + f * s.i1;
+      Sup = (1.0f - f) * s.s0 + f * s.s1;
+      const float tq = T * s.q, bq = b0 * s.q;
       if (L0 >= 0) {
-        const size_t o = static_cast<size_t>(ring_slot(L0)) * lplane + du;
-        IbR[o] = fmaf(1.0f - f, tq, IbR[o]);
-        SbR[o] = fmaf(1.0f - f, bq, SbR[o]);
+        IbR[s.o0] = fmaf(1.0f - f, tq, s.ib0);
+        SbR[s.o0] = fmaf(1.0f - f, bq, s.sb0);
       }
       if (L1 >= 0) {
-        const size_t o = static_cast<size_t>(ring_slot(L1)) * lplane + du;
-        IbR[o] = fmaf(f, tq, IbR[o]);
-        SbR[o] = fmaf(f, bq, SbR[o]);
+        IbR[s.o1] = fmaf(f, tq, s.ib1);
+        SbR[s.o1] = fmaf(f, bq, s.sb1);
       }
-    } else if (kind == 1 && v == g.src_voxel && di.src_amp != 0.0f) {
+    } else if (s.kind == 1 && v == g.src_voxel && di.src_amp != 0.0f) {
       const float on0 = (L0 >= 0 && L0 < g.pulse_steps) ? 1.0f : 0.0f;
       const float on1 = (L1 >= 0 && L1 < g.pulse_steps) ? 1.0f : 0.0f;
       Iup = di.src_amp * ((1.0f - f) * on0 + f * on1);
     }
-    acc = fmaf(di.ds * qpre, fmaf(-T, Iup, db0 * Sup), acc);
+    acc = fmaf(di.ds * s.q, fmaf(-T, Iup, db0 * Sup), acc);
+  };
+#pragma unroll 1
+  for (int d = warp; d < g.na; d += 2 * kPushWarps) {
+    Sample a, b;
+    gather(d, a);
+    gather(d + kPushWarps, b);
+    push(d, a);
+    push(d + kPushWarps, b);
   }
-  gmut[v] += static_cast<double>(acc);
+  acc_s[warp][lane] = acc;
+  __syncthreads();
+  if (warp == 0 && in) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kPushWarps; ++w) s += static_cast<double>(acc_s[w][lane]);
+    gmut[v] += s;
+  }
 }
 
 __global__ void adj_finish_kernel(int nv, const float* __restrict__ mut, const float* __restrict__ eps,
@@ -501,9 +540,8 @@ cudaError_t launch_adj_push(const GridParams& g, const DirInfo* dirs, const int8
                             const float* stI, const float* stS, int lev_base, int n,
                             const float* mut, const float* nidx, const float* Qb, float* IbR,
                             float* SbR, double* gmut, cudaStream_t st) {
-  const int blocks = (g.nv + 255) / 256;
-  adj_push_kernel<<<blocks, 256, g.na * sizeof(DirInfo), st>>>(g, dirs, offs, stI, stS, lev_base, n,
-                                                               mut, nidx, Qb, IbR, SbR, gmut);
+  adj_push_kernel<<<(g.nv + 31) / 32, 32 * kPushWarps, g.na * sizeof(DirInfo), st>>>(
+      g, dirs, offs, stI, stS, lev_base, n, mut, nidx, Qb, IbR, SbR, gmut);
   return cudaGetLastError();
 }
 
