@@ -79,130 +79,163 @@ __global__ void noalloc_prepass(int na, int nvox, const float* __restrict__ b1, 
   if ((threadIdx.x & 31) == 0) atomicMax(&sc->smax, __float_as_uint(sm));
 }
 
-// Split of the caller's P on the device (the host form is scatter_split_image): one CTA.
-// The spectrum of P without the constant vector is estimated by power iteration (the
-// context path knows it from g): it sets the interval of the Chebyshev weights only, and an
-// eigenvalue above the estimate is still damped, as in the plain iteration.
+// Split of the caller's P on the device (the host form is scatter_split_image): blocks
+// 1 .. NA / 8 build eight rows each (every block takes the largest entry and row weight for
+// itself: 147 KB from L2), block 0 estimates the spectrum of P without the constant vector
+// by power iteration, its matrix in registers (the context path knows the spectrum from g).
+// The estimate sets the interval of the Chebyshev weights only; an eigenvalue above it is
+// still damped, as in the plain iteration.  One block doing all of it in turn took 520 us,
+// a third of a 110592-voxel call.
 template <int NA>
 __global__ void __launch_bounds__(1024) noalloc_split_prep(const float* __restrict__ P, NoAllocScratch* sc) {
-  __shared__ float x_s[NA], y_s[NA];
-  __shared__ float red_s[32], red2_s[32];
-  __shared__ float pm_s, rm_s;
-  constexpr int kRows = 32;
+  constexpr int kW = 32;                    // warps
+  constexpr int kC = (NA + 31) / 32;        // columns per lane
+  constexpr int kR = (NA + kW - 1) / kW;    // rows per warp
+  __shared__ float x_s[kC * 32], y_s[kC * 32];
+  __shared__ float red_s[kW], red2_s[kW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // largest off-diagonal entry and row weight
-  float pm = 0.0f, rm = 0.0f;
-  for (int i = warp; i < NA; i += kRows) {
-    float s = 0.0f;
-    for (int j = lane; j < NA; j += 32)
-      if (j != i) {
-        const float p = fabsf(P[static_cast<size_t>(j) * NA + i]);
-        pm = fmaxf(pm, p);
-        s += p;
-      }
+  // every block: the whole matrix, row i = warp + 32 r, column j = lane + 32 c, with the
+  // indices exchanged (P is symmetric; a column of the caller's array is a row here)
+  float p[kR][kC];
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    rm = fmaxf(rm, s);
-  }
+  for (int r = 0; r < kR; ++r)
 #pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
-  if (lane == 0) {
-    red_s[warp] = pm;
-    red2_s[warp] = rm;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < kRows; ++w) {
-      pm = fmaxf(pm, red_s[w]);
-      rm = fmaxf(rm, red2_s[w]);
+    for (int c = 0; c < kC; ++c) {
+      const int i = warp + kW * r, j = lane + 32 * c;
+      p[r][c] = (i < NA && j < NA) ? __ldg(P + static_cast<size_t>(i) * NA + j) : 0.0f;
     }
-    pm_s = pm;
-    rm_s = rm;
-  }
-  __syncthreads();
-  int t = 0;
-  while (t < 20 && ldexpf(pm_s, t + 1) <= 2046.0f && ldexpf(rm_s, t + 1) + NA / 2 <= 16128.0f) ++t;
-  const float whole = floorf(ldexpf(pm_s, t));
-  const float unit_f = whole >= 1.0f ? static_cast<float>(static_cast<double>(pm_s) / whole) : ldexpf(1.0f, -t);
-  const double unit = unit_f;
-  for (int i = warp; i < NA; i += kRows) {
-    double sh = 0.0, sl = 0.0;
-    for (int j = lane; j < NA; j += 32) {
-      double h = 0.0, l = 0.0;
-      if (j != i) {
-        const double u = static_cast<double>(P[static_cast<size_t>(j) * NA + i]) / unit;
-        h = rint(u);
-        l = rint((u - h) * 4096.0) / 4096.0;
-      }
-      sh += h;
-      sl += l;
-      const int k = j >> 6, ch = (j & 63) >> 3;
-      const int in_row = ((ch ^ (i & 7)) << 3) + (j & 7);
-      const int prow = NA >= 192 ? (k * (NA / 96) + i / 96) * 96 + i % 96 : k * NA + i;
-      sc->ph[(k * NA + i) * 64 + in_row] = __half_as_ushort(__float2half_rn(static_cast<float>(h)));
-      sc->pl[prow * 64 + in_row] = __half_as_ushort(__float2half_rn(static_cast<float>(l)));
+  if (blockIdx.x > 0) {
+    float pm = 0.0f, rm = 0.0f;
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      float s = 0.0f;
+#pragma unroll
+      for (int c = 0; c < kC; ++c)
+        if (lane + 32 * c != warp + kW * r) {
+          pm = fmaxf(pm, fabsf(p[r][c]));
+          s += fabsf(p[r][c]);
+        }
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      rm = fmaxf(rm, s);
     }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
+    if (lane == 0) {
+      red_s[warp] = pm;
+      red2_s[warp] = rm;
+    }
+    __syncthreads();
+    pm = red_s[lane];
+    rm = red2_s[lane];
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) {
-      sh += __shfl_xor_sync(0xffffffffu, sh, o);
-      sl += __shfl_xor_sync(0xffffffffu, sl, o);
+      pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
+      rm = fmaxf(rm, __shfl_xor_sync(0xffffffffu, rm, o));
     }
-    if (lane == 0) {
-      const double d = 1.0 - (sh + sl) * unit;
-      sc->diag[i] = static_cast<float>(d);
-      sc->diag[NA + i] = static_cast<float>(d - static_cast<double>(static_cast<float>(d)));
-      sc->diag[2 * NA + i] = static_cast<float>(1.0 - sh * unit);
+    int t = 0;
+    while (t < 20 && ldexpf(pm, t + 1) <= 2046.0f && ldexpf(rm, t + 1) + NA / 2 <= 16128.0f) ++t;
+    const float whole = floorf(ldexpf(pm, t));
+    const float unit = whole >= 1.0f ? pm / whole : ldexpf(1.0f, -t);
+    const float inv = 1.0f / unit;
+    if (warp < 8) {
+      const int i = (blockIdx.x - 1) * 8 + warp;
+      float sh = 0.0f, sl = 0.0f;  // sums of whole numbers and of multiples of 2^-12: exact
+#pragma unroll
+      for (int c = 0; c < kC; ++c) {
+        const int j = lane + 32 * c;
+        if (j >= NA) break;
+        const float u = j != i ? __ldg(P + static_cast<size_t>(j) * NA + i) : 0.0f;
+        const float h = rintf(u * inv);
+        const float l = rintf(fmaf(-h, unit, u) * inv * 4096.0f) * (1.0f / 4096.0f);
+        sh += h;
+        sl += l;
+        const int k = j >> 6, ch = (j & 63) >> 3;
+        const int in_row = ((ch ^ (i & 7)) << 3) + (j & 7);
+        const int prow = NA >= 192 ? (k * (NA / 96) + i / 96) * 96 + i % 96 : k * NA + i;
+        sc->ph[(k * NA + i) * 64 + in_row] = __half_as_ushort(__float2half_rn(h));
+        sc->pl[prow * 64 + in_row] = __half_as_ushort(__float2half_rn(l));
+      }
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) {
+        sh += __shfl_xor_sync(0xffffffffu, sh, o);
+        sl += __shfl_xor_sync(0xffffffffu, sl, o);
+      }
+      if (lane == 0) {
+        const double d = 1.0 - (static_cast<double>(sh) + sl) * unit;
+        sc->diag[i] = static_cast<float>(d);
+        sc->diag[NA + i] = static_cast<float>(d - static_cast<double>(static_cast<float>(d)));
+        sc->diag[2 * NA + i] = static_cast<float>(1.0 - static_cast<double>(sh) * unit);
+      }
     }
+    if (blockIdx.x == 1 && tid == 0) sc->dyn[0] = unit;
+    return;
   }
-  // power iterations: the largest |eigenvalue| besides the constant vector's, then the
-  // largest of (that - eigenvalue), which tells how far the spectrum reaches below zero
+  // block 0: the largest |eigenvalue| besides the constant vector's, then the largest of
+  // (that - eigenvalue), which tells how far the spectrum reaches below zero
   float lam = 0.0f, low = 0.0f;
 #pragma unroll 1
   for (int stage = 0; stage < 2; ++stage) {
-    for (int i = tid; i < NA; i += blockDim.x) {
-      unsigned h = (i + 1) * 2654435761u;
+    if (tid < kC * 32) {
+      unsigned h = (tid + 1) * 2654435761u;
       h ^= h >> 15;
-      x_s[i] = static_cast<float>(h & 0xffffu) / 65536.0f - 0.5f;
+      x_s[tid] = tid < NA ? static_cast<float>(h & 0xffffu) / 65536.0f - 0.5f : 0.0f;
     }
     __syncthreads();
-    float norm0 = 1.0f;
+    float norm = 0.0f;
 #pragma unroll 1
-    for (int it = 0; it < (stage == 0 ? 48 : 24); ++it) {
-      for (int i = warp; i < NA; i += kRows) {
+    for (int it = 0; it < (stage == 0 ? 40 : 24); ++it) {
+      float xv[kC];
+#pragma unroll
+      for (int c = 0; c < kC; ++c) xv[c] = x_s[lane + 32 * c];
+#pragma unroll
+      for (int r = 0; r < kR; ++r) {
         float s = 0.0f;
-        for (int j = lane; j < NA; j += 32) s = fmaf(P[static_cast<size_t>(i) * NA + j], x_s[j], s);
+#pragma unroll
+        for (int c = 0; c < kC; ++c) s = fmaf(p[r][c], xv[c], s);
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) y_s[i] = stage == 0 ? s : fmaf(lam, x_s[i], -s);
+        const int i = warp + kW * r;
+        if (lane == 0 && i < NA) y_s[i] = stage == 0 ? s : fmaf(lam, x_s[i], -s);
       }
       __syncthreads();
-      float m = 0.0f;  // every warp the same sums, in the same order
-      for (int j = lane; j < NA; j += 32) m += y_s[j];
+      if (warp == 0) {  // without the mean, to unit length
+        float yv[kC], m = 0.0f, q = 0.0f;
 #pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-      m /= NA;
-      float q = 0.0f;
-      for (int j = lane; j < NA; j += 32) q = fmaf(y_s[j] - m, y_s[j] - m, q);
+        for (int c = 0; c < kC; ++c) {
+          yv[c] = lane + 32 * c < NA ? y_s[lane + 32 * c] : 0.0f;
+          m += yv[c];
+        }
 #pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-      norm0 = sqrtf(q);
-      const float inv = norm0 > 1e-30f ? 1.0f / norm0 : 0.0f;
-      for (int j = tid; j < NA; j += blockDim.x) x_s[j] = (y_s[j] - m) * inv;
+        for (int o = 16; o >= 1; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+        m /= NA;
+#pragma unroll
+        for (int c = 0; c < kC; ++c) {
+          yv[c] = lane + 32 * c < NA ? yv[c] - m : 0.0f;
+          q = fmaf(yv[c], yv[c], q);
+        }
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        norm = sqrtf(q);
+        const float iv = norm > 1e-30f ? 1.0f / norm : 0.0f;
+#pragma unroll
+        for (int c = 0; c < kC; ++c) x_s[lane + 32 * c] = yv[c] * iv;
+        if (lane == 0) red_s[0] = norm;
+      }
       __syncthreads();
     }
+    norm = red_s[0];
     if (stage == 0)
-      lam = norm0;
+      lam = norm;
     else
-      low = lam - norm0;
+      low = lam - norm;
+    __syncthreads();
   }
   if (tid == 0) {
-    const float l = fminf(fmaxf(lam, 0.0f) * 1.01f + 0.01f, 0.5f * (fminf(lam, 0.999f) + 1.0f));
-    sc->dyn[0] = unit_f;
-    sc->dyn[1] = l;
+    sc->dyn[1] = fminf(fmaxf(lam, 0.0f) * 1.01f + 0.01f, 0.5f * (fminf(lam, 0.999f) + 1.0f));
     sc->dyn[2] = low < -0.02f ? -1.0f : 0.0f;
     const int root[8] = {15, 1, 9, 7, 13, 3, 11, 5};  // as scatter_split_image orders them
-    for (int k = 0; k < 8; ++k) sc->cw[k] = cospif(root[k] / 16.0f);
-    for (int k = 8; k < 64; ++k) sc->cw[k] = 0.0f;
+    for (int k = 0; k < 64; ++k) sc->cw[k] = k < 8 ? cospif(root[k] / 16.0f) : 0.0f;
   }
 }
 
@@ -405,9 +438,9 @@ extern "C" int trinity_source_iteration_noalloc(int na, int nvox, const float* P
   } else {
     if (!scatter_split_supported(na, 0)) return TRINITY_E_CUDA;
     if (na == 48)
-      noalloc_split_prep<48><<<1, 1024, 0, st>>>(P, sc);
+      noalloc_split_prep<48><<<1 + 48 / 8, 1024, 0, st>>>(P, sc);
     else
-      noalloc_split_prep<192><<<1, 1024, 0, st>>>(P, sc);
+      noalloc_split_prep<192><<<1 + 192 / 8, 1024, 0, st>>>(P, sc);
     SplitTables sp{};
     sp.ph = reinterpret_cast<const uint8_t*>(sc->ph);
     sp.pl = reinterpret_cast<const uint8_t*>(sc->pl);
