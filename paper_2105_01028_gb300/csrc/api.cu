@@ -65,6 +65,7 @@ struct trinity_ctx {
   int* d_nonconv = nullptr;
   int* d_error = nullptr;
   int* d_tile_ctr = nullptr;
+  int* d_done = nullptr;
   float* d_rcorr = nullptr;
   uint8_t* d_cls = nullptr;
   float* d_cls_ds = nullptr;
@@ -76,7 +77,7 @@ struct trinity_ctx {
   double* d_escaped = nullptr;
   double* d_absorbed = nullptr;
   double* d_residual = nullptr;
-  double* d_balance = nullptr;   // [1] running photon balance (see advance_kernel)
+  double* d_balance = nullptr;   // [1] running photon balance (see tally_kernel)
   double energy_init = 0.0;      // energy of the state before step 0
   int* d_refl = nullptr;         // [na][8] reflected directions (mirror faces)
   int* d_bins = nullptr;
@@ -257,6 +258,7 @@ RunState run_state(trinity_ctx* c) {
   rs.bins = c->d_bins;
   rs.error = c->d_error;
   rs.tile_ctr = c->d_tile_ctr;
+  rs.done = c->d_done;
   return rs;
 }
 
@@ -645,7 +647,6 @@ int enqueue_finish(trinity_ctx* ctx, const RunState& rs, double* det) {
                      rs, ctx->stream));
   CK(launch_tally(g, ctx->d_dirs, ctx->I, ctx->d_det_vox, ctx->d_det_dir, ctx->d_det_w,
                   ctx->d_det_id, ctx->n_det_entries, det, ctx->nbins, rs, ctx->stream));
-  CK(launch_advance(ctx->g, rs, ctx->stream));
   return TRINITY_OK;
 }
 
@@ -911,6 +912,7 @@ int trinity_create_grid(const trinity_grid_desc* desc, void* cuda_stream, trinit
       dalloc(&ctx->d_offs, ctx->lat.off.size()) != cudaSuccess || dalloc(&ctx->d_step, 1) != cudaSuccess ||
       dalloc(&ctx->d_smax, 2) != cudaSuccess || dalloc(&ctx->d_nonconv, 1) != cudaSuccess ||
       dalloc(&ctx->d_error, 1) != cudaSuccess || dalloc(&ctx->d_tile_ctr, 2) != cudaSuccess ||
+      dalloc(&ctx->d_done, 1) != cudaSuccess ||
       dalloc(&ctx->d_balance, 1) != cudaSuccess || (g.mirror && dalloc(&ctx->d_refl, 8 * na) != cudaSuccess) ||
       dalloc(&ctx->d_rcorr, na_s) != cudaSuccess || dalloc(&ctx->d_rcorr32, na_s) != cudaSuccess ||
       dalloc(&ctx->d_cls, na_s) != cudaSuccess || dalloc(&ctx->d_cls_ds, 16 * ctx->nch) != cudaSuccess ||
@@ -1816,7 +1818,7 @@ int trinity_kernels_per_step(const trinity_ctx* ctx, int* n) {
   else
     k = 1 + 1 + 1;  // sweep, scatter, tally
   if (ctx->n_iface > 0) k += ctx->two_level ? 2 : 1;  // interface split (and re-coarsening)
-  *n = k + 1;  // the step counter
+  *n = k;
   return TRINITY_OK;
 }
 
@@ -1858,6 +1860,7 @@ int trinity_reset(trinity_ctx* ctx) {
   CK(cudaMemsetAsync(ctx->d_nonconv, 0, sizeof(int), st));
   CK(cudaMemsetAsync(ctx->d_error, 0, sizeof(int), st));
   CK(cudaMemsetAsync(ctx->d_tile_ctr, 0, 2 * sizeof(int), st));
+  CK(cudaMemsetAsync(ctx->d_done, 0, sizeof(int), st));
   CK(cudaMemsetAsync(ctx->d_balance, 0, sizeof(double), st));
   if (ctx->capacity > 0) {
     const size_t c = static_cast<size_t>(ctx->capacity);
@@ -1916,7 +1919,7 @@ void trinity_destroy(trinity_ctx* ctx) {
                   ctx->d_det_vox, ctx->d_det_dir,  ctx->d_det_id,    ctx->d_det_w,   ctx->d_det,
                   ctx->d_step,    ctx->d_smax,     ctx->d_nonconv,   ctx->d_error,   ctx->d_iters_max,
                   ctx->d_iters_sum, ctx->d_energy, ctx->d_escaped,   ctx->d_bins, ctx->d_tile_iters,
-                  ctx->d_tile_ctr, ctx->d_rcorr,   ctx->d_cls,       ctx->d_cls_ds,   ctx->d_split,
+                  ctx->d_tile_ctr, ctx->d_done, ctx->d_rcorr,   ctx->d_cls,       ctx->d_cls_ds,   ctx->d_split,
                   ctx->d_rcorr32, ctx->d_absorbed, ctx->d_residual,  ctx->d_balance, ctx->d_refl};
   for (void* p : bufs)
     if (p) cudaFree(p);

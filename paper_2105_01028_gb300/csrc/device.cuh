@@ -55,6 +55,7 @@ struct RunState {
   int* nonconv;                  // count of voxel-steps that hit max_iters
   int* bins;                     // [capacity] detector bin of each step (-1: none)
   int* error;                    // device error word (0 = ok)
+  int* done;                     // blocks of the step's last kernel that have finished
   int* tile_ctr;                 // [2] work counters of the persistent kernels (ping-pong)
   unsigned long long* tile_iters; // [capacity] iterations executed x voxels per tile, summed
                                   // (tensor-core kernel; null: not counted)
@@ -192,7 +193,6 @@ cudaError_t launch_tally(const GridParams& g, const DirInfo* dirs, const float* 
                          const int* det_vox, const int* det_dir, const float* det_w,
                          const int* det_id, int n_det_entries, double* det, int nbins,
                          RunState rs, cudaStream_t st);
-cudaError_t launch_advance(const GridParams& g, RunState rs, cudaStream_t st);
 
 // The TMA-staged one-level sweep (sweep_tma.cu): uniform refractive index, vacuum faces,
 // nx a multiple of 4 and nx + 8 <= 256.  Tensor maps of the I and S rings, one per
