@@ -35,6 +35,7 @@ struct trinity_ctx {
   // detectors
   struct Det {
     int face;
+    double half_angle;
     std::vector<int> vox;
     std::vector<double> weight;  // per direction, alpha * Omega_cap * cos_out
   };
@@ -1235,7 +1236,11 @@ int trinity_add_detector(trinity_ctx* ctx, int face, double u_mm, double v_mm, d
   if (face < 0 || face > 5 || !(radius_mm > 0.0)) return fail(ctx, TRINITY_E_INVALID, "bad face or radius");
   trinity_ctx::Det det;
   det.face = face;
-  try {
+  det.half_angle = half_angle_deg;
+  // detectors of one face and acceptance share their weights
+  for (const trinity_ctx::Det& other : ctx->dets)
+    if (other.face == face && other.half_angle == half_angle_deg) det.weight = other.weight;
+  if (det.weight.empty()) try {
     const std::vector<double> alpha = cone_weights(ctx->dirs, face, half_angle_deg, false);
     const double cap = 2.0 * 3.14159265358979323846 * (1.0 - std::cos(half_angle_deg * 3.14159265358979323846 / 180.0));
     const int ax = face / 2;
