@@ -126,6 +126,7 @@ struct trinity_ctx {
   float* d_xmua = nullptr;     // [classes] mu_a of each class (absorbed-energy tally)
   uint8_t* d_xcls = nullptr;   // [nv] optics class of each voxel
   std::vector<float> h_P32, h_rc32, h_mut, h_eps;  // host copies the operators are built from
+  std::vector<float> h_mut_lo;                     // mu_a + mu_s - h_mut (FP32 rounding of mu_t)
 
   // index interfaces (Eqs. 13-14)
   bool fresnel = false;
@@ -334,6 +335,20 @@ int ensure_capacity(trinity_ctx* ctx, int need) {
   return TRINITY_OK;
 }
 
+// Upload the direction table.  Where the FP32 iteration takes fine sweep weights, the source
+// amplitudes carry what rounding mu_t of the source voxel to FP32 changes in the light that
+// crosses it: exp(-x) at 15 mean free paths turns half a unit of the last place into 8e-7 of
+// every curve.
+int upload_dirs(trinity_ctx* ctx) {
+  std::vector<DirInfo> h = ctx->hdirs;
+  if (ctx->g.fine && ctx->g.src_voxel >= 0)
+    for (int d = 0; d < ctx->g.na; ++d)
+      h[d].src_amp = static_cast<float>(h[d].src_amp * std::exp(-static_cast<double>(ctx->h_mut_lo[ctx->g.src_voxel]) *
+                                                                 ctx->lat.ds[d]));
+  CK(cudaMemcpy(ctx->d_dirs, h.data(), h.size() * sizeof(DirInfo), cudaMemcpyHostToDevice));
+  return TRINITY_OK;
+}
+
 // Freeze the inputs: upload detector entries and bins before the first step.
 int lock_inputs(trinity_ctx* ctx) {
   if (ctx->locked) return TRINITY_OK;
@@ -364,10 +379,12 @@ int lock_inputs(trinity_ctx* ctx) {
   const size_t ndet = ctx->dets.size() * static_cast<size_t>(std::max(ctx->nbins, 1));
   CK(dalloc(&ctx->d_det, ndet));
   CK(cudaMemset(ctx->d_det, 0, ndet * sizeof(double)));
-  CK(cudaMemcpy(ctx->d_dirs, ctx->hdirs.data(), ctx->hdirs.size() * sizeof(DirInfo),
-                cudaMemcpyHostToDevice));
   // the exact solve's operators hold b1 in FP64, the BF16 iteration is coarser than these weights
   ctx->g.fine = ctx->g_s.fine = ctx->desc.precision == TRINITY_FP32 && !ctx->exact ? 1 : 0;
+  {
+    const int rc = upload_dirs(ctx);
+    if (rc != TRINITY_OK) return rc;
+  }
   // the photon balance starts from the energy of the state held before step 0
   ctx->energy_init = 0.0;
   if (ctx->has_init) {
@@ -1043,7 +1060,7 @@ int trinity_set_optics(trinity_ctx* ctx, const float* mua, const float* mus, con
     dsmin = std::min(dsmin, ds);
     dsmax = std::max(dsmax, ds);
   }
-  std::vector<float> mt(nv), al(nv);  // al: eps = mu_a / mu_t (1 where mu_t = 0)
+  std::vector<float> mt(nv), al(nv), ml(nv);  // al: eps = mu_a / mu_t (1 where mu_t = 0)
   for (size_t v = 0; v < nv; ++v) {
     if (!(a[v] >= 0.0f) || !(s[v] >= 0.0f) || !std::isfinite(a[v]) || !std::isfinite(s[v]) ||
         !(r[v] >= 1.0f) || !std::isfinite(r[v]))
@@ -1053,6 +1070,7 @@ int trinity_set_optics(trinity_ctx* ctx, const float* mua, const float* mus, con
     mt[v] = a[v] + s[v];
     const double t64 = static_cast<double>(a[v]) + static_cast<double>(s[v]);
     al[v] = t64 > 0.0 ? static_cast<float>(static_cast<double>(a[v]) / t64) : 1.0f;
+    ml[v] = static_cast<float>(t64 - static_cast<double>(mt[v]));
   }
   const double dlo = dsmin * nmin / (kC0 * ctx->dt), dhi = dsmax * nmax / (kC0 * ctx->dt);
   if (dlo < 1.0 || dhi >= kRing - 1)
@@ -1118,6 +1136,7 @@ int trinity_set_optics(trinity_ctx* ctx, const float* mua, const float* mus, con
   ctx->h_rc32 = rc;
   ctx->h_mut = mt;
   ctx->h_eps = al;
+  ctx->h_mut_lo = ml;
   {
     const int rc3 = build_exact(ctx);
     if (rc3 != TRINITY_OK) return rc3;
@@ -1126,7 +1145,10 @@ int trinity_set_optics(trinity_ctx* ctx, const float* mua, const float* mus, con
     const int rc2 = build_interface_table(ctx);
     if (rc2 != TRINITY_OK) return rc2;
   }
-  if (ctx->locked) return trinity_reset(ctx);
+  if (ctx->locked) {
+    const int rc5 = upload_dirs(ctx);
+    return rc5 != TRINITY_OK ? rc5 : trinity_reset(ctx);
+  }
   return TRINITY_OK;
 }
 
