@@ -257,7 +257,7 @@ int trinity_read_field(trinity_ctx* ctx, int what, int back, void* out, size_t b
 int trinity_steps_done(const trinity_ctx* ctx, int* n);
 
 /* Kernel launches one time step issues with the context's current inputs (sweep or
- * sweeps, interface split, source iteration, tallies with the step counter). */
+ * sweeps, interface split, source iteration, tallies, step counter). */
 int trinity_kernels_per_step(const trinity_ctx* ctx, int* n);
 
 /* Form of the ray sweep a step runs: 0 plain loads (one kernel), 1 upwind planes staged

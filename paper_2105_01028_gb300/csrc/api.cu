@@ -66,7 +66,6 @@ struct trinity_ctx {
   int* d_nonconv = nullptr;
   int* d_error = nullptr;
   int* d_tile_ctr = nullptr;
-  int* d_done = nullptr;
   float* d_rcorr = nullptr;
   uint8_t* d_cls = nullptr;
   float* d_cls_ds = nullptr;
@@ -78,7 +77,7 @@ struct trinity_ctx {
   double* d_escaped = nullptr;
   double* d_absorbed = nullptr;
   double* d_residual = nullptr;
-  double* d_balance = nullptr;   // [1] running photon balance (see tally_kernel)
+  double* d_balance = nullptr;   // [1] running photon balance (see advance_kernel)
   double energy_init = 0.0;      // energy of the state before step 0
   int* d_refl = nullptr;         // [na][8] reflected directions (mirror faces)
   int* d_bins = nullptr;
@@ -260,7 +259,6 @@ RunState run_state(trinity_ctx* c) {
   rs.bins = c->d_bins;
   rs.error = c->d_error;
   rs.tile_ctr = c->d_tile_ctr;
-  rs.done = c->d_done;
   return rs;
 }
 
@@ -380,7 +378,7 @@ int lock_inputs(trinity_ctx* ctx) {
   CK(dalloc(&ctx->d_det, ndet));
   CK(cudaMemset(ctx->d_det, 0, ndet * sizeof(double)));
   // the exact solve's operators hold b1 in FP64, the BF16 iteration is coarser than these weights
-  ctx->g.fine = ctx->g_s.fine = ctx->desc.precision == TRINITY_FP32 && !ctx->exact ? 1 : 0;
+  ctx->g.fine = ctx->g_s.fine = ctx->split && !ctx->exact ? 1 : 0;
   {
     const int rc = upload_dirs(ctx);
     if (rc != TRINITY_OK) return rc;
@@ -665,6 +663,7 @@ int enqueue_finish(trinity_ctx* ctx, const RunState& rs, double* det) {
                      rs, ctx->stream));
   CK(launch_tally(g, ctx->d_dirs, ctx->I, ctx->d_det_vox, ctx->d_det_dir, ctx->d_det_w,
                   ctx->d_det_id, ctx->n_det_entries, det, ctx->nbins, rs, ctx->stream));
+  CK(launch_advance(ctx->g, rs, ctx->stream));
   return TRINITY_OK;
 }
 
@@ -930,10 +929,9 @@ int trinity_create_grid(const trinity_grid_desc* desc, void* cuda_stream, trinit
       dalloc(&ctx->d_offs, ctx->lat.off.size()) != cudaSuccess || dalloc(&ctx->d_step, 1) != cudaSuccess ||
       dalloc(&ctx->d_smax, 2) != cudaSuccess || dalloc(&ctx->d_nonconv, 1) != cudaSuccess ||
       dalloc(&ctx->d_error, 1) != cudaSuccess || dalloc(&ctx->d_tile_ctr, 2) != cudaSuccess ||
-      dalloc(&ctx->d_done, 1) != cudaSuccess ||
       dalloc(&ctx->d_balance, 1) != cudaSuccess || (g.mirror && dalloc(&ctx->d_refl, 8 * na) != cudaSuccess) ||
       dalloc(&ctx->d_rcorr, na_s) != cudaSuccess || dalloc(&ctx->d_rcorr32, na_s) != cudaSuccess ||
-      dalloc(&ctx->d_cls, na_s) != cudaSuccess || dalloc(&ctx->d_cls_ds, 16 * ctx->nch) != cudaSuccess ||
+      dalloc(&ctx->d_cls, na_s) != cudaSuccess || dalloc(&ctx->d_cls_ds, 32 * ctx->nch) != cudaSuccess ||
       dalloc(&ctx->d_children, children.size()) != cudaSuccess ||
       dalloc(&ctx->d_b1ds, b1ds.size()) != cudaSuccess ||
       (ctx->two_level && (dalloc(&ctx->Qc, na_s * nv) != cudaSuccess ||
@@ -983,13 +981,25 @@ int trinity_create_grid(const trinity_grid_desc* desc, void* cuda_stream, trinit
     // on a two-level grid a class is the list of a coarse direction's children spacings
     const int nch = ctx->nch;
     std::vector<uint8_t> cls(na_s);
-    std::vector<std::vector<float>> cds;
+    std::vector<std::vector<float>> cds, cds_lo;
     for (size_t c = 0; c < na_s; ++c) {
-      std::vector<float> key(b1ds.begin() + c * nch, b1ds.begin() + (c + 1) * nch);
-      std::sort(key.begin(), key.end());
+      std::vector<std::pair<float, float>> pr(nch);  // spacing and its rounding remainder
+      for (int j = 0; j < nch; ++j) {
+        const double ds = ctx->lat.ds[children[c * nch + j]];
+        pr[j] = {b1ds[c * nch + j], static_cast<float>(ds - static_cast<double>(b1ds[c * nch + j]))};
+      }
+      std::sort(pr.begin(), pr.end());
+      std::vector<float> key(nch), lo(nch);
+      for (int j = 0; j < nch; ++j) {
+        key[j] = pr[j].first;
+        lo[j] = pr[j].second;
+      }
       size_t k = 0;
       while (k < cds.size() && cds[k] != key) ++k;
-      if (k == cds.size()) cds.push_back(key);
+      if (k == cds.size()) {
+        cds.push_back(key);
+        cds_lo.push_back(lo);
+      }
       cls[c] = static_cast<uint8_t>(k < 255 ? k : 255);
     }
     ctx->ncls = static_cast<int>(cds.size());
@@ -999,9 +1009,11 @@ int trinity_create_grid(const trinity_grid_desc* desc, void* cuda_stream, trinit
     ctx->split = desc->precision == TRINITY_FP32 && na_s >= 48;
     if (ctx->split && !scatter_split_supported(static_cast<int>(na_s), ctx->ncls))
       return bail(TRINITY_E_UNSUPPORTED);
-    std::vector<float> flat(16 * static_cast<size_t>(nch), 0.0f);
-    for (size_t k = 0; k < cds.size() && k < 16; ++k)
+    std::vector<float> flat(32 * static_cast<size_t>(nch), 0.0f);
+    for (size_t k = 0; k < cds.size() && k < 16; ++k) {
       std::copy(cds[k].begin(), cds[k].end(), flat.begin() + k * nch);
+      std::copy(cds_lo[k].begin(), cds_lo[k].end(), flat.begin() + (16 + k) * nch);
+    }
     if (cudaMemcpy(ctx->d_cls, cls.data(), na_s, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(ctx->d_cls_ds, flat.data(), flat.size() * sizeof(float), cudaMemcpyHostToDevice) !=
             cudaSuccess)
@@ -1845,7 +1857,7 @@ int trinity_kernels_per_step(const trinity_ctx* ctx, int* n) {
   else
     k = 1 + 1 + 1;  // sweep, scatter, tally
   if (ctx->n_iface > 0) k += ctx->two_level ? 2 : 1;  // interface split (and re-coarsening)
-  *n = k;
+  *n = k + 1;  // the step counter
   return TRINITY_OK;
 }
 
@@ -1887,7 +1899,6 @@ int trinity_reset(trinity_ctx* ctx) {
   CK(cudaMemsetAsync(ctx->d_nonconv, 0, sizeof(int), st));
   CK(cudaMemsetAsync(ctx->d_error, 0, sizeof(int), st));
   CK(cudaMemsetAsync(ctx->d_tile_ctr, 0, 2 * sizeof(int), st));
-  CK(cudaMemsetAsync(ctx->d_done, 0, sizeof(int), st));
   CK(cudaMemsetAsync(ctx->d_balance, 0, sizeof(double), st));
   if (ctx->capacity > 0) {
     const size_t c = static_cast<size_t>(ctx->capacity);
@@ -1946,7 +1957,7 @@ void trinity_destroy(trinity_ctx* ctx) {
                   ctx->d_det_vox, ctx->d_det_dir,  ctx->d_det_id,    ctx->d_det_w,   ctx->d_det,
                   ctx->d_step,    ctx->d_smax,     ctx->d_nonconv,   ctx->d_error,   ctx->d_iters_max,
                   ctx->d_iters_sum, ctx->d_energy, ctx->d_escaped,   ctx->d_bins, ctx->d_tile_iters,
-                  ctx->d_tile_ctr, ctx->d_done, ctx->d_rcorr,   ctx->d_cls,       ctx->d_cls_ds,   ctx->d_split,
+                  ctx->d_tile_ctr, ctx->d_rcorr,   ctx->d_cls,       ctx->d_cls_ds,   ctx->d_split,
                   ctx->d_rcorr32, ctx->d_absorbed, ctx->d_residual,  ctx->d_balance, ctx->d_refl};
   for (void* p : bufs)
     if (p) cudaFree(p);

@@ -55,7 +55,6 @@ struct RunState {
   int* nonconv;                  // count of voxel-steps that hit max_iters
   int* bins;                     // [capacity] detector bin of each step (-1: none)
   int* error;                    // device error word (0 = ok)
-  int* done;                     // blocks of the step's last kernel that have finished
   int* tile_ctr;                 // [2] work counters of the persistent kernels (ping-pong)
   unsigned long long* tile_iters; // [capacity] iterations executed x voxels per tile, summed
                                   // (tensor-core kernel; null: not counted)
@@ -65,7 +64,8 @@ struct RunState {
 struct BfTables {
   const float* rcorr;    // [na] 1 - row sum of bf16(P): diagonal correction (FP32)
   const uint8_t* cls;    // [na] class of each direction's sample spacing ds
-  const float* cls_ds;   // [ncls][nch] spacings of each class (b1 = mean of their b1)
+  const float* cls_ds;   // [16][nch] spacings of each class (b1 = mean of their b1), then [16][nch]
+                         // their rounding remainders
   int ncls;              // <= 16
   int nch;               // 1, or the children per coarse direction on a two-level grid
   // TMA descriptors of the I and S rings (4-D: x, y, z, plane; boxes of one 8 x 4 x 4
@@ -155,15 +155,30 @@ __device__ __forceinline__ float ray_b0_over_x(float x, float T) {
   return (1.0f - (1.0f + x) * T) / (x * x);
 }
 
-// Sweep weights T = e^-x and b0 of a segment x = mu ds, as the FP32 source iteration needs
-// them (lo: remainder of b0):
-//  - the rounding error of x = fl(mu fl(ds)) is carried into T to first order (15 mean free
-//    paths multiply it by 15 in the light that crosses the source cell: 1e-6 of every curve);
-//  - for x >= 1 b0 is the complement (1 - b1) - T of the FP32 b1 that the iteration applies
-//    (T < 1 - b1 there, so both differences are exact with their error terms).  With b0 and
-//    b1 rounded on their own T + b0 + b1 is off by up to 3e-8, which the scattering
-//    multiplies by 1 / (1 - a b1) ~ 14 in every segment, always to the same side in a
-//    uniform medium: up to 1.5e-5 of the field after 100 steps at 16^3 voxels, 48 directions.
+// The weights of a segment x = mu ds as the FP32 source iteration and its sweep take them.
+// Rounding errors of the weights are the same in every step and, in a uniform medium, in
+// every cell, so they add up; these forms keep them out of what the scattering amplifies:
+//  - the rounding error e of x = fl(mu fl(ds)) is carried to first order (the light that
+//    crosses the source cell multiplies it by 15 mean free paths: 1e-6 of every curve);
+//  - b1 is held as u = 1 - b1 = (1 - T) / x, whose rounding is a tenth of b1's in thick
+//    cells (a rounding of b1 is multiplied by 1 / (1 - a b1) ~ 14);
+//  - for x >= 1 b0 is u - T as a float and its remainder (T < u there, so the differences
+//    are exact), so that T + b0 + b1 = 1 to 2^-48.  With b0 and b1 rounded on their own the
+//    sum is off by up to 3e-8, amplified in every segment: up to 1.7e-5 of the field after
+//    100 steps at 16^3 voxels and 48 directions.
+__device__ __forceinline__ float ray_u(float x, float e, float T) {
+  if (x < 1.0f) return __fsub_rn(1.0f, ray_b1(x, T));  // (no contraction: every caller the same bits)
+  const float u = (1.0f - T) / x;
+  return fmaf(-u, e / x, u);
+}
+
+__device__ __forceinline__ float ray_u_fine(float mu, float ds, float ds_lo) {
+  const float x = mu * ds;
+  const float e = fmaf(mu, ds_lo, fmaf(mu, ds, -x));
+  const float T0 = expf(-x);
+  return ray_u(x, e, fmaf(-e, T0, T0));
+}
+
 __device__ __forceinline__ void ray_weights_fine(float mu, float ds, float ds_lo, float& T, float& b0, float& lo) {
   const float x = mu * ds;
   const float e = fmaf(mu, ds_lo, fmaf(mu, ds, -x));
@@ -171,12 +186,11 @@ __device__ __forceinline__ void ray_weights_fine(float mu, float ds, float ds_lo
   T = fmaf(-e, T0, T0);
   lo = 0.0f;
   if (x < 1.0f) {
-    b0 = ray_b0(x, T0);
+    b0 = ray_b0(x, T);
   } else {
-    const float b1 = ray_b1(x, T0);
-    const float h = 1.0f - b1;
-    b0 = h - T;
-    lo = ((1.0f - h) - b1) + ((h - b0) - T);
+    const float u = ray_u(x, e, T);
+    b0 = u - T;
+    lo = (u - b0) - T;
   }
 }
 
@@ -206,6 +220,7 @@ cudaError_t make_sweep_maps(const GridParams& g, float* Iring, float* Sring, Swe
 cudaError_t launch_sweep_tma(const GridParams& g, const DirInfo* dirs, const int* const dlist[3],
                              const int ndir[3], const int8_t* offs, const int8_t* hsh, const SweepMaps& maps,
                              const float* mut, float* Q, RunState rs, const cudaStream_t st[3]);
+cudaError_t launch_advance(const GridParams& g, RunState rs, cudaStream_t st);
 cudaError_t launch_energy_density(const GridParams& g, const float* I, const float* nidx, float scale, float* u,
                                   cudaStream_t st);
 cudaError_t launch_interface(int nvox, int na, const int* vox, const int* rowptr, const int* src,

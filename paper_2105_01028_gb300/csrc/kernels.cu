@@ -1,6 +1,6 @@
 // FP32 kernels of one time step: the per-voxel source iteration on CUDA cores (Eq. 12,
-// Section 2.4 steps 5-6), the end of the step (detector / escape tallies of
-// Section 3.1, photon balance, step counter) and the interface split.
+// Section 2.4 steps 5-6), the detector / escape tallies (Section 3.1), the interface
+// split and the step counter.
 #include <cfloat>
 #include <cstdint>
 
@@ -343,14 +343,13 @@ __global__ void __launch_bounds__(ScatterCfg<NA>::kThreads, 2)
 }
 
 // ----------------------------------------------------------------------------------------
-// End of step n: detector curves (FP64 bins, Section 3.1), the energy leaving through the
-// faces, the photon balance and the step counter.
+// Tallies of level n (Section 3.1): detector curves (FP64 bins) and the energy leaving
+// through all faces.
 // Work items are (face, 256 face voxels, 16 directions): a thread loads its voxel's 16
 // values together, so a step's face values (16 MB on the 96x96x64 slab at 192 directions)
 // are in flight at once.  A thread that walked all directions of its voxel in one chain left
 // the kernel bound by that chain's latency: 35 us at 32^3, 572 us at 3072 directions on
-// 32x32x24 voxels; now 8 and 62 us.  The last block to finish takes the balance and advances the
-// counter, which saves the launch of its own (2 us of a step).
+// 32x32x24 voxels; now 8 and 62 us.
 // ----------------------------------------------------------------------------------------
 constexpr int kTallyDirs = 16;
 
@@ -431,21 +430,18 @@ __global__ void __launch_bounds__(256) tally_kernel(GridParams g, const DirInfo*
       atomicAdd(rs.escaped + n, s);
     }
   }
-  if (threadIdx.x == 0) {
-    __threadfence();
-    if (atomicAdd(rs.done, 1) == static_cast<int>(gridDim.x) - 1) {
-      // every block has added its part: the photon balance (energy before step 0 plus what
-      // came in minus what left or was absorbed), its residual against the energy in the box
-      __threadfence();
-      *rs.done = 0;
-      double b = *rs.balance;
-      if (n >= 0 && n < g.pulse_steps) b += g.inj_step;
-      b -= __ldcg(rs.escaped + n) + rs.absorbed[n];
-      *rs.balance = b;
-      rs.residual[n] = b - rs.energy[n];
-      *rs.step = n + 1;
-    }
-  }
+}
+
+// End of step n: the photon balance (energy before step 0 plus what came in minus what
+// left or was absorbed), its residual against the energy in the box, and the step counter.
+__global__ void advance_kernel(GridParams g, RunState rs) {
+  const int n = *rs.step;
+  double b = *rs.balance;
+  if (n >= 0 && n < g.pulse_steps) b += g.inj_step;
+  b -= rs.escaped[n] + rs.absorbed[n];
+  *rs.balance = b;
+  rs.residual[n] = b - rs.energy[n];
+  *rs.step = n + 1;
 }
 
 // Photon energy density of one stored level (Section 3.1 plots its maps): u_v =
@@ -523,6 +519,11 @@ cudaError_t launch_interface(int nvox, int na, const int* vox, const int* rowptr
   const int blocks = (nvox + kIfaceWarps - 1) / kIfaceWarps;
   interface_kernel<<<blocks, 32 * kIfaceWarps, kIfaceWarps * na * sizeof(float), st>>>(
       nvox, na, vox, rowptr, src, w, keep, Q, static_cast<size_t>(nv));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_advance(const GridParams& g, RunState rs, cudaStream_t st) {
+  advance_kernel<<<1, 1, 0, st>>>(g, rs);
   return cudaGetLastError();
 }
 

@@ -119,12 +119,17 @@ __device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// u (|u| < 2^11) = h + l: h the nearest whole number, l the rest to multiples of 2^-12.
-// The magic additions round to nearest even at bit 0 and bit -12; every step is exact.
-__device__ __forceinline__ void split_u(float u, float& h, float& l) {
+// u (|u| < 2^11) = h + l: h the nearest whole number, l the rest to multiples of 2^-12 with
+// the rounding error of the elements before it carried along.  The errors of a row then sum
+// to less than one unit: rounded each on its own, they are noise in the row's photon number
+// (1e-6 of the source function where one direction outshines the others eight times), the
+// mode that the scattering amplifies.  The magic additions round to nearest even at bit 0
+// and bit -12; every other step is exact.
+__device__ __forceinline__ void split_u(float u, float& carry, float& h, float& l) {
   h = (u + 12582912.0f) - 12582912.0f;
-  const float d = u - h;
+  const float d = (u - h) + carry;
   l = (d + 3072.0f) - 3072.0f;
+  carry = d - l;
 }
 
 __device__ __forceinline__ void bulk_to_smem(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -165,7 +170,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
   __shared__ uint64_t mbar;
   __shared__ uint64_t pl_full[C::kSlots], pl_empty[C::kSlots];
   __shared__ uint32_t tmem_base_s;
-  __shared__ int tile_s, next_s;
+  __shared__ int tile_s;
   __shared__ int abort_s;
   __shared__ float e_s[kM], rho_s[kM], den_s[kM];
   __shared__ int ccnt_s[kMaxClasses];
@@ -247,10 +252,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
     if (kUniB1) {  // the same operations as the per-row table below, on the same mu_t
       const int k = cls[i];
       float bs = 0.0f;
-      for (int j = 0; j < nch; ++j) {
-        const float x = g.mut_u * cls_ds[k * nch + j];
-        bs += ray_b1(x, expf(-x));
-      }
+      for (int j = 0; j < nch; ++j) bs += ray_u_fine(g.mut_u, cls_ds[k * nch + j], cls_ds[(16 + k) * nch + j]);
       sB1c[i] = bs * (1.0f / static_cast<float>(nch));
     }
   }
@@ -280,16 +282,17 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
   double esum = 0.0;
   float smax_loc = 0.0f;
   float S[C::HALF];                       // S of the thread's row and columns
-  float qr[C::QR > 0 ? C::QR : 1];        // Q of the thread's last QR columns
+  float qr[C::QR];                        // Q of the thread's last QR columns
   // one unit of Ph and the Chebyshev interval (from the device where P came from there)
   const float tscale = t.dyn ? t.dyn[0] : t.unit, lam = t.dyn ? t.dyn[1] : t.lam, lam_lo = t.dyn ? t.dyn[2] : t.lo;
   bool first_tile = true;
+  int claimed = (kMode == kStep && tid == 0) ? atomicAdd(rs.tile_ctr + (n & 1), 1) : 0;
 
-  // b1 of 8 columns from c0 on (volatile or asm loads: hoisted out of the iterations these
+  // Weight of 8 columns from c0 on, as b1_of and form_x read it (volatile or asm loads: hoisted out of the iterations these
   // tables would cost more registers than there are)
   // (kBuffers: from the caller's array; in the inner iterations as FP16, kept where Xl was)
   int v = 0;
-  const auto load_b1 = [&](int c0, float (&bv)[8], bool inner_pass = false) {
+  const auto load_w = [&](int c0, float (&bv)[8], bool inner_pass = false) {
     if (kMode == kBuffers) {
       if (inner_pass) {
         const volatile __half* hb = reinterpret_cast<const volatile __half*>(sXl) + c0 * kM + row;
@@ -336,6 +339,12 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
     for (int gi = 1; gi < kGroups; ++gi) s += red[gi][row];
     return s;
   };
+  // b1 is held as u = 1 - b1 (kBuffers: as the caller gave it): in thick cells the rounding of
+  // b1 itself would be multiplied by 1 / (1 - a b1), u carries ten times less of it
+  const auto b1_of = [](float w) { return kMode == kBuffers ? w : 1.0f - w; };
+  const auto form_x = [](float w, float sv, float q) {  // Q + b1 S
+    return kMode == kBuffers ? fmaf(w, sv, q) : fmaf(-w, sv, q + sv);
+  };
   // wait for the MMAs committed to mbar; false for the whole warp if the wait ran out
   const auto wait_mma = [&]() {
     const bool ok = mbar_wait_bounded(&mbar, phase);
@@ -348,16 +357,36 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
   // thread 0: the two accumulators of an FP32-accurate product
   const auto issue_product = [&]() {
     tc_fence_after();
+    bool ok = true;
+    // Pl block b (K block b / 2, output directions 96 (b & 1) .. + 95) into the second
+    // accumulator, from ring slot pl_used % kSlots
+    const auto pl_block = [&](int b) {
+      const uint32_t sl = pl_used % C::kSlots;
+      if (ok) ok = mbar_wait_bounded(&pl_full[sl], (pl_used / C::kSlots) & 1u);
+      if (!ok) return;
+      tc_fence_after();
+      const uint32_t kb = static_cast<uint32_t>(b >> 1), d = tmem + C::ROFF + (b & 1) * C::kBlkRows;
 #pragma unroll
-    for (int s = 0; s < C::KSTEPS; ++s) {
-      const uint32_t ko = static_cast<uint32_t>((s & 3) * 32), kb = static_cast<uint32_t>(s >> 2);
-      mma_f16(tmem, sw128_desc(aXh + kb * kM * 128 + ko), sw128_desc(aPh + kb * NA * 128 + ko), C::IDESC, s > 0);
+      for (int ks = 0; ks < 4; ++ks) {
+        const uint64_t pd = sw128_desc(aPl + sl * C::kBlkBytes + ks * 32);
+        mma_f16(d, sw128_desc(aXh + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, (b > 1 || ks > 0) ? 1u : 0u);
+        mma_f16(d, sw128_desc(aXl + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, 1u);
+      }
+      mma_commit(&pl_empty[sl]);
+      ++pl_used;
+    };
+    if constexpr (C::kRing) {
+      // the blocks that are there go first: the others take their slots while the Ph MMAs run
+      static_assert(C::kNblk == 2 * C::kSlots, "the second half of the blocks refills the ring once");
+#pragma unroll 1
+      for (int b = 0; b < C::kSlots; ++b) pl_block(b);
     }
 #pragma unroll
     for (int s = 0; s < C::KSTEPS; ++s) {
       const uint32_t ko = static_cast<uint32_t>((s & 3) * 32), kb = static_cast<uint32_t>(s >> 2);
-      mma_f16(tmem + C::ROFF, sw128_desc(aXl + kb * kM * 128 + ko), sw128_desc(aPh + kb * NA * 128 + ko), C::IDESC,
-              s > 0);
+      const uint64_t pd = sw128_desc(aPh + kb * NA * 128 + ko);
+      mma_f16(tmem, sw128_desc(aXh + kb * kM * 128 + ko), pd, C::IDESC, s > 0);
+      mma_f16(tmem + C::ROFF, sw128_desc(aXl + kb * kM * 128 + ko), pd, C::IDESC, (C::kRing || s > 0) ? 1u : 0u);
     }
     if constexpr (!C::kRing) {
 #pragma unroll
@@ -366,37 +395,16 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
         mma_f16(tmem + C::ROFF, sw128_desc(aXh + ko), sw128_desc(aPl + ko), C::IDESC, 1u);
         mma_f16(tmem + C::ROFF, sw128_desc(aXl + ko), sw128_desc(aPl + ko), C::IDESC, 1u);
       }
-      mma_commit(&mbar);
     } else {
-      // blocks b: K block b / 2, output directions 96 (b & 1) .. + 95; the first three are
-      // resident or in flight
-      static_assert(C::kNblk == 2 * C::kSlots, "the second half of the blocks refills the ring once");
-      bool ok = true;
-#pragma unroll 1
-      for (int b = 0; b < C::kNblk; ++b) {
-        if (b == C::kSlots) {  // as the first blocks' MMAs complete, the others take their slots
-          for (uint32_t q = pl_used; ok && q < pl_used + C::kSlots; ++q) {
-            ok = mbar_wait_bounded(&pl_empty[q % C::kSlots], ((q / C::kSlots) & 1u) ^ 1u);
-            if (ok) pl_load();
-          }
-        }
-        const uint32_t s = pl_used % C::kSlots;
-        if (ok) ok = mbar_wait_bounded(&pl_full[s], (pl_used / C::kSlots) & 1u);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t kb = static_cast<uint32_t>(b >> 1), d = tmem + C::ROFF + (b & 1) * C::kBlkRows;
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-          const uint64_t pd = sw128_desc(aPl + s * C::kBlkBytes + ks * 32);
-          mma_f16(d, sw128_desc(aXh + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, 1u);
-          mma_f16(d, sw128_desc(aXl + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, 1u);
-        }
-        mma_commit(&pl_empty[s]);
-        ++pl_used;
+      for (uint32_t q = pl_used - C::kSlots; ok && q < pl_used; ++q) {
+        ok = mbar_wait_bounded(&pl_empty[q % C::kSlots], (q / C::kSlots) & 1u);
+        if (ok) pl_load();
       }
-      mma_commit(&mbar);
-      if (!ok) abort_s = 1;
+#pragma unroll 1
+      for (int b = C::kSlots; b < C::kNblk; ++b) pl_block(b);
     }
+    mma_commit(&mbar);
+    if (!ok) abort_s = 1;
   };
 
   while (true) {
@@ -405,8 +413,8 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
     if (tid == 0) {
       if (tma_out) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       if (kMode == kStep) {
-        tile_s = first_tile ? atomicAdd(rs.tile_ctr + (n & 1), 1) : next_s;
-        next_s = atomicAdd(rs.tile_ctr + (n & 1), 1);
+        tile_s = claimed;
+        claimed = atomicAdd(rs.tile_ctr + (n & 1), 1);  // needed for the next tile only
       } else {
         tile_s = first_tile ? static_cast<int>(blockIdx.x) : tile_s + static_cast<int>(gridDim.x);
       }
@@ -439,10 +447,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
       float bs = 0.0f;
       if (vv >= 0) {
         const float mu = io.mut[vv];
-        for (int j = 0; j < nch; ++j) {
-          const float x = mu * cls_ds[k * nch + j];
-          bs += ray_b1(x, expf(-x));
-        }
+        for (int j = 0; j < nch; ++j) bs += ray_u_fine(mu, cls_ds[k * nch + j], cls_ds[(16 + k) * nch + j]);
       }
       b1t[k * kM + r] = bs * (1.0f / static_cast<float>(nch));
     }
@@ -456,7 +461,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
         sb = 0.0f;
         for (int k2 = 0; k2 < ncls; ++k2) sb = fmaf(static_cast<float>(ccnt_s[k2]), b1t[k2 * kM + tid], sb);
       }
-      den_s[tid] = static_cast<float>(NA) - (1.0f - e_s[tid]) * sb;
+      den_s[tid] = fmaf(static_cast<float>(NA), e_s[tid], (1.0f - e_s[tid]) * sb);  // sb sums u = 1 - b1
     }
 
     // ---- warm start (the previous level or its extrapolation in time) into registers; Q
@@ -483,17 +488,17 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
         for (int u = 0; u < PR; ++u) {
           const int ch = c2 + u;
           float bv[8];
-          load_b1(cb + ch * CH, bv);
+          load_w(cb + ch * CH, bv);
 #pragma unroll
           for (int j = 0; j < CH; ++j) {
-            if (kMode == kAdjoint) qc[u][j] = fmaf(bv[j], qi[u][j], qc[u][j]);  // Sbar + b1 Ibar
+            if (kMode == kAdjoint) qc[u][j] = form_x(bv[j], qi[u][j], qc[u][j]);  // Sbar + b1 Ibar
             if (kMode == kBuffers) {
               bmax = fmaxf(bmax, bv[j]);
               bsum += bv[j];
             }
             const float s0 = (vin && sp2) ? fmaf(2.0f, s1[u][j], -s2[u][j]) : s1[u][j];
             S[ch * CH + j] = s0;
-            xmax = fmaxf(xmax, fabsf(fmaf(bv[j], s0, qc[u][j])));
+            xmax = fmaxf(xmax, fabsf(form_x(bv[j], s0, qc[u][j])));
             if (ch >= NCT) qr[(ch - NCT) * CH + j] = qc[u][j];
           }
           if (ch < NCT) tmem_st<CH>(t_q + ch * CH, qc[u]);
@@ -527,20 +532,21 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
       // ---- X = Q + b1 S, split
       const int ex = scale_exponent(row_max(red_d), 9);
       const float sx = pow2f(ex);
+      float carry = 0.0f;
 #pragma unroll
       for (int ch = 0; ch < NCH; ++ch) {
         const int c0 = cb + ch * CH;
         float qv[CH], bv[8];
         load_q(ch, qv);
-        load_b1(c0, bv);
+        load_w(c0, bv);
         if (ch < NCT) tmem_wait_ld();
         reg_q(ch, qv);
         uint32_t hi[4], lo[4];
 #pragma unroll
         for (int j = 0; j < CH; j += 2) {
           float h0, l0, h1, l1;
-          split_u(fmaf(bv[j], S[ch * CH + j], qv[j]) * sx, h0, l0);
-          split_u(fmaf(bv[j + 1], S[ch * CH + j + 1], qv[j + 1]) * sx, h1, l1);
+          split_u(form_x(bv[j], S[ch * CH + j], qv[j]) * sx, carry, h0, l0);
+          split_u(form_x(bv[j + 1], S[ch * CH + j + 1], qv[j + 1]) * sx, carry, h1, l1);
           hi[j / 2] = pack_f16x2(h0, h1);
           lo[j / 2] = pack_f16x2(l0, l1);
         }
@@ -568,7 +574,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
           tmem_ld<CH>(t_row + c0, a0);
           tmem_ld<CH>(t_row + C::ROFF + c0, a1);
           load_q(ch, qv);
-          load_b1(c0, bv);
+          load_w(c0, bv);
           lds_vec<8>(sDi + c0, dv);
           lds_vec<8>(sDi + NA + c0, dl);
           tmem_wait_ld();
@@ -576,11 +582,16 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
 #pragma unroll
           for (int j = 0; j < CH; ++j) {
             const float s = S[ch * CH + j];
-            const float x = fmaf(bv[j], s, qv[j]);
-            float y = fmaf(dl[j], x, (a0[j] + a1[j]) * ky);
-            y = fmaf(dv[j], x, y);
-            const float sh = fmaf(-ev, y, y);
-            float r = sh - s;
+            const float x = form_x(bv[j], s, qv[j]);
+            // where scattering prevails y - S is summed from the start (rounding y itself,
+            // alike in all directions of an isotropic field, would be multiplied by
+            // 1 / (1 - a b1)), then r = (y - S) - eps y
+            const float base = al > 0.5f ? s : 0.0f;
+            const float dy = fmaf(dl[j], x, fmaf(dv[j], x, fmaf(a1[j], ky, fmaf(a0[j], ky, -base))));
+            const float y = dy + base;
+            const float da = fmaf(-ev, y, dy);
+            float r = da - (s - base);
+            const float sh = base + da;
             if (kMode == kBuffers)
               reinterpret_cast<__half*>(sXl)[(c0 + j) * kM + row] = __float2half_rn(bv[j]);
             // adjoint, no scattering: y = 0 now; its P z goes where the residual would
@@ -592,7 +603,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
             }
             rm = fmaxf(rm, fabsf(r));
             sm = fmaxf(sm, fabsf(sh));
-            cs = fmaf(bv[j], r, cs);
+            cs = fmaf(b1_of(bv[j]), r, cs);
           }
           tmem_st<CH>(t_row + C::ROFF + c0, a0);
         }
@@ -631,21 +642,28 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
         const float sc = inner ? pow2f(er) : 0.0f;
         if (__any_sync(0xffffffffu, w != 0.0f)) {
 #pragma unroll
-          for (int ch = 0; ch < NCH; ++ch) {
-            const int c0 = cb + ch * CH;
-            float rv[CH], bv[8];
-            tmem_ld<CH>(t_row + C::ROFF + c0, rv);
-            load_b1(c0, bv, true);
-            tmem_wait_ld();
-            uint32_t hi[4];
+          for (int c2 = 0; c2 < NCH; c2 += 2) {
+            const int c0 = cb + c2 * CH;
+            float rv[2 * CH];
+            tmem_ld<2 * CH>(t_row + C::ROFF + c0, rv);
 #pragma unroll
-            for (int j = 0; j < CH; j += 2) {
-              const float d0 = rv[j] + crow, d1 = rv[j + 1] + crow;
-              S[ch * CH + j] = fmaf(w, d0, S[ch * CH + j]);
-              S[ch * CH + j + 1] = fmaf(w, d1, S[ch * CH + j + 1]);
-              hi[j / 2] = pack_f16x2(bv[j] * d0 * sc, bv[j + 1] * d1 * sc);
+            for (int u = 0; u < 2; ++u) {
+              float bv[8];
+              load_w(c0 + u * CH, bv, true);
+              if (u == 0) tmem_wait_ld();
+              uint32_t hi[4];
+#pragma unroll
+              for (int j = 0; j < CH; j += 2) {
+                const float d0 = rv[u * CH + j] + crow, d1 = rv[u * CH + j + 1] + crow;
+                float& s0 = S[(c2 + u) * CH + j];
+                float& s1 = S[(c2 + u) * CH + j + 1];
+                s0 = fmaf(w, d0, s0);
+                s1 = fmaf(w, d1, s1);
+                hi[j / 2] = pack_f16x2(b1_of(bv[j]) * d0 * sc, b1_of(bv[j + 1]) * d1 * sc);
+              }
+              *reinterpret_cast<uint4*>(sXh + sw128_chunk_off(kM, row, c0 + u * CH)) =
+                  make_uint4(hi[0], hi[1], hi[2], hi[3]);
             }
-            *reinterpret_cast<uint4*>(sXh + sw128_chunk_off(kM, row, c0)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
           }
         }
         if (inner) es += om * (rm + fabsf(crow));
@@ -672,17 +690,18 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
             float rv[CH], dd[CH], bv[8], di[8];
             tmem_ld<CH>(t_row + c0, dd);
             tmem_ld<CH>(t_row + C::ROFF + c0, rv);
-            load_b1(c0, bv, true);
+            load_w(c0, bv, true);
             lds_vec<8>(sDi + 2 * NA + c0, di);
             tmem_wait_ld();
 #pragma unroll
             for (int j = 0; j < CH; ++j) {
               const float d = rv[j] + crow;
-              const float y = fmaf(di[j], bv[j] * d, dd[j] * kd);  // P B1 d
+              const float b1 = b1_of(bv[j]);
+              const float y = fmaf(di[j], b1 * d, dd[j] * kd);  // P B1 d
               const float rn = fmaf(wa, y, fmaf(-w, d, rv[j]));
               rv[j] = inner ? rn : rv[j];
               rmx = fmaxf(rmx, fabsf(rv[j]));
-              csx = fmaf(bv[j], rv[j], csx);
+              csx = fmaf(b1, rv[j], csx);
             }
             tmem_st<CH>(t_row + C::ROFF + c0, rv);
           }
@@ -723,11 +742,11 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
       for (int ch = 0; ch < NCH; ++ch) {
         float qv[CH], bv[8];
         load_q(ch, qv);
-        load_b1(cb + ch * CH, bv);
+        load_w(cb + ch * CH, bv);
         if (ch < NCT) tmem_wait_ld();
         reg_q(ch, qv);
 #pragma unroll
-        for (int j = 0; j < CH; ++j) xmax = fmaxf(xmax, fabsf(fmaf(bv[j], S[ch * CH + j], qv[j])));
+        for (int j = 0; j < CH; ++j) xmax = fmaxf(xmax, fabsf(form_x(bv[j], S[ch * CH + j], qv[j])));
       }
       red_d[grp][row] = xmax;
       __syncthreads();
@@ -807,7 +826,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
           float qv[CH], bv[8];
           if (pass == 0) {
             load_q(ch, qv);
-            load_b1(c0, bv);
+            load_w(c0, bv);
             if (ch < NCT) tmem_wait_ld();
             reg_q(ch, qv);
           }
@@ -816,7 +835,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
             const int col = c0 + j;
             float val = S[ch * CH + j];
             if (pass == 0) {
-              val = fmaf(bv[j], S[ch * CH + j], qv[j]);
+              val = form_x(bv[j], S[ch * CH + j], qv[j]);
               if (vin) {
                 esum_row += val;
                 smax_loc = fmaxf(smax_loc, fabsf(S[ch * CH + j]));
@@ -847,14 +866,14 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
       for (int ch = 0; ch < NCH; ++ch) {
         float qv[CH], bv[8];
         load_q(ch, qv);
-        load_b1(cb + ch * CH, bv);
+        load_w(cb + ch * CH, bv);
         if (ch < NCT) tmem_wait_ld();
         reg_q(ch, qv);
         if (vin) {
 #pragma unroll
           for (int j = 0; j < CH; ++j) {
             const float s = S[ch * CH + j];
-            const float Iv = fmaf(bv[j], s, qv[j]);
+            const float Iv = form_x(bv[j], s, qv[j]);
             pI[static_cast<size_t>(ch * CH + j) * plane] = Iv;
             pS[static_cast<size_t>(ch * CH + j) * plane] = s;
             esum_row += Iv;

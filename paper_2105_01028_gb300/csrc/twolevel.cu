@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(256) refine_kernel(GridParams g, const DirInfo
                                                      float* __restrict__ Iring, RunState rs) {
   __shared__ int n_s;
   __shared__ int chd_s[64];
-  __shared__ float ds_s[64];  // the child's ds, or its b1 when mu_t is uniform
+  __shared__ float ds_s[64], dl_s[64];  // the child's ds, or its b1 (u = 1 - b1) when mu_t is uniform
   const int c = blockIdx.y;
   const int tid = threadIdx.x;
   for (int k = tid; k < nch; k += blockDim.x) {
@@ -238,9 +238,10 @@ __global__ void __launch_bounds__(256) refine_kernel(GridParams g, const DirInfo
     chd_s[k] = d;
     if (kUniMu) {
       const float xo = g.mut_u * dirs[d].ds;
-      ds_s[k] = ray_b1(xo, expf(-xo));
+      ds_s[k] = g.fine ? ray_u_fine(g.mut_u, dirs[d].ds, dirs[d].ds_lo) : ray_b1(xo, expf(-xo));
     } else {
       ds_s[k] = dirs[d].ds;
+      dl_s[k] = dirs[d].ds_lo;
     }
   }
   if (tid == 0) n_s = *rs.step;
@@ -254,6 +255,12 @@ __global__ void __launch_bounds__(256) refine_kernel(GridParams g, const DirInfo
   float* Iout = Iring + static_cast<size_t>(ring_slot(n)) * g.na * plane;
   for (int k = 0; k < nch; ++k) {
     const size_t o = static_cast<size_t>(chd_s[k]) * plane + v;
+    const float q = Qf[o];
+    if (g.fine) {
+      const float u = kUniMu ? ds_s[k] : ray_u_fine(mu, ds_s[k], dl_s[k]);
+      Iout[o] = fmaf(-u, s, q + s);
+      continue;
+    }
     float b1;
     if (kUniMu) {
       b1 = ds_s[k];
@@ -261,7 +268,7 @@ __global__ void __launch_bounds__(256) refine_kernel(GridParams g, const DirInfo
       const float xo = mu * ds_s[k];
       b1 = ray_b1(xo, expf(-xo));
     }
-    Iout[o] = fmaf(b1, s, Qf[o]);
+    Iout[o] = fmaf(b1, s, q);
   }
 }
 
