@@ -342,6 +342,9 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
   // b1 is held as u = 1 - b1 (kBuffers: as the caller gave it): in thick cells the rounding of
   // b1 itself would be multiplied by 1 / (1 - a b1), u carries ten times less of it
   const auto b1_of = [](float w) { return kMode == kBuffers ? w : 1.0f - w; };
+  const auto b1_of2 = [](float w0, float w1) {
+    return kMode == kBuffers ? pk(w0, w1) : fma2(pk(w0, w1), pk(-1.0f, -1.0f), pk(1.0f, 1.0f));
+  };
   const auto form_x = [](float w, float sv, float q) {  // Q + b1 S
     return kMode == kBuffers ? fmaf(w, sv, q) : fmaf(-w, sv, q + sv);
   };
@@ -522,6 +525,8 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
     const float ev = e_s[row], al = 1.0f - ev;
     const float amp = rho / (1.0f - rho);           // error bound per unit change
     const float span = rho * lam;                   // Chebyshev interval [lam_lo span, span]
+    const float half = 0.5f * (span - lam_lo * span), mid = 1.0f - 0.5f * (span + lam_lo * span);
+    const float cden = al / den;
     const float eta = kInnerError * fmaxf(1.0f, 0.08f * amp);
     bool live = vin;       // the row takes part in this outer iteration
     bool hitmax = false, bad = false;
@@ -630,17 +635,17 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
         const bool conv = amp * rm <= thr;
         inner = !conv && iters < max_iters && rm <= 3.0e38f;
         hitmax = !conv && !inner;
-        if (inner) crow = al * row_sum(red_c) / den;
+        if (inner) crow = cden * row_sum(red_c);
       }
       // ---- inner iterations on the error equation
-      int k = 0;
+      int k = 0, kc = 0;  // iteration, and its place in the Chebyshev cycle
+      float om = __fdividef(1.0f, fmaf(-half, cw_s[0], mid));
       while (true) {
-        const float half = 0.5f * (span - lam_lo * span), mid = 0.5f * (span + lam_lo * span);
-        const float om = 1.0f / (1.0f - fmaf(half, cw_s[k % t.cycle], mid));
         const float w = inner ? om : (fin ? 0.0f : 1.0f);
         const int er = scale_exponent(rm + fabsf(crow), 13);
         const float sc = inner ? pow2f(er) : 0.0f;
         if (__any_sync(0xffffffffu, w != 0.0f)) {
+          const f32x2 c2p = pk(crow, crow), w2 = pk(w, w), sc2 = pk(sc, sc);
 #pragma unroll
           for (int c2 = 0; c2 < NCH; c2 += 2) {
             const int c0 = cb + c2 * CH;
@@ -654,12 +659,13 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
               uint32_t hi[4];
 #pragma unroll
               for (int j = 0; j < CH; j += 2) {
-                const float d0 = rv[u * CH + j] + crow, d1 = rv[u * CH + j + 1] + crow;
+                const f32x2 d = add2(pk(rv[u * CH + j], rv[u * CH + j + 1]), c2p);
                 float& s0 = S[(c2 + u) * CH + j];
                 float& s1 = S[(c2 + u) * CH + j + 1];
-                s0 = fmaf(w, d0, s0);
-                s1 = fmaf(w, d1, s1);
-                hi[j / 2] = pack_f16x2(b1_of(bv[j]) * d0 * sc, b1_of(bv[j + 1]) * d1 * sc);
+                unpk(fma2(w2, d, pk(s0, s1)), s0, s1);
+                float x0, x1;
+                unpk(mul2(mul2(b1_of2(bv[j], bv[j + 1]), d), sc2), x0, x1);
+                hi[j / 2] = pack_f16x2(x0, x1);
               }
               *reinterpret_cast<uint4*>(sXh + sw128_chunk_off(kM, row, c0 + u * CH)) =
                   make_uint4(hi[0], hi[1], hi[2], hi[3]);
@@ -684,6 +690,8 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
         float rmx = 0.0f, csx = 0.0f;
         if (mma_ok && __any_sync(0xffffffffu, inner)) {
           const float kd = tscale * pow2f(-er), wa = w * al;
+          const f32x2 c2p = pk(crow, crow), nw2 = pk(-w, -w), wa2 = pk(wa, wa), kd2 = pk(kd, kd);
+          f32x2 cs2 = pk(0.0f, 0.0f);
 #pragma unroll
           for (int ch = 0; ch < NCH; ++ch) {
             const int c0 = cb + ch * CH;
@@ -693,20 +701,27 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
             load_w(c0, bv, true);
             lds_vec<8>(sDi + 2 * NA + c0, di);
             tmem_wait_ld();
+            // a row that has stopped has w = 0 and x = 0, so D = 0: its r stays
 #pragma unroll
-            for (int j = 0; j < CH; ++j) {
-              const float d = rv[j] + crow;
-              const float b1 = b1_of(bv[j]);
-              const float y = fmaf(di[j], b1 * d, dd[j] * kd);  // P B1 d
-              const float rn = fmaf(wa, y, fmaf(-w, d, rv[j]));
-              rv[j] = inner ? rn : rv[j];
-              rmx = fmaxf(rmx, fabsf(rv[j]));
-              csx = fmaf(b1, rv[j], csx);
+            for (int j = 0; j < CH; j += 2) {
+              const f32x2 r2 = pk(rv[j], rv[j + 1]), b1 = b1_of2(bv[j], bv[j + 1]);
+              const f32x2 d = add2(r2, c2p);
+              const f32x2 y = fma2(pk(di[j], di[j + 1]), mul2(b1, d), mul2(pk(dd[j], dd[j + 1]), kd2));  // P B1 d
+              const f32x2 rn = fma2(wa2, y, fma2(nw2, d, r2));
+              unpk(rn, rv[j], rv[j + 1]);
+              rmx = fmaxf(rmx, fmaxf(fabsf(rv[j]), fabsf(rv[j + 1])));
+              cs2 = fma2(b1, rn, cs2);
             }
             tmem_st<CH>(t_row + C::ROFF + c0, rv);
           }
+          float cs0, cs1;
+          unpk(cs2, cs0, cs1);
+          csx = cs0 + cs1;
           tmem_wait_st();
         }
+        // the next weight, off the path between the barrier and the next operand
+        kc = kc + 1 < t.cycle ? kc + 1 : 0;
+        om = __fdividef(1.0f, fmaf(-half, cw_s[kc], mid));
         red_d[grp][row] = rmx;
         red_c[grp][row] = csx;
         __syncthreads();
@@ -724,7 +739,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
             if (!conv && iters >= max_iters) hitmax = true;
             crow = 0.0f;
           } else {
-            crow = al * row_sum(red_c) / den;
+            crow = cden * row_sum(red_c);
           }
         }
       }

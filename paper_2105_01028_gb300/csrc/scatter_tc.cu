@@ -92,7 +92,8 @@ struct Tc {
   static constexpr int OFF_R = OFF_B1T + kMaxClasses * kM * 4;      // [NA] f32
   static constexpr int OFF_CLS = OFF_R + NA * 4;                    // [NA] u8 (padded)
   static constexpr int OFF_B1C = OFF_CLS + ((NA + 15) / 16) * 16;   // [NA] f32 (uniform mu_t)
-  static constexpr int OFF_END = OFF_B1C + NA * 4;
+  static constexpr int OFF_GP = OFF_B1C + NA * 4;                   // [NA] f32 b1 (1 - r) (uniform mu_t)
+  static constexpr int OFF_END = OFF_GP + NA * 4;
   static constexpr int SMEM = OFF_END + 1024;                       // + alignment slack
   static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) |
                                     (static_cast<uint32_t>(NA >> 3) << 17) |
@@ -109,6 +110,15 @@ __device__ __forceinline__ void split_bf16x2(float x0, float x1, uint32_t& hi, u
   const float h0 = __uint_as_float(hi << 16);
   const float h1 = __uint_as_float(hi & 0xffff0000u);
   lo = pack_bf16x2(x0 - h0, x1 - h1);
+}
+
+__device__ __forceinline__ void split_bf16x2(f32x2 x, uint32_t& hi, uint32_t& lo) {
+  float x0, x1;
+  unpk(x, x0, x1);
+  hi = pack_bf16x2(x0, x1);
+  const f32x2 h = pk(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+  unpk(fma2(h, pk(-1.0f, -1.0f), x), x0, x1);
+  lo = pack_bf16x2(x0, x1);
 }
 
 // Issue the two MMA chains of one iteration: D = X_hi Pb^T + X_lo Pb^T.
@@ -171,10 +181,11 @@ __global__ void __launch_bounds__(TcThreads<NA>::kThreads, 1)
   float* sR = reinterpret_cast<float*>(smem + C::OFF_R);
   uint8_t* sCls = smem + C::OFF_CLS;
   float* sB1c = reinterpret_cast<float*>(smem + C::OFF_B1C);
+  float* sGp = reinterpret_cast<float*>(smem + C::OFF_GP);
 
   __shared__ uint64_t mbar;
   __shared__ uint32_t tmem_base_s;
-  __shared__ int tile_s, next_s;
+  __shared__ int tile_s;
   __shared__ int plane_s;
   __shared__ int abort_s;
   __shared__ float e_s[kM], rho_s[kM], den_s[kM];
@@ -227,6 +238,7 @@ __global__ void __launch_bounds__(TcThreads<NA>::kThreads, 1)
         bs += ray_b1(x, expf(-x));
       }
       sB1c[i] = bs * (1.0f / static_cast<float>(nch));
+      sGp[i] = fmaf(-sB1c[i], rcorr[i], sB1c[i]);
     }
   }
   // zero the K padding of both A operands once (columns >= NA are never written again)
@@ -265,7 +277,7 @@ __global__ void __launch_bounds__(TcThreads<NA>::kThreads, 1)
   float smax_loc = 0.0f;
 
   float qr[C::QR > 0 ? C::QR : 1];  // Q of the thread's last QR columns
-  bool first_tile = true;
+  int claimed = tid == 0 ? atomicAdd(rs.tile_ctr + (n & 1), 1) : 0;
 
 
   while (true) {
@@ -274,10 +286,9 @@ __global__ void __launch_bounds__(TcThreads<NA>::kThreads, 1)
     // operands) before the warm start writes X again
     if (tid == 0) {
       if (tma_out) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-      tile_s = first_tile ? atomicAdd(rs.tile_ctr + (n & 1), 1) : next_s;
-      next_s = atomicAdd(rs.tile_ctr + (n & 1), 1);
+      tile_s = claimed;
+      claimed = atomicAdd(rs.tile_ctr + (n & 1), 1);  // needed for the next tile only
     }
-    first_tile = false;
     __syncthreads();
     const int tile = tile_s;
     if (tile >= ntiles) break;
@@ -415,6 +426,7 @@ __global__ void __launch_bounds__(TcThreads<NA>::kThreads, 1)
       // the compiler hoists them out of the iteration loop they cost ~190 registers.
       const volatile float* vb1t = b1t;
       float dmax = 0.0f, smax = 0.0f, cpart = 0.0f;
+      const f32x2 crow2 = pk(crow, crow), nev2 = pk(-ev, -ev), neg1 = pk(-1.0f, -1.0f);
       // tcgen05.ld / st are warp-collective: a warp with any active row runs them on every
       // lane; inactive lanes keep S_old (so they rewrite the same X) and report no change.
       if (!to && __any_sync(0xffffffffu, act)) {
@@ -434,40 +446,47 @@ __global__ void __launch_bounds__(TcThreads<NA>::kThreads, 1)
 #pragma unroll
           for (int j8 = 0; j8 < CH; j8 += 8) {
             uint32_t hi[4], lo[4];
-            float rv[8], bv[8];
+            float rv[8], bv[8], gv[8];
             uint32_t cv[2];
             lds_vec<8>(sR + c0 + j8, rv);
-            if (kUniB1)
+            if (kUniB1) {
               lds_vec<8>(sB1c + c0 + j8, bv);
-            else
+              lds_vec<8>(sGp + c0 + j8, gv);
+            } else {
               lds_bytes<8>(sCls + c0 + j8, cv);
+            }
+            // two columns per instruction; every operation and its rounding as written out
+            // one column at a time
 #pragma unroll
             for (int jj = 0; jj < 8; jj += 2) {
-              float xn[2];
+              const int j = j8 + jj;
+              if (!kUniB1) {
 #pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const int j = j8 + jj + e;
-                float b1;
-                if (kUniB1) {
-                  b1 = bv[jj + e];
-                } else {
+                for (int e = 0; e < 2; ++e) {
                   const int cl = static_cast<int>((cv[(jj + e) >> 2] >> (8 * ((jj + e) & 3))) & 0xffu);
-                  b1 = vb1t[cl * kM + row];
+                  bv[jj + e] = vb1t[cl * kM + row];
+                  gv[jj + e] = fmaf(-bv[jj + e], rv[jj + e], bv[jj + e]);  // (Pb b1)_i, estimated
                 }
-                const float qv = qv_[j];
-                const float gp = fmaf(-b1, rv[jj + e], b1);            // (Pb b1)_i, estimated
-                const float sk = so[j] + crow;                         // S_k (correction applied)
-                const float xo = fmaf(b1, sk, qv);                     // X_k = Q + b1 S_k
-                const float yc = fmaf(rv[jj + e], xo, fmaf(crow, gp, y[j]));  // Pb X_k + r X_k
-                const float sn = act ? fmaf(-ev, yc, yc) : sk;         // S_half = (1 - eps) Y
-                const float dl = sn - sk;
-                dmax = fmaxf(dmax, fabsf(dl));
-                smax = fmaxf(smax, fabsf(sn));
-                cpart = fmaf(b1, dl, cpart);
-                so[j] = sn;
-                xn[e] = fmaf(b1, sn, qv);                              // X~ for the next MMA
               }
-              split_bf16x2(xn[0], xn[1], hi[jj / 2], lo[jj / 2]);
+              const f32x2 b1 = pk(bv[jj], bv[jj + 1]), q2 = pk(qv_[j], qv_[j + 1]);
+              const f32x2 sk = add2(pk(so[j], so[j + 1]), crow2);             // S_k (correction applied)
+              const f32x2 xo = fma2(b1, sk, q2);                              // X_k = Q + b1 S_k
+              const f32x2 yc = fma2(pk(rv[jj], rv[jj + 1]), xo,
+                                    fma2(crow2, pk(gv[jj], gv[jj + 1]), pk(y[j], y[j + 1])));  // Pb X_k + r X_k
+              float n0, n1, k0, k1, d0, d1;
+              unpk(fma2(nev2, yc, yc), n0, n1);                               // S_half = (1 - eps) Y
+              unpk(sk, k0, k1);
+              n0 = act ? n0 : k0;
+              n1 = act ? n1 : k1;
+              const f32x2 sn = pk(n0, n1);
+              unpk(fma2(sk, neg1, sn), d0, d1);
+              dmax = fmaxf(dmax, fmaxf(fabsf(d0), fabsf(d1)));
+              smax = fmaxf(smax, fmaxf(fabsf(n0), fabsf(n1)));
+              cpart = fmaf(bv[jj], d0, cpart);
+              cpart = fmaf(bv[jj + 1], d1, cpart);
+              so[j] = n0;
+              so[j + 1] = n1;
+              split_bf16x2(fma2(b1, sn, q2), hi[jj / 2], lo[jj / 2]);          // X~ for the next MMA
             }
             *reinterpret_cast<uint4*>(sAhi + sw128_chunk_off(kM, row, c0 + j8)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
             *reinterpret_cast<uint4*>(sAlo + sw128_chunk_off(kM, row, c0 + j8)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
