@@ -99,6 +99,10 @@ struct trinity_ctx {
   SweepMaps maps{};
   int* d_dlist[3] = {nullptr, nullptr, nullptr};
   int ndir[3] = {0, 0, 0};
+  // plain-load sweep: directions of one ray spacing in groups of four, upwind displacements
+  int* d_group = nullptr;
+  int n_group = 0;
+  int2* d_disp = nullptr;
   int8_t* d_hsh = nullptr;  // per direction: bit 0 / 1 set when its y / z lattice offsets are positive
   GridParams graph_g{}, graph_gs{};  // the parameters the captured kernels were given
 
@@ -620,7 +624,7 @@ int enqueue_transport(trinity_ctx* ctx, const RunState& rs) {
       CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_join[k], 0));
     }
   } else {
-    CK(launch_sweep(g, ctx->d_dirs, ctx->d_offs, ctx->I, ctx->S, ctx->mut, ctx->nidx, ctx->d_refl, ctx->Q, rs,
+    CK(launch_sweep(g, ctx->d_dirs, ctx->d_offs, ctx->d_group, ctx->n_group, ctx->d_disp, ctx->I, ctx->S, ctx->mut, ctx->nidx, ctx->d_refl, ctx->Q, rs,
                     ctx->stream));
   }
   CK(launch_interface(ctx->n_iface, g.na, ctx->d_if_vox, ctx->d_if_rowptr, ctx->d_if_src, ctx->d_if_w,
@@ -1017,6 +1021,43 @@ int trinity_create_grid(const trinity_grid_desc* desc, void* cuda_stream, trinit
     if (cudaMemcpy(ctx->d_cls, cls.data(), na_s, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(ctx->d_cls_ds, flat.data(), flat.size() * sizeof(float), cudaMemcpyHostToDevice) !=
             cudaSuccess)
+      return bail(TRINITY_E_CUDA);
+  }
+  if (!ctx->two_level && !g.periodic && !g.mirror) {
+    // directions whose spacing and delay constants agree to the bit share a segment's weights
+    std::vector<int> group;
+    std::vector<char> used(g.na, 0);
+    for (int d = 0; d < g.na; ++d) {
+      if (used[d]) continue;
+      const DirInfo& a = ctx->hdirs[d];
+      int cnt = 0;
+      for (int e = d; e < g.na && cnt < 4; ++e) {
+        const DirInfo& b = ctx->hdirs[e];
+        if (used[e] || a.ds != b.ds || a.ds_lo != b.ds_lo || a.dcoef != b.dcoef || a.dcoef_lo != b.dcoef_lo) continue;
+        used[e] = 1;
+        group.push_back(e);
+        ++cnt;
+      }
+      for (; cnt < 4; ++cnt) group.push_back(-1);
+    }
+    ctx->n_group = static_cast<int>(group.size() / 4);
+    std::vector<int2> disp(static_cast<size_t>(g.na) * g.nmax);
+    const int str[3] = {1, g.nx, g.nx * g.ny}, ext[3] = {g.nx, g.ny, g.nz};
+    for (int d = 0; d < g.na; ++d) {
+      const DirInfo& a = ctx->hdirs[d];
+      for (int k = 0; k < ext[a.dom]; ++k) {
+        const int o0 = ctx->lat.off[(static_cast<size_t>(d) * 2 + 0) * g.nmax + k];
+        const int o1 = ctx->lat.off[(static_cast<size_t>(d) * 2 + 1) * g.nmax + k];
+        disp[static_cast<size_t>(d) * g.nmax + k] = make_int2(a.sgn * str[a.dom] + o0 * str[a.a0] + o1 * str[a.a1],
+                                                              (o0 & 0xff) | ((o1 & 0xff) << 8));
+      }
+    }
+    if (dalloc(&ctx->d_group, group.size()) != cudaSuccess || dalloc(&ctx->d_disp, disp.size()) != cudaSuccess) {
+      cudaGetLastError();
+      return bail(TRINITY_E_OOM);
+    }
+    if (cudaMemcpy(ctx->d_group, group.data(), group.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(ctx->d_disp, disp.data(), disp.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess)
       return bail(TRINITY_E_CUDA);
   }
   if (!ctx->two_level && sweep_tma_supported(g)) {
@@ -1946,6 +1987,8 @@ void trinity_destroy(trinity_ctx* ctx) {
   cudaFree(ctx->d_tmask);
   for (int c = 0; c < 3; ++c) cudaFree(ctx->d_dlist[c]);
   cudaFree(ctx->d_hsh);
+  cudaFree(ctx->d_group);
+  cudaFree(ctx->d_disp);
   for (int k = 0; k < 2; ++k) {
     if (ctx->side[k]) cudaStreamDestroy(ctx->side[k]);
     if (ctx->ev_join[k]) cudaEventDestroy(ctx->ev_join[k]);

@@ -195,8 +195,10 @@ __device__ __forceinline__ void ray_weights_fine(float mu, float ds, float ds_lo
 }
 
 // Kernel launchers (defined in kernels.cu / scatter_tc.cu).
-cudaError_t launch_sweep(const GridParams& g, const DirInfo* dirs, const int8_t* offs,
-                         const float* Iring, const float* Sring, const float* mut,
+// group: [ngroups][4] directions of one ray spacing (-1: none); disp: [na][nmax] displacement
+// of the upwind voxel and the two lattice offsets (a byte each) per direction and slab.
+cudaError_t launch_sweep(const GridParams& g, const DirInfo* dirs, const int8_t* offs, const int* group, int ngroups,
+                         const int2* disp, const float* Iring, const float* Sring, const float* mut,
                          const float* nidx, const int* refl, float* Q, RunState rs, cudaStream_t st);
 cudaError_t launch_scatter_fp32(const GridParams& g, const float* b1ds, int nch, const float* P,
                                 const float* rcorr, const float* Q, const float* mut,
