@@ -262,7 +262,7 @@ int trinity_kernels_per_step(const trinity_ctx* ctx, int* n);
 
 /* Form of the ray sweep a step runs: 0 plain loads (one kernel), 1 upwind planes staged
  * through TMA tile loads (one kernel per dominant-axis class, run concurrently: vacuum
- * faces, a uniform refractive index, nx a multiple of 4), 2 the fused two-level sweep. */
+ * faces, uniform refractive index and mu_t, nx a multiple of 4), 2 the fused two-level sweep. */
 int trinity_sweep_form(const trinity_ctx* ctx, int* form);
 
 /* on = 0: the plain-load sweep even where the TMA-staged one applies (both perform the

@@ -99,7 +99,7 @@ struct trinity_ctx {
   SweepMaps maps{};
   int* d_dlist[3] = {nullptr, nullptr, nullptr};
   int ndir[3] = {0, 0, 0};
-  // plain-load sweep: directions of one ray spacing in groups of four, upwind displacements
+  // plain-load sweep: directions of one ray spacing in groups, upwind displacements
   int* d_group = nullptr;
   int n_group = 0;
   int2* d_disp = nullptr;
@@ -600,9 +600,15 @@ int restore_checkpoint(trinity_ctx* ctx, int k, int c, bool store) {
 // Sweep (Eq. 10's known part Q) and the interface split; on a two-level grid also the
 // mean of Q over each coarse direction's children.
 // The step's sweep stages its upwind planes through the TMA: supported box, uniform
-// refractive index (one retarded delay per direction), not switched off.
+// refractive index (one retarded delay per direction), not switched off, and a uniform mu_t
+// (0.445 ms on the 96x96x64 slab, the plain-load form 0.476).  Where mu_t varies the plain-load
+// form is the faster one, as it shares a voxel's weights among directions: 0.230 against
+// 0.261 ms at 64^3, 0.181 against 0.213 at 56^3 (192 directions, the same bits).  On the
+// smallest boxes its one launch beats three with a fork and a join: 9 against 14 us at 16^3 and
+// 48 directions (2^17.6 updates; from 2^19 on the TMA form is kept).
 bool sweep_uses_tma(const trinity_ctx* ctx) {
-  return !ctx->two_level && ctx->tma && !ctx->tma_off && ctx->g.n_u >= 1.0f;
+  return !ctx->two_level && ctx->tma && !ctx->tma_off && ctx->g.n_u >= 1.0f && ctx->g.mut_u >= 0.0f &&
+         static_cast<long>(ctx->g.nv) * ctx->g.na >= (1L << 19);
 }
 
 int enqueue_transport(trinity_ctx* ctx, const RunState& rs) {
@@ -617,7 +623,7 @@ int enqueue_transport(trinity_ctx* ctx, const RunState& rs) {
     const cudaStream_t st3[3] = {ctx->stream, ctx->side[0], ctx->side[1]};
     CK(cudaEventRecord(ctx->ev_fork, ctx->stream));
     for (int k = 0; k < 2; ++k) CK(cudaStreamWaitEvent(ctx->side[k], ctx->ev_fork, 0));
-    CK(launch_sweep_tma(g, ctx->d_dirs, dl, ctx->ndir, ctx->d_offs, ctx->d_hsh, ctx->maps, ctx->mut, ctx->Q, rs,
+    CK(launch_sweep_tma(g, ctx->d_dirs, dl, ctx->ndir, ctx->d_offs, ctx->d_hsh, ctx->maps, ctx->Q, rs,
                         st3));
     for (int k = 0; k < 2; ++k) {
       CK(cudaEventRecord(ctx->ev_join[k], ctx->side[k]));
@@ -1031,16 +1037,16 @@ int trinity_create_grid(const trinity_grid_desc* desc, void* cuda_stream, trinit
       if (used[d]) continue;
       const DirInfo& a = ctx->hdirs[d];
       int cnt = 0;
-      for (int e = d; e < g.na && cnt < 4; ++e) {
+      for (int e = d; e < g.na && cnt < kSweepGroup; ++e) {
         const DirInfo& b = ctx->hdirs[e];
         if (used[e] || a.ds != b.ds || a.ds_lo != b.ds_lo || a.dcoef != b.dcoef || a.dcoef_lo != b.dcoef_lo) continue;
         used[e] = 1;
         group.push_back(e);
         ++cnt;
       }
-      for (; cnt < 4; ++cnt) group.push_back(-1);
+      for (; cnt < kSweepGroup; ++cnt) group.push_back(-1);
     }
-    ctx->n_group = static_cast<int>(group.size() / 4);
+    ctx->n_group = static_cast<int>(group.size() / kSweepGroup);
     std::vector<int2> disp(static_cast<size_t>(g.na) * g.nmax);
     const int str[3] = {1, g.nx, g.nx * g.ny}, ext[3] = {g.nx, g.ny, g.nz};
     for (int d = 0; d < g.na; ++d) {

@@ -195,7 +195,8 @@ __device__ __forceinline__ void ray_weights_fine(float mu, float ds, float ds_lo
 }
 
 // Kernel launchers (defined in kernels.cu / scatter_tc.cu).
-// group: [ngroups][4] directions of one ray spacing (-1: none); disp: [na][nmax] displacement
+constexpr int kSweepGroup = 4;  // directions per thread of the plain-load sweep
+// group: [ngroups][kSweepGroup] directions of one ray spacing (-1: none); disp: [na][nmax] displacement
 // of the upwind voxel and the two lattice offsets (a byte each) per direction and slab.
 cudaError_t launch_sweep(const GridParams& g, const DirInfo* dirs, const int8_t* offs, const int* group, int ngroups,
                          const int2* disp, const float* Iring, const float* Sring, const float* mut,
@@ -221,7 +222,7 @@ bool sweep_tma_supported(const GridParams& g);
 cudaError_t make_sweep_maps(const GridParams& g, float* Iring, float* Sring, SweepMaps* out);
 cudaError_t launch_sweep_tma(const GridParams& g, const DirInfo* dirs, const int* const dlist[3],
                              const int ndir[3], const int8_t* offs, const int8_t* hsh, const SweepMaps& maps,
-                             const float* mut, float* Q, RunState rs, const cudaStream_t st[3]);
+                             float* Q, RunState rs, const cudaStream_t st[3]);
 cudaError_t launch_advance(const GridParams& g, RunState rs, cudaStream_t st);
 cudaError_t launch_energy_density(const GridParams& g, const float* I, const float* nidx, float scale, float* u,
                                   cudaStream_t st);

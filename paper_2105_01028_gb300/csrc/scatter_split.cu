@@ -148,8 +148,10 @@ __device__ __forceinline__ void bulk_to_smem(uint32_t dst, const void* src, uint
 enum SplitMode { kStep = 0, kBuffers = 1, kAdjoint = 2 };
 
 // kUniB1: mu_t is the same in every voxel, so b1 depends on the column's ray spacing only.
-template <int NA, bool kUniB1, int kMode>
-__global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
+// kPer: CTAs per SM (two at 48 directions where there are tiles enough; the registers that this
+// takes would cost a single CTA 20%).
+template <int NA, bool kUniB1, int kMode, int kPer>
+__global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
     scatter_split_kernel(GridParams g, SplitTables t, const uint8_t* __restrict__ cls,
                          const float* __restrict__ cls_ds, int ncls, int nch, SplitIo io, float tol, int max_iters,
                          const __grid_constant__ CUtensorMap tmOutI, const __grid_constant__ CUtensorMap tmOutS,
@@ -963,13 +965,21 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, 1)
 
 int g_split_sms = 0;
 
-template <int NA, int kMode>
+template <int NA, int kMode, int kPer>
 cudaError_t configure_split() {
-  cudaError_t e = cudaFuncSetAttribute(scatter_split_kernel<NA, false, kMode>,
+  cudaError_t e = cudaFuncSetAttribute(scatter_split_kernel<NA, false, kMode, kPer>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, Sp<NA>::SMEM);
   if (e != cudaSuccess || kMode == kBuffers) return e;
-  return cudaFuncSetAttribute(scatter_split_kernel<NA, kMode != kBuffers, kMode>,
+  return cudaFuncSetAttribute(scatter_split_kernel<NA, kMode != kBuffers, kMode, kPer>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, Sp<NA>::SMEM);
+}
+
+template <int kMode>
+cudaError_t configure_mode() {
+  cudaError_t e = configure_split<48, kMode, 1>();
+  if (e == cudaSuccess) e = configure_split<48, kMode, 2>();
+  if (e == cudaSuccess) e = configure_split<192, kMode, 1>();
+  return e;
 }
 
 template <int kMode>
@@ -978,15 +988,21 @@ cudaError_t launch_split(const GridParams& g, const SplitTables& sp, const BfTab
                          cudaStream_t st) {
   if (g_split_sms == 0) return cudaErrorInvalidValue;
   const int ntiles = kMode == kBuffers ? (g.nv + kM - 1) / kM : brick_tiles(g.nx, g.ny, g.nz);
-  const int grid = ntiles < g_split_sms ? ntiles : g_split_sms;
   constexpr bool kU = kMode != kBuffers;
   const bool uni = kU && g.mut_u >= 0.0f;
   if (g.na == 48) {
-    auto k = uni ? scatter_split_kernel<48, kU, kMode> : scatter_split_kernel<48, false, kMode>;
+    // two CTAs per SM from 2.5 tiles per SM on (as scatter_tc.cu): 0.273 against 0.307 ms at
+    // 56^3 with varying mu_t, 0.683 against 0.809 at 80^3; one CTA otherwise (0.061 against
+    // 0.073 ms a step at 16^3)
+    const bool two = 2 * ntiles > 5 * g_split_sms;
+    const int cap = two ? 2 * g_split_sms : g_split_sms, grid = ntiles < cap ? ntiles : cap;
+    auto k = two ? (uni ? scatter_split_kernel<48, kU, kMode, 2> : scatter_split_kernel<48, false, kMode, 2>)
+                 : (uni ? scatter_split_kernel<48, kU, kMode, 1> : scatter_split_kernel<48, false, kMode, 1>);
     k<<<grid, Sp<48>::kThreads, Sp<48>::SMEM, st>>>(g, sp, t.cls, t.cls_ds, t.ncls, t.nch, io, tol, max_iters, mI, mS,
                                                     tma_out, rs);
   } else if (g.na == 192) {
-    auto k = uni ? scatter_split_kernel<192, kU, kMode> : scatter_split_kernel<192, false, kMode>;
+    const int grid = ntiles < g_split_sms ? ntiles : g_split_sms;
+    auto k = uni ? scatter_split_kernel<192, kU, kMode, 1> : scatter_split_kernel<192, false, kMode, 1>;
     k<<<grid, Sp<192>::kThreads, Sp<192>::SMEM, st>>>(g, sp, t.cls, t.cls_ds, t.ncls, t.nch, io, tol, max_iters, mI,
                                                       mS, tma_out, rs);
   } else {
@@ -1010,9 +1026,8 @@ bool scatter_split_supported(int na, int ncls) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        configure_split<48, kStep>() != cudaSuccess || configure_split<192, kStep>() != cudaSuccess ||
-        configure_split<48, kBuffers>() != cudaSuccess || configure_split<192, kBuffers>() != cudaSuccess ||
-        configure_split<48, kAdjoint>() != cudaSuccess || configure_split<192, kAdjoint>() != cudaSuccess) {
+        configure_mode<kStep>() != cudaSuccess || configure_mode<kBuffers>() != cudaSuccess ||
+        configure_mode<kAdjoint>() != cudaSuccess) {
       cudaGetLastError();
       return false;
     }

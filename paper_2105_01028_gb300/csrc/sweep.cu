@@ -248,11 +248,12 @@ __global__ void __launch_bounds__(256) sweep_kernel(GridParams g, const DirInfo*
 // where an upwind sample lies follows from a table per (direction, slab): its displacement
 // and the two lattice offsets.  One direction per thread was bound by instruction issue, not
 // by HBM, where the optics vary (a division, an exponential and the index arithmetic for 20
-// bytes): 2.05 ms at 128x128x96 voxels, 192 directions with n and mu_t varying, now 1.50;
-// 0.63 ms at 77^3 with mu_t varying, now 0.50.
+// bytes): 2.05 ms at 128x128x96 voxels, 192 directions with n and mu_t varying, now 1.48;
+// 0.63 ms at 77^3 with mu_t varying, now 0.49.  Eight directions per thread gain nothing (1.49)
+// and cost a uniform medium 20%.
 // ----------------------------------------------------------------------------------------
-constexpr int kGroupDirs = 4;
-constexpr int kRowSweepsG = 4;  // row groups per block
+constexpr int kGroupDirs = kSweepGroup;
+constexpr int kRowSweepsG = 8;  // row groups per block at most (2: 8% slower, the set-up weighs more)
 
 template <bool kUniN, bool kUniMu>
 __global__ void __launch_bounds__(256)
@@ -391,7 +392,11 @@ cudaError_t launch_sweep(const GridParams& g, const DirInfo* dirs, const int8_t*
   dim3 grid((groups + kRowSweeps - 1) / kRowSweeps, g.na);
   const bool un = g.n_u >= 1.0f, um = g.mut_u >= 0.0f;
   if (!g.periodic && !g.mirror) {
-    const dim3 gg((groups + kRowSweepsG - 1) / kRowSweepsG, ngroups);
+    // fewer row groups per block where the grid would otherwise not fill the chip (16^3 at 48
+    // directions: 60 blocks of eight row groups take 19 us, 480 of one row group 14)
+    int rs_n = groups * ngroups / (152 * 8);
+    rs_n = rs_n < 1 ? 1 : (rs_n > kRowSweepsG ? kRowSweepsG : rs_n);
+    const dim3 gg((groups + rs_n - 1) / rs_n, ngroups);
     auto k = un ? (um ? sweep_group_kernel<true, true> : sweep_group_kernel<true, false>)
                 : (um ? sweep_group_kernel<false, true> : sweep_group_kernel<false, false>);
     k<<<gg, block, 0, st>>>(g, dirs, group, disp, Iring, Sring, mut, nidx, Q, rs);

@@ -1,7 +1,8 @@
 // The one-level ray sweep with its upwind planes staged through the Tensor Memory
 // Accelerator: Eq. 10 without its S(n) term, on the slab lattice of Section 2.1, for
 // boxes with a uniform refractive index (the retarded delay is then the same for every
-// voxel of a direction, so each output tile needs exactly two stored levels of I and S).
+// voxel of a direction, so each output tile needs exactly two stored levels of I and S) and a
+// uniform mu_t (where it varies the plain-load form is faster, see sweep_uses_tma in api.cu).
 //
 // Q(v, d) = T (I_up) + b0 (S_up), the upwind values interpolated in time between levels
 // n - m and n - m - 1 (the same arithmetic as sweep.cu's kUniN forms).  Work items are
@@ -98,7 +99,7 @@ struct Box {
 // Per-direction constants of the current step (same for all of its items).
 struct DirStep {
   int d, sgn, m;
-  float f, T, b0, b0l, src_amp;  // per-voxel weights: b0, b0l hold the spacing and its remainder
+  float f, T, b0, b0l, src_amp;
   int p0, p1;       // plane coordinates of levels n - m and n - m - 1 in the ring tensor
   bool h0, h1;      // the level lies in the stored history (else it reads as zero)
 };
@@ -113,14 +114,14 @@ struct ItemInfo {
   int dx;       // x shift of the upwind samples (dom y, z)
 };
 
-template <int DOM, bool kUniMu>
+template <int DOM>
 __global__ void __launch_bounds__(256) sweep_tma_kernel(GridParams g, const DirInfo* __restrict__ dirs,
                                                         const int* __restrict__ dlist, int ndir,
                                                         const int8_t* __restrict__ offs,
                                                         const int8_t* __restrict__ hsh,
                                                         const __grid_constant__ CUtensorMap tmI,
                                                         const __grid_constant__ CUtensorMap tmS,
-                                                        const float* __restrict__ mut, float* __restrict__ Q,
+                                                        float* __restrict__ Q,
                                                         RunState rs, int first) {
   using B = Box<DOM>;
   const int W = DOM == 0 ? kXw : g.nx + 2 * kPad;
@@ -167,16 +168,10 @@ __global__ void __launch_bounds__(256) sweep_tma_kernel(GridParams g, const DirI
     s.f = f;
     s.src_amp = di.src_amp;
     s.b0l = 0.0f;
-    if (kUniMu) {
-      const float xo = g.mut_u * di.ds;
-      s.T = expf(-xo);
-      s.b0 = ray_b0(xo, s.T);
-      if (g.fine) ray_weights_fine(g.mut_u, di.ds, di.ds_lo, s.T, s.b0, s.b0l);
-    } else {
-      s.T = 0.0f;
-      s.b0 = di.ds;
-      s.b0l = di.ds_lo;
-    }
+    const float xo = g.mut_u * di.ds;
+    s.T = expf(-xo);
+    s.b0 = ray_b0(xo, s.T);
+    if (g.fine) ray_weights_fine(g.mut_u, di.ds, di.ds_lo, s.T, s.b0, s.b0l);
     const int L0 = n - s.m, L1 = n - s.m - 1;
     s.h0 = L0 >= g.hist_from;
     s.h1 = L1 >= g.hist_from;
@@ -282,22 +277,7 @@ __global__ void __launch_bounds__(256) sweep_tma_kernel(GridParams g, const DirI
         Iup = fmaf(w1, i1, w0 * i0);
         Sup = fmaf(w1, s1v, w0 * s0v);
       }
-      float T, b0, b0l = 0.0f;
-      if (kUniMu) {
-        T = s.T;
-        b0 = s.b0;
-        b0l = s.b0l;
-      } else {
-        const float mu = __ldg(mut + v);
-        if (g.fine) {
-          ray_weights_fine(mu, s.b0, s.b0l, T, b0, b0l);
-        } else {
-          const float xo = mu * s.b0;
-          T = expf(-xo);
-          b0 = ray_b0(xo, T);
-        }
-      }
-      Qd[v] = fmaf(Sup, b0, fmaf(Sup, b0l, Iup * T));
+      Qd[v] = fmaf(Sup, s.b0, fmaf(Sup, s.b0l, Iup * s.T));
     };
     if (DOM == 2 || DOM == 1) {
       // warps over the item's rows, lanes along x
@@ -386,7 +366,7 @@ namespace {
 
 template <int DOM>
 cudaError_t launch_class(const GridParams& g, const DirInfo* dirs, const int* dlist, int ndir, const int8_t* offs,
-                         const int8_t* hsh, const SweepMaps& maps, const float* mut, float* Q, RunState rs,
+                         const int8_t* hsh, const SweepMaps& maps, float* Q, RunState rs,
                          int first, int nsm, cudaStream_t st) {
   if (ndir == 0) return cudaSuccess;
   using Bx = Box<DOM>;
@@ -396,15 +376,14 @@ cudaError_t launch_class(const GridParams& g, const DirInfo* dirs, const int* dl
   CUtensorMap mI, mS;
   std::memcpy(&mI, maps.I[DOM], sizeof(CUtensorMap));
   std::memcpy(&mS, maps.S[DOM], sizeof(CUtensorMap));
-  const bool um = g.mut_u >= 0.0f;
-  auto kern = um ? sweep_tma_kernel<DOM, true> : sweep_tma_kernel<DOM, false>;
+  auto kern = sweep_tma_kernel<DOM>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   int per_sm = 1;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  kern<<<nsm * per_sm, 256, smem, st>>>(g, dirs, dlist, ndir, offs, hsh, mI, mS, mut, Q, rs, first);
+  kern<<<nsm * per_sm, 256, smem, st>>>(g, dirs, dlist, ndir, offs, hsh, mI, mS, Q, rs, first);
   return cudaGetLastError();
 }
 
@@ -412,7 +391,7 @@ cudaError_t launch_class(const GridParams& g, const DirInfo* dirs, const int* dl
 
 cudaError_t launch_sweep_tma(const GridParams& g, const DirInfo* dirs, const int* const dlist[3],
                              const int ndir[3], const int8_t* offs, const int8_t* hsh, const SweepMaps& maps,
-                             const float* mut, float* Q, RunState rs, const cudaStream_t st[3]) {
+                             float* Q, RunState rs, const cudaStream_t st[3]) {
   static int nsm = 0;
   if (nsm == 0) {
     int dev = 0;
@@ -424,9 +403,9 @@ cudaError_t launch_sweep_tma(const GridParams& g, const DirInfo* dirs, const int
   const int f2 = ndir[2] > 0, f1 = !f2 && ndir[1] > 0, f0 = !f2 && !f1;
   // the classes write disjoint planes of Q and only read the rings: st[k] may run them
   // concurrently (the caller joins the streams before the next kernel)
-  cudaError_t e = launch_class<2>(g, dirs, dlist[2], ndir[2], offs, hsh, maps, mut, Q, rs, f2, nsm, st[0]);
-  if (e == cudaSuccess) e = launch_class<1>(g, dirs, dlist[1], ndir[1], offs, hsh, maps, mut, Q, rs, f1, nsm, st[1]);
-  if (e == cudaSuccess) e = launch_class<0>(g, dirs, dlist[0], ndir[0], offs, hsh, maps, mut, Q, rs, f0, nsm, st[2]);
+  cudaError_t e = launch_class<2>(g, dirs, dlist[2], ndir[2], offs, hsh, maps, Q, rs, f2, nsm, st[0]);
+  if (e == cudaSuccess) e = launch_class<1>(g, dirs, dlist[1], ndir[1], offs, hsh, maps, Q, rs, f1, nsm, st[1]);
+  if (e == cudaSuccess) e = launch_class<0>(g, dirs, dlist[0], ndir[0], offs, hsh, maps, Q, rs, f0, nsm, st[2]);
   return e;
 }
 
