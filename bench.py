@@ -432,12 +432,12 @@ def run_adjoint(args):
     copy_ach = copy_bytes / (st[2] * 1e-3) / 1e9
     fwd_flops = 2.0 * na * na * nv * float(np.mean(fit_mean)) * steps
     phases = [
-        {"name": "forward, checkpointed (sweep + scatter_fp32 + tallies)", "ms": ms_fwd},
+        {"name": "forward, checkpointed (sweep + source iteration + tallies)", "ms": ms_fwd},
         {"name": "checkpoint restores", "ms": st[0]},
         {"name": "recomputed forward steps", "ms": st[1]},
         {"name": "segment-store copies", "ms": st[2], "bound": "hbm", "achieved": copy_ach, "peak": hbm,
          "unit": "GB/s", "frac": copy_ach / hbm},
-        {"name": "adj_scatter_fp32 (transposed solve) + injection", "ms": st[3], "bound": "alu",
+        {"name": "transposed solve (scatter_split, adjoint mode) + injection", "ms": st[3], "bound": "alu",
          "achieved": solve_ach, "peak": fp32_peak, "unit": "TFLOP/s", "frac": solve_ach / fp32_peak,
          "iterations_mean": it_adj},
         {"name": "adj_push (+ transposed interface split)", "ms": st[4], "bound": "hbm",
@@ -460,9 +460,9 @@ def run_adjoint(args):
                              % (T.adjoint_footprint_bytes(p, steps, every) / 1e9)},
             "gpu_launches": int(8 * steps + 3 * steps + (steps + every - 1) // every + 2),
             "status": status,
-            "roofline": {"kernel": "adj_scatter_fp32", "bound": "alu", "achieved": solve_ach,
+            "roofline": {"kernel": "scatter_split (adjoint mode)", "bound": "alu", "achieved": solve_ach,
                          "peak": fp32_peak, "unit": "TFLOP/s", "frac": solve_ach / fp32_peak,
-                         "traffic": measured_traffic("adj_scatter_fp32_kernel", nv * na),
+                         "traffic": measured_traffic("scatter_split_kernel", nv * na),
                          "peak_source": "FP32 FFMA: %d SMs x 128 lanes x 2 x max SM clock" % sm_count()},
             "phases": phases,
             "forward_scatter_tflops": fwd_flops / (ms_fwd * 1e-3) / 1e12,
@@ -579,9 +579,9 @@ def measure_window(T, torch, prob, stream, spinup, warmup, steps, what, slab_tra
                                     exact=xform)
     # measured DRAM bytes of the dominant kernel (committed ncu table, captured on the slab,
     # while its source is unchanged); not for workloads whose kernel instances differ
-    names = {"sweep": {"tma": "sweep_tma_kernel", "plain": "sweep_kernel"}.get(sform, "sweep2_kernel"),
+    names = {"sweep": {"tma": "sweep_tma_kernel", "plain": "sweep_group_kernel"}.get(sform, "sweep2_kernel"),
              "exact_tc": "exact_tc_kernel", "exact_fp32": "exact_gemm192_kernel",
-             "scatter_bf16": "scatter_tc_kernel", "scatter_fp32": "scatter_fp32_kernel"}
+             "scatter_bf16": "scatter_tc_kernel", "scatter_fp32": "scatter_split_kernel"}
     if slab_traffic and roof["kernel"] in names:
         roof["traffic"] = measured_traffic(names[roof["kernel"]], nv * na)
     return {"workload": what, "precision": prec, "value": nv * na * steps / (ms * 1e-3), "unit": "updates/s",
@@ -750,7 +750,7 @@ def main():
     k_exec = float(np.mean(fwd.executed_iterations()[-kp:]))  # the profiled steps
     kps = fwd.kernels_per_step()
     xform = fwd.exact_form()
-    sweep_kernel = {"plain": "sweep_kernel", "tma": "sweep_tma_kernel", "two-level": "sweep2_kernel"}[fwd.sweep_form()]
+    sweep_kernel = {"plain": "sweep_group_kernel", "tma": "sweep_tma_kernel", "two-level": "sweep2_kernel"}[fwd.sweep_form()]
     fwd.close()
 
     updates = nv * na * args.steps
@@ -818,7 +818,7 @@ def main():
                       "algorithmic_bytes": fin_bytes}
     dom = max(kernels[:2], key=lambda k: k["ms"])
     scat_kernel = (("exact_tc_kernel" if xform == "tc" else "exact_gemm192_kernel") if args.exact else
-                   "scatter_tc_kernel" if args.precision == "bf16" else "scatter_fp32_kernel")
+                   "scatter_tc_kernel" if args.precision == "bf16" else "scatter_split_kernel")
     traffic = (measured_traffic(scat_kernel, nv * na_s) if dom is kernels[1]
                else measured_traffic(sweep_kernel, nv * na))
     roof = {"kernel": dom["name"], "bound": dom["bound"], "achieved": dom["achieved"],
@@ -847,7 +847,7 @@ def main():
     if plain and args.precision != "fp32" and not args.no_fp32:
         p32 = W.config_slab(steps=total, precision="fp32", nx=nx, ny=ny, nz=nz)
         sub = measure_window(T, torch, p32, stream, args.spinup, args.warmup, args.steps,
-                             "the same slab and time window, plain FP32 (source iteration on CUDA cores)")
+                             "the same slab and time window, plain FP32 (source iteration on split FP16 products)")
         sub["value"] *= ws
         sub["bf16_speedup"] = line["value"] / sub["value"]
         line["fp32"] = sub

@@ -196,11 +196,12 @@ int trinity_set_initial_state(trinity_ctx* ctx, const float* I0, const float* S0
  * from 2 S(n-1) - S(n-2) (trinity_set_warm_start) and stopped when
  *   rho/(1-rho) |S^k - S^(k-1)|_inf <= tol * scale,  scale = max(|S^k|_inf, 1e-6 max|S(n-1)|)
  * (rho = a * max_d b1, a bound on the contraction) or when the iterate sits at the noise
- * floor of the mode's arithmetic: FP32 mode, the change has not reached a new minimum for
- * three iterations; BF16 mode, |S^k - S^(k-1)|_inf <= 2^-17 scale (the resolution of X
+ * floor of the mode's arithmetic: FP32 mode (12 directions), the change has not reached a new
+ * minimum for three iterations (from 48 directions on the bound is taken at tol / 4 on
+ * residuals formed with FP32 accuracy, corrected by Chebyshev iterations, until a residual
+ * is no longer halved); BF16 mode, |S^k - S^(k-1)|_inf <= 2^-17 scale (the resolution of X
  * carried as two BF16 terms) or no new minimum for two iterations.  Then the detector and
- * energy tallies.  iters_out (may be
- * NULL) receives the largest iteration count of each step.  Returns
+ * energy tallies.  iters_out (may be NULL) receives the largest iteration count of each step.  Returns
  * TRINITY_W_NOT_CONVERGED if any voxel hit max_iters. */
 int trinity_step(trinity_ctx* ctx, int nsteps, int* iters_out);
 
