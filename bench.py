@@ -420,7 +420,7 @@ def run_adjoint(args):
     ad = float(np.sum(ga * (p["mua"] * da).ravel()) + np.sum(gs * (p["mus"] * ds).ravel()))
 
     pk = peaks()
-    fp32_peak = fp32_peak_tflops(pk)
+    tc_peak = pk.get("bf16_tflops_sustained", 1700.0)
     hbm = pk["hbm_gbs"]
     upd = nv * na * steps
     it_adj = float(st[6])
@@ -437,8 +437,8 @@ def run_adjoint(args):
         {"name": "recomputed forward steps", "ms": st[1]},
         {"name": "segment-store copies", "ms": st[2], "bound": "hbm", "achieved": copy_ach, "peak": hbm,
          "unit": "GB/s", "frac": copy_ach / hbm},
-        {"name": "transposed solve (scatter_split, adjoint mode) + injection", "ms": st[3], "bound": "alu",
-         "achieved": solve_ach, "peak": fp32_peak, "unit": "TFLOP/s", "frac": solve_ach / fp32_peak,
+        {"name": "transposed solve (scatter_split, adjoint mode) + injection", "ms": st[3], "bound": "tensor",
+         "achieved": solve_ach, "peak": tc_peak, "unit": "TFLOP/s", "frac": solve_ach / tc_peak,
          "iterations_mean": it_adj},
         {"name": "adj_push (+ transposed interface split)", "ms": st[4], "bound": "hbm",
          "achieved": push_ach, "peak": hbm, "unit": "GB/s", "frac": push_ach / hbm,
@@ -460,10 +460,10 @@ def run_adjoint(args):
                              % (T.adjoint_footprint_bytes(p, steps, every) / 1e9)},
             "gpu_launches": int(8 * steps + 3 * steps + (steps + every - 1) // every + 2),
             "status": status,
-            "roofline": {"kernel": "scatter_split (adjoint mode)", "bound": "alu", "achieved": solve_ach,
-                         "peak": fp32_peak, "unit": "TFLOP/s", "frac": solve_ach / fp32_peak,
+            "roofline": {"kernel": "scatter_split (adjoint mode)", "bound": "tensor", "achieved": solve_ach,
+                         "peak": tc_peak, "unit": "TFLOP/s", "frac": solve_ach / tc_peak,
                          "traffic": measured_traffic("scatter_split_kernel", nv * na),
-                         "peak_source": "FP32 FFMA: %d SMs x 128 lanes x 2 x max SM clock" % sm_count()},
+                         "peak_source": pk["_source"]},
             "phases": phases,
             "forward_scatter_tflops": fwd_flops / (ms_fwd * 1e-3) / 1e12,
             "misfit": L, "grad_max": {"mua": float(np.abs(ga).max()), "mus": float(np.abs(gs).max())},
@@ -493,10 +493,12 @@ def iteration_bound(flops, nbytes, ms, c_bound, c_ach, c_peak, hbm):
     return "hbm", m_ach, hbm, "GB/s", extra
 
 
-def kernel_roofline(nv, na, na_s, kms, kp, k_mean, precision, pk, exact=None):
+def kernel_roofline(nv, na, na_s, kms, kp, k_mean, precision, pk, exact=None, split=False):
     """Per-kernel times (ms per step) and the roofline object of the dominant kernel from
     ``kp`` profiled steps (``kms``: summed ms of sweep, source function, tallies).
-    ``exact``: None (the source iteration), "tc" or "simt" (the exact solve's form)."""
+    ``exact``: None (the source iteration), "tc" or "simt" (the exact solve's form).
+    ``split``: the FP32 iteration runs on the tensor cores (48 and 192 directions), counted
+    as one product per iteration at the 16-bit rate."""
     hbm = pk["hbm_gbs"]
     sweep_bytes = nv * na * 20 + nv * 8  # I,S at two levels read (16 B), Q written (4 B); optics
     # Q, S(n-1), S(n-2) read (the extrapolated start), I and S written; optics
@@ -518,7 +520,7 @@ def kernel_roofline(nv, na, na_s, kms, kp, k_mean, precision, pk, exact=None):
                  "tensor_frac_of_tf32": tc_tf / tf32_peak,
                  "tf32_peak": "%.0f TFLOP/s (measured BF16 burst x 1.1/2.25 nominal ratio)" % tf32_peak}
     else:
-        if precision == "bf16" and not exact:
+        if (precision == "bf16" or split) and not exact:
             s_bound, s_peak = "tensor", pk.get("bf16_tflops_sustained", 1700.0)
         else:
             s_bound, s_peak = "alu", fp32_peak_tflops(pk)
@@ -576,7 +578,7 @@ def measure_window(T, torch, prob, stream, spinup, warmup, steps, what, slab_tra
     na = 12 * prob["nside"] ** 2
     prec = prob.get("precision", "fp32")
     kernels, roof = kernel_roofline(nv, na, na, kms, kp, float(np.mean(k_it_mean[-kp:])), prec, peaks(),
-                                    exact=xform)
+                                    exact=xform, split=na > 12)
     # measured DRAM bytes of the dominant kernel (committed ncu table, captured on the slab,
     # while its source is unchanged); not for workloads whose kernel instances differ
     names = {"sweep": {"tma": "sweep_tma_kernel", "plain": "sweep_group_kernel"}.get(sform, "sweep2_kernel"),
@@ -622,7 +624,8 @@ def measure_whole_run(T, torch, prob, stream, steps, what, repeats=5):
     nv = prob["nx"] * prob["ny"] * prob["nz"]
     na = 12 * prob["nside"] ** 2
     prec = prob.get("precision", "fp32")
-    kernels, roof = kernel_roofline(nv, na, na, kms, steps, float(np.mean(k_it_mean)), prec, peaks())
+    kernels, roof = kernel_roofline(nv, na, na, kms, steps, float(np.mean(k_it_mean)), prec, peaks(),
+                                    split=na > 12)
     return {"workload": what, "precision": prec, "value": nv * na * steps / (best * 1e-3), "unit": "updates/s",
             "ms_per_step": best / steps, "steps": steps,
             "timing": "whole %d-step solve from step 0, best of %d (CUDA events; graph replay)" % (steps, repeats),
@@ -770,7 +773,7 @@ def main():
     per = [kms[0] / kp, kms[1] / kp, kms[2] / kp]
     tot = sum(per)
     fp32_peak = fp32_peak_tflops(pk)
-    if args.precision == "bf16" and not args.exact:
+    if not args.exact:  # BF16, or FP32 on split FP16 products (48 and 192 directions)
         s_bound, s_peak, s_unit = "tensor", pk.get("bf16_tflops_sustained", 1700.0), "TFLOP/s"
     else:
         s_bound, s_peak, s_unit = "alu", fp32_peak, "TFLOP/s"
