@@ -374,11 +374,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           *reinterpret_cast<float4*>(aLo + off) = make_float4(lo[4 * c], lo[4 * c + 1], lo[4 * c + 2], lo[4 * c + 3]);
         }
         // The raw slot is released only now: the stores above consume every value read
-        // from it, so the reads have returned.  (Released right after the loads were
-        // issued, a late load now and then read the TMA's next chunk: one or two directions
-        // of a warp's 32 voxels wrong in a few of 4608 tiles, 2e-5 of the field's norm.)
-        bar_arrive(&raw_empty[s]);
+        // from it, so the reads have returned, and the fence orders them (generic proxy)
+        // before the TMA's next write to the slot (async proxy).  Released right after the
+        // loads were issued, a late load now and then read the next chunk: one or two
+        // directions of a warp's 32 voxels wrong in a few of 4608 tiles a step, 1e-4 of the
+        // field's norm after eight steps.
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        bar_arrive(&raw_empty[s]);
         bar_arrive(&a_full[so]);
       }
     }
