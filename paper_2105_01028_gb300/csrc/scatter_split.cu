@@ -86,6 +86,8 @@ struct Sp {
   static constexpr int ROFF = POW2;                // residual / second accumulator
   static constexpr bool kRing = NA >= 192;         // Pl streamed through a ring
   static constexpr int kBlkRows = 96;
+  static constexpr int kBlkN = kRing ? kBlkRows : NA;  // N of the second accumulator's MMAs
+  static constexpr int kHalves = NA / kBlkN;
   static constexpr int kBlkBytes = kBlkRows * 128;
   static constexpr int kNblk = kRing ? KB * (NA / kBlkRows) : 1;
   static constexpr int kSlots = 3;
@@ -103,7 +105,7 @@ struct Sp {
   static constexpr int SMEM = OFF_CLS + ((NA + 15) / 16) * 16 + 1024;
   static constexpr uint32_t IDESC_ANY = (1u << 4) | (static_cast<uint32_t>(kM >> 4) << 24);  // FP16 x FP16 -> FP32
   static constexpr uint32_t IDESC = IDESC_ANY | (static_cast<uint32_t>(NA >> 3) << 17);
-  static constexpr uint32_t IDESC_BLK = IDESC_ANY | (static_cast<uint32_t>(kBlkRows >> 3) << 17);
+  static constexpr uint32_t IDESC_BLK = IDESC_ANY | (static_cast<uint32_t>(kBlkN >> 3) << 17);
 };
 
 __device__ __forceinline__ float pow2f(int e) { return __uint_as_float(static_cast<uint32_t>(127 + e) << 23); }
@@ -391,16 +393,20 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
 #pragma unroll
     for (int s = 0; s < C::KSTEPS; ++s) {
       const uint32_t ko = static_cast<uint32_t>((s & 3) * 32), kb = static_cast<uint32_t>(s >> 2);
-      const uint64_t pd = sw128_desc(aPh + kb * NA * 128 + ko);
-      mma_f16(tmem, sw128_desc(aXh + kb * kM * 128 + ko), pd, C::IDESC, s > 0);
-      mma_f16(tmem + C::ROFF, sw128_desc(aXl + kb * kM * 128 + ko), pd, C::IDESC, (C::kRing || s > 0) ? 1u : 0u);
+      mma_f16(tmem, sw128_desc(aXh + kb * kM * 128 + ko), sw128_desc(aPh + kb * NA * 128 + ko), C::IDESC, s > 0);
+      // the second accumulator is built by MMAs of one shape: only these are executed in the
+      // order of their issue (96 rows are twelve swizzle atoms, so a half starts on one)
+#pragma unroll
+      for (int h = 0; h < C::kHalves; ++h)
+        mma_f16(tmem + C::ROFF + h * C::kBlkN, sw128_desc(aXl + kb * kM * 128 + ko),
+                sw128_desc(aPh + (kb * NA + h * C::kBlkN) * 128 + ko), C::IDESC_BLK, (C::kRing || s > 0) ? 1u : 0u);
     }
     if constexpr (!C::kRing) {
 #pragma unroll
       for (int s = 0; s < C::KSTEPS; ++s) {
         const uint32_t ko = static_cast<uint32_t>(s * 32);
-        mma_f16(tmem + C::ROFF, sw128_desc(aXh + ko), sw128_desc(aPl + ko), C::IDESC, 1u);
-        mma_f16(tmem + C::ROFF, sw128_desc(aXl + ko), sw128_desc(aPl + ko), C::IDESC, 1u);
+        mma_f16(tmem + C::ROFF, sw128_desc(aXh + ko), sw128_desc(aPl + ko), C::IDESC_BLK, 1u);
+        mma_f16(tmem + C::ROFF, sw128_desc(aXl + ko), sw128_desc(aPl + ko), C::IDESC_BLK, 1u);
       }
     } else {
       for (uint32_t q = pl_used - C::kSlots; ok && q < pl_used; ++q) {
