@@ -407,9 +407,9 @@ int lock_inputs(trinity_ctx* ctx) {
   return TRINITY_OK;
 }
 
-// Device bytes of the split phase matrix: the two operand images, diagonals and roots.
+// Device bytes of the split phase matrix: the three operand images, diagonals and roots.
 size_t split_bytes(int na) {
-  return 2 * static_cast<size_t>((na + 63) / 64) * na * 128 + 3 * static_cast<size_t>(na) * 4 + 64 * 4;
+  return 3 * static_cast<size_t>((na + 63) / 64) * na * 128 + 3 * static_cast<size_t>(na) * 4 + 64 * 4;
 }
 
 // Build the split of the phase matrix for the tensor-core iteration and upload it.
@@ -420,15 +420,15 @@ int upload_split(trinity_ctx* ctx, const std::vector<double>& P, int na, double 
   uint8_t* p = buf.data();
   const size_t op = im.ph.size() * 2, dg = im.diag.size() * 4, cw = im.cw.size() * 4;
   std::memcpy(p, im.ph.data(), op);
-  std::memcpy(p + op, im.pl.data(), op);
-  std::memcpy(p + 2 * op, im.diag.data(), dg);
-  std::memcpy(p + 2 * op + dg, im.cw.data(), cw);
+  std::memcpy(p + op, im.pl.data(), 2 * op);
+  std::memcpy(p + 3 * op, im.diag.data(), dg);
+  std::memcpy(p + 3 * op + dg, im.cw.data(), cw);
   CK(cudaMemcpy(ctx->d_split, p, buf.size(), cudaMemcpyHostToDevice));
   SplitTables t = ctx->sp;
   t.ph = ctx->d_split;
   t.pl = ctx->d_split + op;
-  t.diag = reinterpret_cast<const float*>(ctx->d_split + 2 * op);
-  t.cw = reinterpret_cast<const float*>(ctx->d_split + 2 * op + dg);
+  t.diag = reinterpret_cast<const float*>(ctx->d_split + 3 * op);
+  t.cw = reinterpret_cast<const float*>(ctx->d_split + 3 * op + dg);
   t.unit = im.unit;
   t.cycle = im.cycle;
   t.max_inner = im.max_inner;

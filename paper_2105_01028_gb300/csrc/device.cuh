@@ -231,14 +231,14 @@ cudaError_t launch_interface(int nvox, int na, const int* vox, const int* rowptr
 // FP32 source iteration on the tensor cores (scatter_split.cu): the phase matrix split into
 // FP16 operands, on the host and on the device.
 struct SplitImage {
-  std::vector<uint16_t> ph, pl;  // operand images
+  std::vector<uint16_t> ph, pl;  // operand images; pl: Pm, then Pl
   std::vector<float> diag;       // [3][na] diagonal: high, low; of the inner operator
   std::vector<float> cw;         // [64] Chebyshev roots of the inner iteration
   int cycle, max_inner;
   float unit, lam, lo;
 };
 struct SplitTables {
-  const uint8_t *ph, *pl;
+  const uint8_t *ph, *pl;  // pl: Pm, then Pl
   const float *diag, *cw;
   const float* dyn;  // unit, lam, lo on the device, or null: the values below
   int cycle, max_inner;

@@ -34,7 +34,7 @@ struct NoAllocScratch {
   float rho[kNoAllocMaxVoxels];  // per-voxel contraction bound (1 - eps) max_d b1
   // the caller's P, split for the tensor cores (48 and 192 directions; see scatter_split.cu)
   alignas(128) uint16_t ph[3 * 192 * 64];
-  alignas(128) uint16_t pl[3 * 192 * 64];
+  alignas(128) uint16_t pl[2 * 3 * 192 * 64];  // Pm, then Pl
   float diag[3 * 192];
   float cw[64];
   float dyn[4];        // unit, Chebyshev interval
@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(1024) noalloc_split_prep(const float* __restri
   constexpr int kW = 32;                    // warps
   constexpr int kC = (NA + 31) / 32;        // columns per lane
   constexpr int kR = (NA + kW - 1) / kW;    // rows per warp
+  constexpr int kKb = (NA + 63) / 64;       // K blocks of the operand images
   __shared__ float x_s[kC * 32], y_s[kC * 32];
   __shared__ float red_s[kW], red2_s[kW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -136,36 +137,38 @@ __global__ void __launch_bounds__(1024) noalloc_split_prep(const float* __restri
     int t = 0;
     while (t < 20 && ldexpf(pm, t + 1) <= 2046.0f && ldexpf(rm, t + 1) + NA / 2 <= 16128.0f) ++t;
     const float whole = floorf(ldexpf(pm, t));
-    const float unit = whole >= 1.0f ? pm / whole : ldexpf(1.0f, -t);
-    const float inv = 1.0f / unit;
+    const float unit = (whole >= 1.0f ? pm / whole : ldexpf(1.0f, -t)) * 0.0625f;
+    const double inv = 1.0 / static_cast<double>(unit);
     if (warp < 8) {
       const int i = (blockIdx.x - 1) * 8 + warp;
-      float sh = 0.0f, sl = 0.0f;  // sums of whole numbers and of multiples of 2^-12: exact
+      double sh = 0.0, sum = 0.0;
 #pragma unroll
       for (int c = 0; c < kC; ++c) {
         const int j = lane + 32 * c;
         if (j >= NA) break;
-        const float u = j != i ? __ldg(P + static_cast<size_t>(j) * NA + i) : 0.0f;
-        const float h = rintf(u * inv);
-        const float l = rintf(fmaf(-h, unit, u) * inv * 4096.0f) * (1.0f / 4096.0f);
+        const double u = j != i ? __ldg(P + static_cast<size_t>(j) * NA + i) : 0.0f;
+        const double uu = u * inv, h = 16.0 * rint(uu * 0.0625);
+        const __half l = __double2half(uu - h);
+        const __half m = __double2half(uu - h - static_cast<double>(__half2float(l)));
         sh += h;
-        sl += l;
+        sum += u;
         const int k = j >> 6, ch = (j & 63) >> 3;
         const int in_row = ((ch ^ (i & 7)) << 3) + (j & 7);
         const int prow = NA >= 192 ? (k * (NA / 96) + i / 96) * 96 + i % 96 : k * NA + i;
-        sc->ph[(k * NA + i) * 64 + in_row] = __half_as_ushort(__float2half_rn(h));
-        sc->pl[prow * 64 + in_row] = __half_as_ushort(__float2half_rn(l));
+        sc->ph[(k * NA + i) * 64 + in_row] = __half_as_ushort(__double2half(h));
+        sc->pl[prow * 64 + in_row] = __half_as_ushort(m);
+        sc->pl[(kKb * NA + prow) * 64 + in_row] = __half_as_ushort(l);
       }
 #pragma unroll
       for (int o = 16; o >= 1; o >>= 1) {
         sh += __shfl_xor_sync(0xffffffffu, sh, o);
-        sl += __shfl_xor_sync(0xffffffffu, sl, o);
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
       }
       if (lane == 0) {
-        const double d = 1.0 - (static_cast<double>(sh) + sl) * unit;
+        const double d = 1.0 - sum;
         sc->diag[i] = static_cast<float>(d);
         sc->diag[NA + i] = static_cast<float>(d - static_cast<double>(static_cast<float>(d)));
-        sc->diag[2 * NA + i] = static_cast<float>(1.0 - static_cast<double>(sh) * unit);
+        sc->diag[2 * NA + i] = static_cast<float>(1.0 - sh * unit);
       }
     }
     if (blockIdx.x == 1 && tid == 0) sc->dyn[0] = unit;

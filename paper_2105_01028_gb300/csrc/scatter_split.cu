@@ -17,15 +17,20 @@
 // is below the tolerance (two outers per voxel and step on a developed slab).
 //
 // FP32-accurate product.  The diagonal of P~ is applied in FP32 (it holds half a row's
-// weight at g = 0.9); the off-diagonal part, in units of about 2^-t, is split as Ph + Pl with
-// Ph whole numbers of at most 11 bits and Pl multiples of 2^-12, X, scaled per voxel by a
-// power of two, as Xh + Xl likewise (Xh below 2^10).  t is chosen so that every partial sum
+// weight at g = 0.9); the off-diagonal part, in units of about 2^-t, is split as Ph + Pl + Pm
+// with Ph whole numbers of at most 11 bits, Pl the FP16 number nearest to the rest and Pm that
+// nearest to what is left (the entries of a peaked kernel span a factor of 500, and the smallest
+// are two units: with Ph and Pl alone they are off by 5e-5 of themselves, and all that a
+// detector beside the source sees first went through them).  X, scaled per voxel by a
+// power of two, is split as Xh + Xl, Xh whole below 2^10 and Xl multiples of 2^-12.  t is
+// chosen so that every partial sum
 // of Xh Ph stays below 2^24: the FP32 accumulator in TMEM then holds it exactly, whatever
 // the order, and its truncation (the tensor core does not round an accumulation to
 // nearest: three TF32 products summed in one accumulator are 1.7e-6 off, one-sided) has
-// nothing to act on.  Xl Ph + Xh Pl + Xl Pl goes to a second accumulator, 2^-10 of the
+// nothing to act on.  Xh Pm + Xl Pl + Xh Pl + Xl Ph goes to a second accumulator, 2^-10 of the
 // first in size, where the truncation is below 2^-32 of the result.  Each row of
-// Ph + Pl + diag sums to one (the diagonal is a float pair), so photons are conserved.
+// Ph + Pl + Pm + diag sums to one (the diagonal is a float pair; what the terms drop is 1e-10 of
+// the row), so photons are conserved.
 // Measured against FP64 on the 96x96x64 slab: 1.0e-7 in 2-norm of I and S after two steps;
 // the sum of 192 FP32 products on the CUDA cores that it replaces: 2.3e-7.  Two steps of that
 // slab at 192 directions: 5.8 ms (152 ms before); 100 steps of 16^3 at 48 directions: 5.7 ms
@@ -44,8 +49,8 @@
 // column groups of 48 directions (three of 16 at 48 directions).  TMEM: D / first
 // accumulator in [0, N_a), r / second accumulator in [256, 256 + N_a) and, at 192
 // directions, two thirds of Q in the columns left over; S stays in registers.  Shared
-// memory at 192 directions: Ph 72 KB, Xh and Xl 48 KB each; Pl (72 KB) does not fit beside
-// them and is streamed from L2 in six 12 KB blocks through a ring of three.
+// memory at 192 directions: Ph 72 KB, Xh and Xl 48 KB each; Pm and Pl (72 KB each) do not fit
+// beside them and are streamed from L2 in twelve 12 KB blocks through a ring of three.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -89,7 +94,7 @@ struct Sp {
   static constexpr int kBlkN = kRing ? kBlkRows : NA;  // N of the second accumulator's MMAs
   static constexpr int kHalves = NA / kBlkN;
   static constexpr int kBlkBytes = kBlkRows * 128;
-  static constexpr int kNblk = kRing ? KB * (NA / kBlkRows) : 1;
+  static constexpr int kNblk = kRing ? 2 * KB * (NA / kBlkRows) : 1;  // blocks of Pm, then of Pl
   static constexpr int kSlots = 3;
   static constexpr int P_BYTES = KB * NA * 128;
   static constexpr int A_BYTES = KB * kM * 128;
@@ -97,7 +102,8 @@ struct Sp {
   static constexpr int OFF_XH = (P_BYTES + 1023) / 1024 * 1024;
   static constexpr int OFF_XL = OFF_XH + A_BYTES;
   static constexpr int OFF_PL = OFF_XL + A_BYTES;
-  static constexpr int PL_BYTES = kRing ? kSlots * kBlkBytes : (P_BYTES + 1023) / 1024 * 1024;
+  static constexpr int PL_BYTES = kRing ? kSlots * kBlkBytes : 2 * P_BYTES;  // ring, or Pm and then Pl
+  static_assert(P_BYTES % 1024 == 0, "operand images follow one another");
   static constexpr int OFF_B1T = OFF_PL + PL_BYTES;                // [kMaxClasses][kM] f32
   static constexpr int OFF_DI = OFF_B1T + kMaxClasses * kM * 4;    // [3][NA] f32: diagonals
   static constexpr int OFF_B1C = OFF_DI + 3 * NA * 4;              // [NA] f32 (uniform mu_t)
@@ -242,7 +248,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
   for (int u = tid; u < C::P_BYTES / 16; u += blockDim.x)
     reinterpret_cast<uint4*>(sPh)[u] = __ldg(reinterpret_cast<const uint4*>(t.ph) + u);
   if constexpr (!C::kRing) {
-    for (int u = tid; u < C::P_BYTES / 16; u += blockDim.x)
+    for (int u = tid; u < C::PL_BYTES / 16; u += blockDim.x)
       reinterpret_cast<uint4*>(sPl)[u] = __ldg(reinterpret_cast<const uint4*>(t.pl) + u);
   }
   if (tid < kMaxClasses) ccnt_s[tid] = 0;
@@ -367,54 +373,81 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
   const auto issue_product = [&]() {
     tc_fence_after();
     bool ok = true;
-    // Pl block b (K block b / 2, output directions 96 (b & 1) .. + 95) into the second
-    // accumulator, from ring slot pl_used % kSlots
-    const auto pl_block = [&](int b) {
-      const uint32_t sl = pl_used % C::kSlots;
-      if (ok) ok = mbar_wait_bounded(&pl_full[sl], (pl_used / C::kSlots) & 1u);
-      if (!ok) return;
-      tc_fence_after();
-      const uint32_t kb = static_cast<uint32_t>(b >> 1), d = tmem + C::ROFF + (b & 1) * C::kBlkRows;
+    const auto xl_ph = [&]() {
 #pragma unroll
-      for (int ks = 0; ks < 4; ++ks) {
-        const uint64_t pd = sw128_desc(aPl + sl * C::kBlkBytes + ks * 32);
-        mma_f16(d, sw128_desc(aXh + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, (b > 1 || ks > 0) ? 1u : 0u);
-        mma_f16(d, sw128_desc(aXl + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, 1u);
+      for (int s = 0; s < C::KSTEPS; ++s) {
+        const uint32_t ko = static_cast<uint32_t>((s & 3) * 32), kb = static_cast<uint32_t>(s >> 2);
+        // the second accumulator is built by MMAs of one shape: only these are executed in the
+        // order of their issue (96 rows are twelve swizzle atoms, so a half starts on one)
+#pragma unroll
+        for (int h = 0; h < C::kHalves; ++h)
+          mma_f16(tmem + C::ROFF + h * C::kBlkN, sw128_desc(aXl + kb * kM * 128 + ko),
+                  sw128_desc(aPh + (kb * NA + h * C::kBlkN) * 128 + ko), C::IDESC_BLK, 1u);
       }
-      mma_commit(&pl_empty[sl]);
-      ++pl_used;
+    };
+    const auto xh_ph = [&](int from, int to) {
+#pragma unroll
+      for (int s = from; s < to; ++s) {
+        const uint32_t ko = static_cast<uint32_t>((s & 3) * 32), kb = static_cast<uint32_t>(s >> 2);
+        mma_f16(tmem, sw128_desc(aXh + kb * kM * 128 + ko), sw128_desc(aPh + kb * NA * 128 + ko), C::IDESC, s > 0);
+      }
     };
     if constexpr (C::kRing) {
-      // the blocks that are there go first: the others take their slots while the Ph MMAs run
-      static_assert(C::kNblk == 2 * C::kSlots, "the second half of the blocks refills the ring once");
+      // Block b of Pm (b < 6, with Xh alone) or Pl: K block (b % 6) / 2, output directions
+      // 96 (b & 1) .. + 95, into the second accumulator, from ring slot pl_used % kSlots
+      const auto pl_blocks = [&](int b0) {
 #pragma unroll 1
-      for (int b = 0; b < C::kSlots; ++b) pl_block(b);
-    }
+        for (int b = b0; b < b0 + C::kSlots; ++b) {
+          const uint32_t sl = pl_used % C::kSlots;
+          if (ok) ok = mbar_wait_bounded(&pl_full[sl], (pl_used / C::kSlots) & 1u);
+          if (!ok) return;
+          tc_fence_after();
+          const bool low = b < C::kNblk / 2;
+          const uint32_t kb = static_cast<uint32_t>((low ? b : b - C::kNblk / 2) >> 1);
+          const uint32_t d = tmem + C::ROFF + (b & 1) * C::kBlkRows;
 #pragma unroll
-    for (int s = 0; s < C::KSTEPS; ++s) {
-      const uint32_t ko = static_cast<uint32_t>((s & 3) * 32), kb = static_cast<uint32_t>(s >> 2);
-      mma_f16(tmem, sw128_desc(aXh + kb * kM * 128 + ko), sw128_desc(aPh + kb * NA * 128 + ko), C::IDESC, s > 0);
-      // the second accumulator is built by MMAs of one shape: only these are executed in the
-      // order of their issue (96 rows are twelve swizzle atoms, so a half starts on one)
-#pragma unroll
-      for (int h = 0; h < C::kHalves; ++h)
-        mma_f16(tmem + C::ROFF + h * C::kBlkN, sw128_desc(aXl + kb * kM * 128 + ko),
-                sw128_desc(aPh + (kb * NA + h * C::kBlkN) * 128 + ko), C::IDESC_BLK, (C::kRing || s > 0) ? 1u : 0u);
-    }
-    if constexpr (!C::kRing) {
+          for (int ks = 0; ks < 4; ++ks) {
+            const uint64_t pd = sw128_desc(aPl + sl * C::kBlkBytes + ks * 32);
+            if (!low) mma_f16(d, sw128_desc(aXl + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, 1u);
+            mma_f16(d, sw128_desc(aXh + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, (b > 1 || ks > 0) ? 1u : 0u);
+          }
+          mma_commit(&pl_empty[sl]);
+          ++pl_used;
+        }
+      };
+      const auto refill = [&]() {  // the slots just used take the next blocks once their MMAs are done
+        for (uint32_t q = pl_used - C::kSlots; ok && q < pl_used; ++q) {
+          ok = mbar_wait_bounded(&pl_empty[q % C::kSlots], (q / C::kSlots) & 1u);
+          if (ok) pl_load();
+        }
+      };
+      // the ring is refilled while the MMAs on Ph between two groups of blocks run
+      static_assert(C::kNblk == 4 * C::kSlots, "a product takes the ring four times");
+      pl_blocks(0);
+      xl_ph();
+      refill();
+      pl_blocks(C::kSlots);
+      xh_ph(0, C::KSTEPS / 2);
+      refill();
+      pl_blocks(2 * C::kSlots);
+      xh_ph(C::KSTEPS / 2, C::KSTEPS);
+      refill();
+      pl_blocks(3 * C::kSlots);
+    } else {
+      // terms in order of size, the small ones first
 #pragma unroll
       for (int s = 0; s < C::KSTEPS; ++s) {
         const uint32_t ko = static_cast<uint32_t>(s * 32);
-        mma_f16(tmem + C::ROFF, sw128_desc(aXh + ko), sw128_desc(aPl + ko), C::IDESC_BLK, 1u);
-        mma_f16(tmem + C::ROFF, sw128_desc(aXl + ko), sw128_desc(aPl + ko), C::IDESC_BLK, 1u);
+        mma_f16(tmem + C::ROFF, sw128_desc(aXh + ko), sw128_desc(aPl + ko), C::IDESC_BLK, s > 0);
       }
-    } else {
-      for (uint32_t q = pl_used - C::kSlots; ok && q < pl_used; ++q) {
-        ok = mbar_wait_bounded(&pl_empty[q % C::kSlots], (q / C::kSlots) & 1u);
-        if (ok) pl_load();
+#pragma unroll
+      for (int s = 0; s < C::KSTEPS; ++s) {
+        const uint32_t ko = static_cast<uint32_t>(s * 32);
+        mma_f16(tmem + C::ROFF, sw128_desc(aXl + ko), sw128_desc(aPl + C::P_BYTES + ko), C::IDESC_BLK, 1u);
+        mma_f16(tmem + C::ROFF, sw128_desc(aXh + ko), sw128_desc(aPl + C::P_BYTES + ko), C::IDESC_BLK, 1u);
       }
-#pragma unroll 1
-      for (int b = C::kSlots; b < C::kNblk; ++b) pl_block(b);
+      xl_ph();
+      xh_ph(0, C::KSTEPS);
     }
     mma_commit(&mbar);
     if (!ok) abort_s = 1;
@@ -1019,11 +1052,17 @@ cudaError_t launch_split(const GridParams& g, const SplitTables& sp, const BfTab
   return cudaGetLastError();
 }
 
-uint16_t half_bits(double x) {  // x is an FP16 number
-  const __half h = __float2half(static_cast<float>(x));
+uint16_t half_bits(double x) {  // nearest FP16 number
+  const __half h = __double2half(x);
   uint16_t u;
   std::memcpy(&u, &h, 2);
   return u;
+}
+
+double half_value(uint16_t u) {
+  __half h;
+  std::memcpy(&h, &u, 2);
+  return static_cast<double>(__half2float(h));
 }
 
 }  // namespace
@@ -1044,10 +1083,10 @@ bool scatter_split_supported(int na, int ncls) {
   return true;
 }
 
-// Off-diagonal part of the FP64 phase matrix P split as (Ph + Pl) unit, in the kernel's operand layout: Ph
-// [K block][na rows][128 B], Pl likewise at 48 directions and as six blocks (K block, half
-// of the rows) of 96 rows at 192; diag: the FP32 pair that makes each row of Ph + Pl + diag
-// sum to one, and the diagonal that does so with Ph alone.
+// Off-diagonal part of the FP64 phase matrix P split as (Ph + Pl + Pm) unit, in the kernel's
+// operand layout: Ph [K block][na rows][128 B]; Pm and then Pl likewise at 48 directions, as
+// six blocks each (K block, half of the rows) of 96 rows at 192; diag: the FP32 pair that
+// makes each row of P with it sum to one, and the diagonal that does so with Ph alone.
 SplitImage scatter_split_image(const std::vector<double>& P, int na, double g_aniso) {
   SplitImage im;
   const int kb = (na + 63) / 64;
@@ -1069,30 +1108,34 @@ SplitImage scatter_split_image(const std::vector<double>& P, int na, double g_an
   // one unit of Ph: 2^-t made so that the largest entry is a whole number of units (an
   // isotropic P is then split exactly; its equal entries would else all err to one side)
   const double whole = std::floor(std::ldexp(pmax, t));
-  im.unit = static_cast<float>(whole >= 1.0 ? pmax / whole : std::ldexp(1.0, -t));
+  // (held sixteenfold: the terms below then stay clear of FP16's subnormals)
+  im.unit = static_cast<float>(whole >= 1.0 ? pmax / whole : std::ldexp(1.0, -t)) / 16.0f;
   const double unit = im.unit;
-  im.ph.assign(static_cast<size_t>(kb) * na * 64, 0);
-  im.pl.assign(static_cast<size_t>(kb) * na * 64, 0);
+  const size_t half = static_cast<size_t>(kb) * na * 64;
+  im.ph.assign(half, 0);
+  im.pl.assign(2 * half, 0);
   im.diag.assign(static_cast<size_t>(3) * na, 0.0f);
   const int blk = 96;
   for (int i = 0; i < na; ++i) {
-    double sh = 0.0, sl = 0.0;
+    double sh = 0.0, sum = 0.0;
     for (int j = 0; j < na; ++j) {
       if (j == i) continue;
       const double u = P[static_cast<size_t>(i) * na + j] / unit;
-      const double h = std::nearbyint(u);
-      const double l = std::nearbyint((u - h) * 4096.0) / 4096.0;
+      const double h = 16.0 * std::nearbyint(u / 16.0);
+      const uint16_t lb = half_bits(u - h);
+      const uint16_t mb = half_bits(u - h - half_value(lb));
       sh += h;
-      sl += l;
+      sum += P[static_cast<size_t>(i) * na + j];
       const int k = j >> 6, ch = (j & 63) >> 3;
       const size_t in_row = static_cast<size_t>(((ch ^ (i & 7)) << 3) + (j & 7));
       im.ph[(static_cast<size_t>(k) * na + i) * 64 + in_row] = half_bits(h);
       // 96 is a multiple of 8, so a block's rows keep the swizzle phase i & 7
       const size_t prow = na >= 192 ? static_cast<size_t>(k * (na / blk) + i / blk) * blk + i % blk
                                     : static_cast<size_t>(k) * na + i;
-      im.pl[prow * 64 + in_row] = half_bits(l);
+      im.pl[prow * 64 + in_row] = mb;
+      im.pl[half + prow * 64 + in_row] = lb;
     }
-    const double d = 1.0 - (sh + sl) * unit;
+    const double d = 1.0 - sum;
     im.diag[i] = static_cast<float>(d);
     im.diag[na + i] = static_cast<float>(d - static_cast<double>(im.diag[i]));
     im.diag[2 * na + i] = static_cast<float>(1.0 - sh * unit);
