@@ -21,14 +21,16 @@
 // with Ph whole numbers of at most 11 bits, Pl the FP16 number nearest to the rest and Pm that
 // nearest to what is left (the entries of a peaked kernel span a factor of 500, and the smallest
 // are two units: with Ph and Pl alone they are off by 5e-5 of themselves, and all that a
-// detector beside the source sees first went through them).  X, scaled per voxel by a
-// power of two, is split as Xh + Xl, Xh whole below 2^10 and Xl multiples of 2^-12.  t is
-// chosen so that every partial sum
-// of Xh Ph stays below 2^24: the FP32 accumulator in TMEM then holds it exactly, whatever
-// the order, and its truncation (the tensor core does not round an accumulation to
-// nearest: three TF32 products summed in one accumulator are 1.7e-6 off, one-sided) has
-// nothing to act on.  Xh Pm + Xl Pl + Xh Pl + Xl Ph goes to a second accumulator, 2^-10 of the
-// first in size, where the truncation is below 2^-32 of the result.  Each row of
+// detector beside the source sees first went through them).  X, scaled per voxel by a power of
+// two, is split as Xh + Xl + Xm, Xh whole below 2^10, Xl multiples of 2^-12 and Xm the rest (where
+// one direction outshines the others 1e4 times, Xh + Xl leaves the weak outgoing directions
+// 1.7e-4 off; with Xm they are 5e-7 off at most, a sum of 192 FP32 products 2e-6).  t is
+// chosen so that every partial sum of Xh Ph stays below 2^24: the FP32 accumulator in TMEM then
+// holds it exactly, whatever the order, and its truncation (the tensor core does not round an
+// accumulation to nearest: three TF32 products summed in one accumulator are 1.7e-6 off,
+// one-sided) has nothing to act on.  Xm Ph + Xh Pm + Xl Pl + Xh Pl + Xl Ph goes to a second
+// accumulator, 2^-10 of the first in size, where the truncation is below 2^-32 of the result
+// (3e-8 of it in the weak directions above).  Each row of
 // Ph + Pl + Pm + diag sums to one (the diagonal is a float pair; what the terms drop is 1e-10 of
 // the row), so photons are conserved.
 // Measured against FP64 on the 96x96x64 slab: 1.0e-7 in 2-norm of I and S after two steps;
@@ -50,7 +52,8 @@
 // accumulator in [0, N_a), r / second accumulator in [256, 256 + N_a) and, at 192
 // directions, two thirds of Q in the columns left over; S stays in registers.  Shared
 // memory at 192 directions: Ph 72 KB, Xh and Xl 48 KB each; Pm and Pl (72 KB each) do not fit
-// beside them and are streamed from L2 in twelve 12 KB blocks through a ring of three.
+// beside them and are streamed from L2 in twelve 12 KB blocks through a ring of three, and Xl
+// takes the place of Xm when the MMAs on Xm are done (written under the next ones).
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -59,6 +62,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "device.cuh"
@@ -101,7 +105,8 @@ struct Sp {
   static constexpr int OFF_PH = 0;
   static constexpr int OFF_XH = (P_BYTES + 1023) / 1024 * 1024;
   static constexpr int OFF_XL = OFF_XH + A_BYTES;
-  static constexpr int OFF_PL = OFF_XL + A_BYTES;
+  static constexpr int OFF_XM = kRing ? OFF_XL : OFF_XL + A_BYTES;  // (ring: Xm and Xl take turns)
+  static constexpr int OFF_PL = OFF_XM + A_BYTES;
   static constexpr int PL_BYTES = kRing ? kSlots * kBlkBytes : 2 * P_BYTES;  // ring, or Pm and then Pl
   static_assert(P_BYTES % 1024 == 0, "operand images follow one another");
   static constexpr int OFF_B1T = OFF_PL + PL_BYTES;                // [kMaxClasses][kM] f32
@@ -129,17 +134,14 @@ __device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// u (|u| < 2^11) = h + l: h the nearest whole number, l the rest to multiples of 2^-12 with
-// the rounding error of the elements before it carried along.  The errors of a row then sum
-// to less than one unit: rounded each on its own, they are noise in the row's photon number
-// (1e-6 of the source function where one direction outshines the others eight times), the
-// mode that the scattering amplifies.  The magic additions round to nearest even at bit 0
-// and bit -12; every other step is exact.
-__device__ __forceinline__ void split_u(float u, float& carry, float& h, float& l) {
-  h = (u + 12582912.0f) - 12582912.0f;
-  const float d = (u - h) + carry;
-  l = (d + 3072.0f) - 3072.0f;
-  carry = d - l;
+// u (|u| < 2^14) = h + l + m: h the nearest multiple of 16, l the rest to multiples of 2^-8,
+// m what is left (the magic additions round to nearest even at bits 4 and -8; every other step
+// is exact, and m is rounded when it is packed: 2^-35 of the row's largest element).
+__device__ __forceinline__ void split_u(float u, float& h, float& l, float& m) {
+  h = (u + 201326592.0f) - 201326592.0f;
+  const float d = u - h;
+  l = (d + 49152.0f) - 49152.0f;
+  m = d - l;
 }
 
 __device__ __forceinline__ void bulk_to_smem(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -173,6 +175,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
   uint8_t* sPh = smem + C::OFF_PH;
   uint8_t* sXh = smem + C::OFF_XH;
   uint8_t* sXl = smem + C::OFF_XL;
+  uint8_t* sXm = smem + C::OFF_XM;
   uint8_t* sPl = smem + C::OFF_PL;
   float* b1t = reinterpret_cast<float*>(smem + C::OFF_B1T);
   float* sDi = reinterpret_cast<float*>(smem + C::OFF_DI);  // diagonal of P~ (hi), (lo); of the inner operator
@@ -288,7 +291,8 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
   const uint32_t t_row = tmem + (static_cast<uint32_t>((warp & 3) << 5) << 16);
   // this thread's Q columns in TMEM (column group h: N_a + 32 h for h < 2, ROFF + N_a + 32 (h - 2))
   const uint32_t t_q = t_row + static_cast<uint32_t>(grp < 2 ? NA + C::QT * grp : C::ROFF + NA + C::QT * (grp - 2));
-  const uint32_t aXh = smem_u32(sXh), aXl = smem_u32(sXl), aPh = smem_u32(sPh), aPl = smem_u32(sPl);
+  const uint32_t aXh = smem_u32(sXh), aXl = smem_u32(sXl), aXm = smem_u32(sXm);
+  const uint32_t aPh = smem_u32(sPh), aPl = smem_u32(sPl);
   uint32_t phase = 0;
   bool aborted = false;
   double esum = 0.0;
@@ -369,20 +373,32 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
     tc_fence_after();
     return !to;
   };
-  // thread 0: the two accumulators of an FP32-accurate product
-  const auto issue_product = [&]() {
+  // thread 0: the ring slots just used take the next blocks once their MMAs are done
+  const auto pl_refill = [&]() {
+    bool ok = true;
+    for (uint32_t q = pl_used - C::kSlots; ok && q < pl_used; ++q) {
+      ok = mbar_wait_bounded(&pl_empty[q % C::kSlots], (q / C::kSlots) & 1u);
+      if (ok) pl_load();
+    }
+    return ok;
+  };
+  // thread 0: the two accumulators of an FP32-accurate product.  kHead: the part that needs Xh
+  // and Xm, the rest waits for Xl (at 48 directions all three are there and the head is all)
+  const auto issue_product = [&](auto head) {
+    [[maybe_unused]] constexpr bool kHead = decltype(head)::value;
     tc_fence_after();
     bool ok = true;
-    const auto xl_ph = [&]() {
+    // K steps [from, to) of an X term times Ph into the second accumulator, which is built by
+    // MMAs of one shape: only these are executed in the order of their issue (96 rows are
+    // twelve swizzle atoms, so a half starts on one)
+    const auto low_ph = [&](uint32_t ax, int from, int to, bool first) {
 #pragma unroll
-      for (int s = 0; s < C::KSTEPS; ++s) {
+      for (int s = from; s < to; ++s) {
         const uint32_t ko = static_cast<uint32_t>((s & 3) * 32), kb = static_cast<uint32_t>(s >> 2);
-        // the second accumulator is built by MMAs of one shape: only these are executed in the
-        // order of their issue (96 rows are twelve swizzle atoms, so a half starts on one)
 #pragma unroll
         for (int h = 0; h < C::kHalves; ++h)
-          mma_f16(tmem + C::ROFF + h * C::kBlkN, sw128_desc(aXl + kb * kM * 128 + ko),
-                  sw128_desc(aPh + (kb * NA + h * C::kBlkN) * 128 + ko), C::IDESC_BLK, 1u);
+          mma_f16(tmem + C::ROFF + h * C::kBlkN, sw128_desc(ax + kb * kM * 128 + ko),
+                  sw128_desc(aPh + (kb * NA + h * C::kBlkN) * 128 + ko), C::IDESC_BLK, (first && s == 0) ? 0u : 1u);
       }
     };
     const auto xh_ph = [&](int from, int to) {
@@ -409,44 +425,45 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
           for (int ks = 0; ks < 4; ++ks) {
             const uint64_t pd = sw128_desc(aPl + sl * C::kBlkBytes + ks * 32);
             if (!low) mma_f16(d, sw128_desc(aXl + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, 1u);
-            mma_f16(d, sw128_desc(aXh + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, (b > 1 || ks > 0) ? 1u : 0u);
+            mma_f16(d, sw128_desc(aXh + kb * kM * 128 + ks * 32), pd, C::IDESC_BLK, 1u);
           }
           mma_commit(&pl_empty[sl]);
           ++pl_used;
         }
       };
-      const auto refill = [&]() {  // the slots just used take the next blocks once their MMAs are done
-        for (uint32_t q = pl_used - C::kSlots; ok && q < pl_used; ++q) {
-          ok = mbar_wait_bounded(&pl_empty[q % C::kSlots], (q / C::kSlots) & 1u);
-          if (ok) pl_load();
-        }
-      };
-      // the ring is refilled while the MMAs on Ph between two groups of blocks run
+      // the ring is refilled while MMAs on Ph run
       static_assert(C::kNblk == 4 * C::kSlots, "a product takes the ring four times");
-      pl_blocks(0);
-      xl_ph();
-      refill();
+      if (kHead) {
+        low_ph(aXm, 0, C::KSTEPS, true);
+        mma_commit(&mbar);  // Xm is free for Xl
+        pl_blocks(0);
+        xh_ph(0, C::KSTEPS / 2);
+        if (!ok) abort_s = 1;
+        return;
+      }
+      low_ph(aXl, 0, C::KSTEPS / 2, false);
       pl_blocks(C::kSlots);
-      xh_ph(0, C::KSTEPS / 2);
-      refill();
+      low_ph(aXl, C::KSTEPS / 2, C::KSTEPS, false);
+      ok = ok && pl_refill();
       pl_blocks(2 * C::kSlots);
       xh_ph(C::KSTEPS / 2, C::KSTEPS);
-      refill();
+      ok = ok && pl_refill();
       pl_blocks(3 * C::kSlots);
     } else {
       // terms in order of size, the small ones first
+      low_ph(aXm, 0, C::KSTEPS, true);
 #pragma unroll
       for (int s = 0; s < C::KSTEPS; ++s) {
         const uint32_t ko = static_cast<uint32_t>(s * 32);
-        mma_f16(tmem + C::ROFF, sw128_desc(aXh + ko), sw128_desc(aPl + ko), C::IDESC_BLK, s > 0);
+        mma_f16(tmem + C::ROFF, sw128_desc(aXh + ko), sw128_desc(aPl + ko), C::IDESC_BLK, 1u);
+        mma_f16(tmem + C::ROFF, sw128_desc(aXl + ko), sw128_desc(aPl + C::P_BYTES + ko), C::IDESC_BLK, 1u);
       }
 #pragma unroll
       for (int s = 0; s < C::KSTEPS; ++s) {
         const uint32_t ko = static_cast<uint32_t>(s * 32);
-        mma_f16(tmem + C::ROFF, sw128_desc(aXl + ko), sw128_desc(aPl + C::P_BYTES + ko), C::IDESC_BLK, 1u);
         mma_f16(tmem + C::ROFF, sw128_desc(aXh + ko), sw128_desc(aPl + C::P_BYTES + ko), C::IDESC_BLK, 1u);
       }
-      xl_ph();
+      low_ph(aXl, 0, C::KSTEPS, false);
       xh_ph(0, C::KSTEPS);
     }
     mma_commit(&mbar);
@@ -578,35 +595,50 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
     int outer = 0;
     while (true) {
       // ---- X = Q + b1 S, split
-      const int ex = scale_exponent(row_max(red_d), 9);
+      const int ex = scale_exponent(row_max(red_d), 13);
       const float sx = pow2f(ex);
-      float carry = 0.0f;
+      // tail (ring form): Xl, after the MMAs on Xm, which has its place until then
+      const auto split_x = [&](auto tail) {
+        constexpr bool kTail = decltype(tail)::value;
 #pragma unroll
-      for (int ch = 0; ch < NCH; ++ch) {
-        const int c0 = cb + ch * CH;
-        float qv[CH], bv[8];
-        load_q(ch, qv);
-        load_w(c0, bv);
-        if (ch < NCT) tmem_wait_ld();
-        reg_q(ch, qv);
-        uint32_t hi[4], lo[4];
+        for (int ch = 0; ch < NCH; ++ch) {
+          const int c0 = cb + ch * CH;
+          float qv[CH], bv[8];
+          load_q(ch, qv);
+          load_w(c0, bv);
+          if (ch < NCT) tmem_wait_ld();
+          reg_q(ch, qv);
+          uint32_t hi[4], lo[4], lw[4];
 #pragma unroll
-        for (int j = 0; j < CH; j += 2) {
-          float h0, l0, h1, l1;
-          split_u(form_x(bv[j], S[ch * CH + j], qv[j]) * sx, carry, h0, l0);
-          split_u(form_x(bv[j + 1], S[ch * CH + j + 1], qv[j + 1]) * sx, carry, h1, l1);
-          hi[j / 2] = pack_f16x2(h0, h1);
-          lo[j / 2] = pack_f16x2(l0, l1);
+          for (int j = 0; j < CH; j += 2) {
+            float h0, l0, m0, h1, l1, m1;
+            split_u(form_x(bv[j], S[ch * CH + j], qv[j]) * sx, h0, l0, m0);
+            split_u(form_x(bv[j + 1], S[ch * CH + j + 1], qv[j + 1]) * sx, h1, l1, m1);
+            hi[j / 2] = pack_f16x2(h0, h1);
+            lo[j / 2] = pack_f16x2(l0, l1);
+            lw[j / 2] = pack_f16x2(m0, m1);
+          }
+          const uint32_t off = sw128_chunk_off(kM, row, c0);
+          if (!kTail) {
+            *reinterpret_cast<uint4*>(sXh + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<uint4*>(sXm + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+          }
+          if (kTail || !C::kRing) *reinterpret_cast<uint4*>(sXl + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         }
-        const uint32_t off = sw128_chunk_off(kM, row, c0);
-        *reinterpret_cast<uint4*>(sXh + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *reinterpret_cast<uint4*>(sXl + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-      }
-      fence_async_smem();
-      tc_fence_before();
+        fence_async_smem();
+        tc_fence_before();
+      };
+      split_x(std::false_type{});
       __syncthreads();
-      if (tid == 0) issue_product();
+      if (tid == 0) issue_product(std::true_type{});
       bool mma_ok = wait_mma();
+      if constexpr (C::kRing) {
+        split_x(std::true_type{});
+        if (tid == 0 && !pl_refill()) abort_s = 1;
+        __syncthreads();
+        if (tid == 0) issue_product(std::false_type{});
+        mma_ok = wait_mma() && mma_ok;
+      }
       if (tid == 0 && C::kRing && mma_ok) {
         // the next product's first blocks (its slots' MMAs have completed)
         while (pl_issued < pl_used + C::kSlots) pl_load();

@@ -8,11 +8,20 @@ as the call does).
 One bright direction (a power of two, so that it splits exactly) asks for a column of P: an entry
 is held to 1.5e-8 of itself by its three FP16 terms (1.2e-7 where it is below 1e-4 of the largest:
 g = -0.95), the two accumulators are added with three FP32 roundings of 2^-24: 4e-7.
+
+A row in which one direction outshines the others by up to 1e6: products of third terms that are
+left out and the accumulator's truncation are 6.5e-7 of the weakest output at most (emulated in
+FP64), four FP32 roundings 2.4e-7: 1.5e-6 is asked for (a sum of 192 FP32 products in turn:
+2.9e-6; two terms per factor: 2.8e-4).  The same through a context, in a thin medium (b1 below
+0.006, tolerance at the floor): the residual a P I - S of the stored fields in each direction,
+with the stored I and S rounded and two outer residuals' error in it: 3e-6 of S.
 """
 import ctypes
 
 import numpy as np
 import pytest
+
+import workloads as W
 
 pytestmark = pytest.mark.gpu
 
@@ -51,3 +60,40 @@ def test_every_entry_of_the_phase_matrix_counts(na, g):
     assert rc == 0
     ref = P @ Q
     assert np.all(np.abs(S - ref) <= 4e-7 * np.abs(ref))
+
+
+@pytest.mark.parametrize("na,g", [(48, 0.9), (192, 0.9), (192, 0.99)])
+@pytest.mark.parametrize("weak", [1.0, 1e-2, 1e-4, 1e-6])
+def test_weak_directions_beside_a_bright_one(na, g, weak):
+    P32, P = _matrix(na, g)
+    rng = np.random.default_rng(na)
+    nvox = 300
+    Q = (weak * rng.random((na, nvox))).astype(np.float32)
+    Q[rng.integers(0, na, nvox), np.arange(nvox)] = 1.0 - 0.4 * rng.random(nvox)
+    z = np.zeros_like(Q)
+    rc, S, _ = _buffers(P32, Q, z, np.zeros(nvox), z)
+    assert rc == 0
+    ref = P @ Q.astype(np.float64)
+    assert np.all(np.abs(S - ref) <= 1.5e-6 * np.abs(ref))
+
+
+@pytest.mark.parametrize("nside,uniform", [(2, True), (4, True), (4, False)])
+def test_weak_directions_of_a_step(nside, uniform):
+    import paper_2105_01028_gb300 as T
+    p = W.homogeneous(12, 9, 8, nside, 0.001, 0.01, g=0.9, steps=4, tol=1e-12)
+    rng = np.random.default_rng(nside)
+    if not uniform:
+        p["mus"] = (0.01 * (1.0 - 0.5 * rng.random(p["mus"].shape))).astype(np.float32)
+    p["detectors"] = []
+    fw = T.Forward(p)
+    I0 = np.repeat(1e-4 * rng.random((fw.na, 1)), fw.nv, axis=1)
+    I0[5] = 1.0
+    fw.set_initial_state(I0.astype(np.float32), np.zeros_like(I0, dtype=np.float32))
+    fw.step(1)
+    I, S = fw.field(T.FIELD_I).astype(np.float64), fw.field(T.FIELD_S).astype(np.float64)
+    fw.close()
+    P, _ = T.phase_matrix(nside, 0.9)
+    mua, mus = (p[k].astype(np.float64).ravel() for k in ("mua", "mus"))
+    ref = mus / (mua + mus) * (P @ I)
+    assert ref.min() > 0 and ref.max() > 300 * ref.min()
+    assert np.all(np.abs(ref - S) <= 3e-6 * ref)
