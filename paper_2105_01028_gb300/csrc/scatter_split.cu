@@ -77,6 +77,9 @@ constexpr float kTolShare = 0.25f;             // share of the tolerance the sto
 constexpr float kInnerError = 4.8828125e-04f;  // 2^-11: error of an inner correction, relative to it
 constexpr float kInnerDrop = 9.765625e-04f;    // 2^-10: an inner solve reduces its residual this far at most
 constexpr int kMaxOuter = 8;
+// Rows below this are held scaled up: 2^-50, so that a residual 2^-37 of the row still has its
+// full scale in scale_exponent.
+constexpr float kTiny = 8.8817841970012523e-16f;
 
 template <int NA>
 struct Sp {
@@ -123,10 +126,11 @@ __device__ __forceinline__ float pow2f(int e) { return __uint_as_float(static_ca
 __device__ __forceinline__ int exponent(float x) { return static_cast<int>((__float_as_uint(x) >> 23) & 0xffu) - 127; }
 
 // Power-of-two scale 2^e that brings a row whose largest element is m to [2^top, 2^(top+1)),
-// kept within the range where 2^-(e + 24) is a normal float.
+// kept within the range where 2^-(e + 24) is a normal float (kTiny sees to it that this does not
+// bind).
 __device__ __forceinline__ int scale_exponent(float m, int top) {
   const int e = m > 0.0f ? top - exponent(m) : 0;
-  return e > 100 ? 100 : (e < -100 ? -100 : e);
+  return e > 100 ? 100 : e;
 }
 
 __device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi) {
@@ -188,6 +192,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
   __shared__ int tile_s;
   __shared__ int abort_s;
   __shared__ float e_s[kM], rho_s[kM], den_s[kM];
+  __shared__ int up_s[kM];  // a row's S and Q are held times 2^up (0 but for very dim rows)
   __shared__ int ccnt_s[kMaxClasses];
   __shared__ float clsb1_s[kMaxClasses];
   __shared__ float sumb1_s;
@@ -503,6 +508,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
       }
       e_s[tid] = ev;
       rho_s[tid] = rho;
+      up_s[tid] = 0;
     }
     for (int u = tid; u < (kUniB1 || kMode == kBuffers ? 0 : ncls * kM); u += blockDim.x) {
       const int k = u / kM, r = u % kM;
@@ -574,12 +580,49 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
       red_c[grp][row] = bsum;
     }
     tmem_wait_st();
-    __syncthreads();
+    const bool any_tiny = __syncthreads_or(xmax > 0.0f && xmax < kTiny) != 0;
     float den = den_s[row];
     float rho = rho_s[row];
     if (kMode == kBuffers) {
       rho = (1.0f - e_s[row]) * row_max(red_s);
       den = static_cast<float>(NA) - (1.0f - e_s[row]) * row_sum(red_c);
+    }
+    // Rows so dim that the powers of two below would leave FP32's range (the light front, a
+    // misfit in absolute units) are held multiplied by a power of two, to about one, and
+    // divided by it at the end; both are exact.
+    if (any_tiny) {
+      float s0 = 0.0f, up = 1.0f;
+#pragma unroll
+      for (int j = 0; j < C::HALF; ++j) s0 = fmaxf(s0, fabsf(S[j]));
+      __syncthreads();  // the reads of red_s above
+      red_s[grp][row] = s0;
+      __syncthreads();
+      const float m = row_max(red_d);
+      if (m > 0.0f && m < kTiny) {
+        int e = min(-exponent(m), 100 - exponent(row_max(red_s)));
+        e = e < 0 ? 0 : (e > 120 ? 120 : e);
+        up = pow2f(e);
+        if (grp == 0) up_s[row] = e;
+      }
+      __syncthreads();
+      red_d[grp][row] = xmax * up;
+#pragma unroll
+      for (int ch = 0; ch < NCH; ++ch) {
+        float qv[CH];
+        load_q(ch, qv);
+        if (ch < NCT) tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < CH; ++j) {
+          S[ch * CH + j] *= up;
+          if (ch < NCT)
+            qv[j] *= up;
+          else
+            qr[(ch - NCT) * CH + j] *= up;
+        }
+        if (ch < NCT) tmem_st<CH>(t_q + ch * CH, qv);
+      }
+      tmem_wait_st();
+      __syncthreads();
     }
 
     const float ev = e_s[row], al = 1.0f - ev;
@@ -703,7 +746,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
       rm = row_max(red_d);
       if (live) {
         ++iters;
-        thr = kTolShare * tol * fmaxf(row_max(red_s), 1e-6f * s_glob);
+        thr = kTolShare * tol * fmaxf(row_max(red_s), 1e-6f * s_glob * pow2f(up_s[row]));
         stalled = rm > 0.5f * prevr;
         prevr = rm;
         target = fmaxf(thr, amp * rm * kInnerDrop);
@@ -843,6 +886,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
     }
     if (aborted) break;
     if (bad && grp == 0) atomicAdd(rs.nonconv, 1);
+    const float down = pow2f(-up_s[row]);
 
     if constexpr (kMode == kAdjoint) {
       // ---- Qbar, warm start of the next reverse step, cleared adjoint level, gradient sums
@@ -870,14 +914,14 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
 #pragma unroll
           for (int j = 0; j < CH; ++j) {
             const size_t o = static_cast<size_t>(c0 + j) * plane + v;
-            const float y = S[ch * CH + j], qbar = ib[j] + y;
+            const float y = S[ch * CH + j] * down, qbar = ib[j] + y;
             io.qb[o] = qbar;
             if (io.y2) io.y2[o] = yo[j];
             io.y[o] = y;
             io.ib[o] = 0.0f;
             io.sb[o] = 0.0f;
             smax_loc = fmaxf(smax_loc, fabsf(y));
-            ga = fmaf(in[j], al > 0.0f ? y * inv_al : pz[j], ga);  // I (P z)
+            ga = fmaf(in[j], al > 0.0f ? y * inv_al : pz[j] * down, ga);  // I (P z)
             const float ds = cls_ds[sCls[c0 + j]], x = mu_v * ds;
             gm = fmaf(ds * sn[j] * qbar, ray_b0_over_x(x, expf(-x)), gm);
           }
@@ -923,13 +967,12 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
 #pragma unroll
           for (int j = 0; j < CH; ++j) {
             const int col = c0 + j;
-            float val = S[ch * CH + j];
+            const float s = S[ch * CH + j];
+            float val = s * down;
             if (pass == 0) {
-              val = form_x(bv[j], S[ch * CH + j], qv[j]);
-              if (vin) {
-                esum_row += val;
-                smax_loc = fmaxf(smax_loc, fabsf(S[ch * CH + j]));
-              }
+              smax_loc = fmaxf(smax_loc, vin ? fabsf(val) : 0.0f);
+              val = form_x(bv[j], s, qv[j]) * down;
+              if (vin) esum_row += val;
             }
             stg[(col >> 3) * 1024 + (col & 7) * 128 + row] = val;
           }
@@ -962,8 +1005,8 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
         if (vin) {
 #pragma unroll
           for (int j = 0; j < CH; ++j) {
-            const float s = S[ch * CH + j];
-            const float Iv = form_x(bv[j], s, qv[j]);
+            const float s = S[ch * CH + j] * down;
+            const float Iv = form_x(bv[j], S[ch * CH + j], qv[j]) * down;
             pI[static_cast<size_t>(ch * CH + j) * plane] = Iv;
             pS[static_cast<size_t>(ch * CH + j) * plane] = s;
             esum_row += Iv;
