@@ -76,6 +76,7 @@ constexpr int kSplitCycle = 64;                // longest Chebyshev cycle
 constexpr float kTolShare = 0.25f;             // share of the tolerance the stop test leaves to the change
 constexpr float kInnerError = 4.8828125e-04f;  // 2^-11: error of an inner correction, relative to it
 constexpr float kInnerDrop = 9.765625e-04f;    // 2^-10: an inner solve reduces its residual this far at most
+constexpr float kMinAmp = 2.384185791015625e-07f;  // 2^-22: rounding of S that a change may leave behind
 constexpr int kMaxOuter = 8;
 // Rows below this are held scaled up: 2^-50, so that a residual 2^-37 of the row still has its
 // full scale in scale_exponent.
@@ -750,7 +751,8 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
         stalled = rm > 0.5f * prevr;
         prevr = rm;
         target = fmaxf(thr, amp * rm * kInnerDrop);
-        const bool conv = amp * rm <= thr;
+        // (a change far above the result has left its own rounding in S, however thin the voxel)
+        const bool conv = fmaxf(amp, kMinAmp) * rm <= thr;
         inner = !conv && iters < max_iters && rm <= 3.0e38f;
         hitmax = !conv && !inner;
         if (inner) crow = cden * row_sum(red_c);

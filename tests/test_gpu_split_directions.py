@@ -15,6 +15,9 @@ FP64), four FP32 roundings 2.4e-7: 1.5e-6 is asked for (a sum of 192 FP32 produc
 2.9e-6; two terms per factor: 2.8e-4).  The same through a context, in a thin medium (b1 below
 0.006, tolerance at the floor): the residual a P I - S of the stored fields in each direction,
 with the stored I and S rounded and two outer residuals' error in it: 3e-6 of S.
+
+A start far above the result, in voxels so thin that one update reaches the fixed point: the bar of
+one product, 1.5e-6, as the start's rounding (2^-24 of it) must not stay in the result.
 """
 import ctypes
 
@@ -97,3 +100,18 @@ def test_weak_directions_of_a_step(nside, uniform):
     ref = mus / (mua + mus) * (P @ I)
     assert ref.min() > 0 and ref.max() > 300 * ref.min()
     assert np.all(np.abs(ref - S) <= 3e-6 * ref)
+
+
+@pytest.mark.parametrize("na", [48, 192])
+@pytest.mark.parametrize("b1", [0.0, 1e-9])
+@pytest.mark.parametrize("start", [1e4, 1e9])
+def test_nothing_of_a_bright_start_is_left(na, b1, start):
+    P32, P = _matrix(na, 0.9)
+    rng = np.random.default_rng(na)
+    nvox = 200
+    Q = (0.5 + rng.random((na, nvox))).astype(np.float32)
+    S0 = (start * rng.random((na, nvox))).astype(np.float32)
+    rc, S, _ = _buffers(P32, Q, np.full(Q.shape, b1), np.zeros(nvox), S0)
+    assert rc == 0
+    ref = np.linalg.solve(np.eye(na) - np.float64(np.float32(b1)) * P, P @ Q.astype(np.float64))
+    assert np.all(np.abs(S - ref) <= 1.5e-6 * np.abs(ref))
