@@ -43,8 +43,10 @@
 // makes has its spectrum in about [0, rho |g|], and Chebyshev weights over that interval
 // (roots in an order that keeps the partial products bounded) damp it by 0.43 an
 // iteration instead of 0.8:  d = r + c,  S += w d,  r <- r - w d + w a P B1 d.
-// P B1 d is one chain of K = 16 MMAs of FP16 x (b1 d, scaled by a power of two per voxel)
-// and Ph, its diagonal again FP32.
+// As P c = c, P B1 d = c + P x with x = b1 r - u c = r - u d, u = 1 - b1: in thick voxels c is
+// r / (u + eps), up to thousands of r, and b1 d in FP16 would be off by more than r, alike in all
+// directions (the corrections then diverge); x is of the size of r.  P x is one chain of K = 16
+// MMAs of FP16 x (scaled by a power of two per voxel) and Ph, its diagonal again FP32.
 //
 // Layout: as the BF16 kernel's (scatter_tc.cu): persistent CTAs, tiles of 8 x 4 x 4 voxels
 // (M = 128), operands K-major with the 128-byte swizzle, one voxel row per thread, four
@@ -312,7 +314,8 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
 
   // Weight of 8 columns from c0 on, as b1_of and form_x read it (volatile or asm loads: hoisted out of the iterations these
   // tables would cost more registers than there are)
-  // (kBuffers: from the caller's array; in the inner iterations as FP16, kept where Xl was)
+  // (kBuffers: b1 from the caller's array; in the inner iterations u = 1 - b1 as FP16, kept where
+  // Xl was.  b1 itself in FP16 is one in thick voxels, and the corrections then diverge.)
   int v = 0;
   const auto load_w = [&](int c0, float (&bv)[8], bool inner_pass = false) {
     if (kMode == kBuffers) {
@@ -364,9 +367,6 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
   // b1 is held as u = 1 - b1 (kBuffers: as the caller gave it): in thick cells the rounding of
   // b1 itself would be multiplied by 1 / (1 - a b1), u carries ten times less of it
   const auto b1_of = [](float w) { return kMode == kBuffers ? w : 1.0f - w; };
-  const auto b1_of2 = [](float w0, float w1) {
-    return kMode == kBuffers ? pk(w0, w1) : fma2(pk(w0, w1), pk(-1.0f, -1.0f), pk(1.0f, 1.0f));
-  };
   const auto form_x = [](float w, float sv, float q) {  // Q + b1 S
     return kMode == kBuffers ? fmaf(w, sv, q) : fmaf(-w, sv, q + sv);
   };
@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
             if (kMode == kAdjoint) qc[u][j] = form_x(bv[j], qi[u][j], qc[u][j]);  // Sbar + b1 Ibar
             if (kMode == kBuffers) {
               bmax = fmaxf(bmax, bv[j]);
-              bsum += bv[j];
+              bsum += 1.0f - bv[j];
             }
             const float s0 = (vin && sp2) ? fmaf(2.0f, s1[u][j], -s2[u][j]) : s1[u][j];
             S[ch * CH + j] = s0;
@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
     float rho = rho_s[row];
     if (kMode == kBuffers) {
       rho = (1.0f - e_s[row]) * row_max(red_s);
-      den = static_cast<float>(NA) - (1.0f - e_s[row]) * row_sum(red_c);
+      den = fmaf(static_cast<float>(NA), e_s[row], (1.0f - e_s[row]) * row_sum(red_c));
     }
     // Rows so dim that the powers of two below would leave FP32's range (the light front, a
     // misfit in absolute units) are held multiplied by a power of two, to about one, and
@@ -717,7 +717,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
             float r = da - (s - base);
             const float sh = base + da;
             if (kMode == kBuffers)
-              reinterpret_cast<__half*>(sXl)[(c0 + j) * kM + row] = __float2half_rn(bv[j]);
+              reinterpret_cast<__half*>(sXl)[(c0 + j) * kM + row] = __float2half_rn(1.0f - bv[j]);
             // adjoint, no scattering: y = 0 now; its P z goes where the residual would
             a0[j] = r;
             if (kMode == kAdjoint && al == 0.0f) {
@@ -743,7 +743,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
       }
       bool inner = false, fin = !live || (kMode == kAdjoint && al == 0.0f);  // fin: S has taken its last r of this outer
       bool stalled = false;
-      float target = 0.0f, es = 0.0f, crow = 0.0f;
+      float target = 0.0f, es = 0.0f, crow = 0.0f, xb = 0.0f;  // xb: bound of the operand's elements / 2
       rm = row_max(red_d);
       if (live) {
         ++iters;
@@ -755,17 +755,21 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
         const bool conv = fmaxf(amp, kMinAmp) * rm <= thr;
         inner = !conv && iters < max_iters && rm <= 3.0e38f;
         hitmax = !conv && !inner;
-        if (inner) crow = cden * row_sum(red_c);
+        if (inner) {
+          const float cs0 = row_sum(red_c);
+          crow = cden * cs0;
+          xb = rm + fminf(fabsf(crow), fabsf(cs0));  // (a max u <= den, so u |c| <= |sum b1 r|)
+        }
       }
       // ---- inner iterations on the error equation
       int k = 0, kc = 0;  // iteration, and its place in the Chebyshev cycle
       float om = __fdividef(1.0f, fmaf(-half, cw_s[0], mid));
       while (true) {
         const float w = inner ? om : (fin ? 0.0f : 1.0f);
-        const int er = scale_exponent(rm + fabsf(crow), 13);
+        const int er = scale_exponent(xb, 13);
         const float sc = inner ? pow2f(er) : 0.0f;
         if (__any_sync(0xffffffffu, w != 0.0f)) {
-          const f32x2 c2p = pk(crow, crow), w2 = pk(w, w), sc2 = pk(sc, sc);
+          const f32x2 nc2 = pk(-crow, -crow), neg1 = pk(-1.0f, -1.0f), nw2 = pk(-w, -w), sc2 = pk(sc, sc);
 #pragma unroll
           for (int c2 = 0; c2 < NCH; c2 += 2) {
             const int c0 = cb + c2 * CH;
@@ -779,12 +783,12 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
               uint32_t hi[4];
 #pragma unroll
               for (int j = 0; j < CH; j += 2) {
-                const f32x2 d = add2(pk(rv[u * CH + j], rv[u * CH + j + 1]), c2p);
+                const f32x2 r2 = pk(rv[u * CH + j], rv[u * CH + j + 1]), nd = fma2(r2, neg1, nc2);
                 float& s0 = S[(c2 + u) * CH + j];
                 float& s1 = S[(c2 + u) * CH + j + 1];
-                unpk(fma2(w2, d, pk(s0, s1)), s0, s1);
+                unpk(fma2(nw2, nd, pk(s0, s1)), s0, s1);
                 float x0, x1;
-                unpk(mul2(mul2(b1_of2(bv[j], bv[j + 1]), d), sc2), x0, x1);
+                unpk(mul2(fma2(pk(bv[j], bv[j + 1]), nd, r2), sc2), x0, x1);  // b1 r - u c
                 hi[j / 2] = pack_f16x2(x0, x1);
               }
               *reinterpret_cast<uint4*>(sXh + sw128_chunk_off(kM, row, c0 + u * CH)) =
@@ -792,7 +796,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
             }
           }
         }
-        if (inner) es += om * (rm + fabsf(crow));
+        if (inner) es += om * xb;
         if (!inner) fin = true;
         fence_async_smem();
         tc_fence_before();
@@ -810,8 +814,10 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
         float rmx = 0.0f, csx = 0.0f;
         if (mma_ok && __any_sync(0xffffffffu, inner)) {
           const float kd = tscale * pow2f(-er), wa = w * al;
-          const f32x2 c2p = pk(crow, crow), nw2 = pk(-w, -w), wa2 = pk(wa, wa), kd2 = pk(kd, kd);
-          f32x2 cs2 = pk(0.0f, 0.0f);
+          const float ec = ev * crow;
+          const f32x2 nc2 = pk(-crow, -crow), neg1 = pk(-1.0f, -1.0f), nw2 = pk(-w, -w), wa2 = pk(wa, wa);
+          const f32x2 kd2 = pk(kd, kd), ec2 = pk(ec, ec);
+          f32x2 cr2 = pk(0.0f, 0.0f), cu2 = pk(0.0f, 0.0f);
 #pragma unroll
           for (int ch = 0; ch < NCH; ++ch) {
             const int c0 = cb + ch * CH;
@@ -824,19 +830,20 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
             // a row that has stopped has w = 0 and x = 0, so D = 0: its r stays
 #pragma unroll
             for (int j = 0; j < CH; j += 2) {
-              const f32x2 r2 = pk(rv[j], rv[j + 1]), b1 = b1_of2(bv[j], bv[j + 1]);
-              const f32x2 d = add2(r2, c2p);
-              const f32x2 y = fma2(pk(di[j], di[j + 1]), mul2(b1, d), mul2(pk(dd[j], dd[j + 1]), kd2));  // P B1 d
-              const f32x2 rn = fma2(wa2, y, fma2(nw2, d, r2));
+              const f32x2 r2 = pk(rv[j], rv[j + 1]), u2 = pk(bv[j], bv[j + 1]);
+              const f32x2 x = fma2(u2, fma2(r2, neg1, nc2), r2);
+              const f32x2 y = fma2(pk(di[j], di[j + 1]), x, mul2(pk(dd[j], dd[j + 1]), kd2));  // P x
+              const f32x2 rn = fma2(wa2, y, fma2(nw2, add2(r2, ec2), r2));
               unpk(rn, rv[j], rv[j + 1]);
               rmx = fmaxf(rmx, fmaxf(fabsf(rv[j]), fabsf(rv[j + 1])));
-              cs2 = fma2(b1, rn, cs2);
+              cr2 = add2(cr2, rn);
+              cu2 = fma2(u2, rn, cu2);
             }
             tmem_st<CH>(t_row + C::ROFF + c0, rv);
           }
           float cs0, cs1;
-          unpk(cs2, cs0, cs1);
-          csx = cs0 + cs1;
+          unpk(fma2(cu2, neg1, cr2), cs0, cs1);
+          csx = cs0 + cs1;  // sum b1 r
           tmem_wait_st();
         }
         // the next weight, off the path between the barrier and the next operand
@@ -859,7 +866,9 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
             if (!conv && iters >= max_iters) hitmax = true;
             crow = 0.0f;
           } else {
-            crow = cden * row_sum(red_c);
+            const float cs0 = row_sum(red_c);
+            crow = cden * cs0;
+            xb = rm + fminf(fabsf(crow), fabsf(cs0));
           }
         }
       }
