@@ -79,7 +79,7 @@ constexpr float kTolShare = 0.25f;             // share of the tolerance the sto
 constexpr float kInnerError = 4.8828125e-04f;  // 2^-11: error of an inner correction, relative to it
 constexpr float kInnerDrop = 9.765625e-04f;    // 2^-10: an inner solve reduces its residual this far at most
 constexpr float kMinAmp = 2.384185791015625e-07f;  // 2^-22: rounding of S that a change may leave behind
-constexpr int kMaxOuter = 8;
+constexpr int kMaxStalls = 3;  // residuals that are not halved before a voxel above the floor is given up
 // Rows below this are held scaled up: 2^-50, so that a residual 2^-37 of the row still has its
 // full scale in scale_exponent.
 constexpr float kTiny = 8.8817841970012523e-16f;
@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
     bool hitmax = false, bad = false;
     float thr = 0.0f, prevr = 3.0e38f;
     int iters = 0;
-    int outer = 0;
+    int stalls = 0;
     while (true) {
       // ---- X = Q + b1 S, split
       const int ex = scale_exponent(row_max(red_d), 13);
@@ -742,19 +742,25 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
         break;
       }
       bool inner = false, fin = !live || (kMode == kAdjoint && al == 0.0f);  // fin: S has taken its last r of this outer
-      bool stalled = false;
+      bool stalled = false, lost = false;  // no further outers; ... and the residual is above its noise floor
       float target = 0.0f, es = 0.0f, crow = 0.0f, xb = 0.0f;  // xb: bound of the operand's elements / 2
       rm = row_max(red_d);
       if (live) {
         ++iters;
         thr = kTolShare * tol * fmaxf(row_max(red_s), 1e-6f * s_glob * pow2f(up_s[row]));
-        stalled = rm > 0.5f * prevr;
-        prevr = rm;
+        // the residual is noise below 2^-21 of the row's largest X (2^(14 - ex) bounds that);
+        // above it one that is not halved says that the corrections do not do what they should
+        const bool slow = rm > 0.5f * prevr, at_floor = rm <= pow2f(-7 - ex);
+        stalls += slow ? 1 : 0;
+        prevr = fminf(prevr, rm);
+        stalled = slow && (at_floor || stalls >= kMaxStalls);
+        lost = !(rm <= 3.0e38f) || (stalled && !at_floor);
         target = fmaxf(thr, amp * rm * kInnerDrop);
         // (a change far above the result has left its own rounding in S, however thin the voxel)
         const bool conv = fmaxf(amp, kMinAmp) * rm <= thr;
         inner = !conv && iters < max_iters && rm <= 3.0e38f;
         hitmax = !conv && !inner;
+        lost = (lost && !conv) || ex < -114;  // (an infinite X: its residual is not a number)
         if (inner) {
           const float cs0 = row_sum(red_c);
           crow = cden * cs0;
@@ -873,11 +879,10 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
         }
       }
       if (aborted) break;
-      ++outer;
       // another accurate residual where the inner products' error may exceed the tolerance
-      bool more = live && !hitmax && !stalled && iters < max_iters && outer < kMaxOuter &&
+      bool more = live && !hitmax && !stalled && iters < max_iters &&
                   (amp * rm > thr || eta * es > thr);
-      if (live && amp * rm > thr && iters >= max_iters) bad = true;
+      if (live && (lost || (amp * rm > thr && iters >= max_iters))) bad = true;
       live = more;
       // (the barrier also separates the reads of red_d above from the writes below)
       if (!__syncthreads_or(more ? 1 : 0)) break;

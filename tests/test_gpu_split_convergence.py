@@ -9,6 +9,7 @@ voxel) with kernels of either sign, and a start of the wrong size.
 import numpy as np
 import pytest
 
+import paper_2105_01028_gb300 as T
 from test_gpu_split_directions import _buffers, _matrix
 
 pytestmark = pytest.mark.gpu
@@ -33,3 +34,15 @@ def test_success_means_the_fixed_point(na, g, start):
         rho = a * b.max()
         bound = max(2e-6, rho / (1.0 - rho) * 2.0 ** -20)
         assert np.max(np.abs(S[:, v] - ref)) <= bound * np.max(np.abs(ref)), v
+
+
+@pytest.mark.parametrize("na", [48, 192])
+def test_an_overflow_is_reported(na):
+    P32, _ = _matrix(na, 0.9)
+    Q = np.full((na, 140), 1.0, dtype=np.float32)
+    Q[:, 7] = 3e38  # its fixed point is not an FP32 number
+    b1, eps = np.full(Q.shape, 0.9), np.full(140, 0.01)
+    rc, S, _ = _buffers(P32, Q, b1, eps, Q, max_iters=200)
+    assert rc == T.W_NOT_CONVERGED
+    # (the start's largest value sets the scale of the stop test: the others take one update)
+    assert np.isfinite(np.delete(S, 7, axis=1)).all()
