@@ -5,7 +5,31 @@
 #include <cuda_runtime.h>
 #include <vector>
 
+#include "per_device.h"
+
 namespace trinity {
+
+// SM count of the current device, after ``attributes`` (launch attributes of the kernels that
+// ``done`` stands for) has succeeded there once; 0 if it fails.
+template <class F>
+int configured_sms(PerDevice& done, F attributes) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  return done.get(dev, [&] {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        attributes() != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return sms;
+  });
+}
+
+inline int device_sms() {
+  static PerDevice counted;
+  return configured_sms(counted, [] { return cudaSuccess; });
+}
 
 // Per-direction constants of the ray lattice (built on the host in FP64, stored FP32).
 struct DirInfo {

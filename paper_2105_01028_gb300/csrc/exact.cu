@@ -302,15 +302,16 @@ cudaError_t launch_exact_fp32(const GridParams& g, const float* b1ds, int nch, c
                               cudaStream_t st) {
   if (g.na == kGNa && b1tab) {
     constexpr size_t kDyn = (static_cast<size_t>(kGNa) * kGV + static_cast<size_t>(kGKc) * kGNa) * sizeof(float);
-    static cudaError_t attr = [] {
+    static PerDevice set_up;
+    const int sms = configured_sms(set_up, [] {
       cudaError_t e = cudaFuncSetAttribute(exact_gemm192_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            static_cast<int>(kDyn));
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(exact_gemm192_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  cudaSharedmemCarveoutMaxShared);
       return e;
-    }();
-    if (attr != cudaSuccess) return attr;
+    });
+    if (sms == 0) return cudaErrorUnknown;
     const int blocks = (g.nv + kGV - 1) / kGV;
     exact_gemm192_kernel<<<blocks, 256, kDyn, st>>>(g, Mt, b1tab, cls, mua_cls, Q, nidx, Iring, Sring, rs);
     return cudaGetLastError();

@@ -568,16 +568,11 @@ cudaError_t make_exact_qmap(const GridParams& g, const float* Q, void* out) {
 cudaError_t launch_exact_tc(const GridParams& g, const void* qmap, const float* Mimg, const uint8_t* tmask,
                             const float* b1tab, int ncls, const uint8_t* cls, const float* mua_cls, const float* Q,
                             const float* nidx, float* Iring, float* Sring, RunState rs, cudaStream_t st) {
-  static int nsm = 0;
-  static cudaError_t attr = cudaErrorUnknown;
-  if (nsm == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return cudaErrorUnknown;
-    attr = cudaFuncSetAttribute(exact_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-  }
-  if (attr != cudaSuccess) return attr;
+  static PerDevice set_up;
+  const int nsm = configured_sms(set_up, [] {
+    return cudaFuncSetAttribute(exact_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  });
+  if (nsm == 0) return cudaErrorUnknown;
   if (!exact_tc_supported(g, ncls)) return cudaErrorInvalidValue;
   const int ntiles = exact_tc_tiles(g.nv);
   const int grid = ntiles < nsm ? ntiles : nsm;

@@ -507,7 +507,9 @@ cudaError_t launch_tally(const GridParams& g, const DirInfo* dirs, const float* 
   const auto chunks = [](int n) { return (n + 255) / 256; };
   const long items = 2L * (chunks(g.ny * g.nz) + chunks(g.nx * g.nz) + chunks(g.nx * g.ny)) *
                      ((g.na + kTallyDirs - 1) / kTallyDirs);
-  const int grid = items > 4 * 152 ? 4 * 152 : static_cast<int>(items);
+  const int sms = device_sms();
+  if (sms == 0) return cudaErrorUnknown;
+  const int grid = items > 4 * sms ? 4 * sms : static_cast<int>(items);
   tally_kernel<<<grid, 256, 0, st>>>(g, dirs, Iring, det_vox, det_dir, det_w, det_id,
                                      n_det_entries, det, nbins, rs);
   return cudaGetLastError();

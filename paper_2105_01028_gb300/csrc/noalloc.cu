@@ -24,7 +24,6 @@ namespace {
 
 constexpr int kNoAllocMaxVoxels = 1 << 20;  // 1,048,576 voxels: 4 MiB of bounds
 constexpr int kNaTile = 32;                   // voxels per CTA (as in the FP32 kernel)
-constexpr int kMaxDevices = 64;
 
 struct NoAllocScratch {
   unsigned smax;       // max |S_prev| as float bits (the stop rule's floor scale)

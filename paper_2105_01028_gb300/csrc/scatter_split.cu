@@ -1095,7 +1095,7 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
   }
 }
 
-int g_split_sms = 0;
+PerDevice g_split;
 
 template <int NA, int kMode, int kPer>
 cudaError_t configure_split() {
@@ -1114,11 +1114,22 @@ cudaError_t configure_mode() {
   return e;
 }
 
+// SM count of the current device, its kernels configured; 0 if they cannot be.
+int split_sms() {
+  return configured_sms(g_split, [] {
+    cudaError_t e = configure_mode<kStep>();
+    if (e == cudaSuccess) e = configure_mode<kBuffers>();
+    if (e == cudaSuccess) e = configure_mode<kAdjoint>();
+    return e;
+  });
+}
+
 template <int kMode>
 cudaError_t launch_split(const GridParams& g, const SplitTables& sp, const BfTables& t, const SplitIo& io, float tol,
                          int max_iters, const CUtensorMap& mI, const CUtensorMap& mS, int tma_out, const RunState& rs,
                          cudaStream_t st) {
-  if (g_split_sms == 0) return cudaErrorInvalidValue;
+  const int sms = split_sms();
+  if (sms == 0) return cudaErrorInvalidValue;
   const int ntiles = kMode == kBuffers ? (g.nv + kM - 1) / kM : brick_tiles(g.nx, g.ny, g.nz);
   constexpr bool kU = kMode != kBuffers;
   const bool uni = kU && g.mut_u >= 0.0f;
@@ -1126,14 +1137,14 @@ cudaError_t launch_split(const GridParams& g, const SplitTables& sp, const BfTab
     // two CTAs per SM from 2.5 tiles per SM on (as scatter_tc.cu): 0.273 against 0.307 ms at
     // 56^3 with varying mu_t, 0.683 against 0.809 at 80^3; one CTA otherwise (0.061 against
     // 0.073 ms a step at 16^3)
-    const bool two = 2 * ntiles > 5 * g_split_sms;
-    const int cap = two ? 2 * g_split_sms : g_split_sms, grid = ntiles < cap ? ntiles : cap;
+    const bool two = 2 * ntiles > 5 * sms;
+    const int cap = two ? 2 * sms : sms, grid = ntiles < cap ? ntiles : cap;
     auto k = two ? (uni ? scatter_split_kernel<48, kU, kMode, 2> : scatter_split_kernel<48, false, kMode, 2>)
                  : (uni ? scatter_split_kernel<48, kU, kMode, 1> : scatter_split_kernel<48, false, kMode, 1>);
     k<<<grid, Sp<48>::kThreads, Sp<48>::SMEM, st>>>(g, sp, t.cls, t.cls_ds, t.ncls, t.nch, io, tol, max_iters, mI, mS,
                                                     tma_out, rs);
   } else if (g.na == 192) {
-    const int grid = ntiles < g_split_sms ? ntiles : g_split_sms;
+    const int grid = ntiles < sms ? ntiles : sms;
     auto k = uni ? scatter_split_kernel<192, kU, kMode, 1> : scatter_split_kernel<192, false, kMode, 1>;
     k<<<grid, Sp<192>::kThreads, Sp<192>::SMEM, st>>>(g, sp, t.cls, t.cls_ds, t.ncls, t.nch, io, tol, max_iters, mI,
                                                       mS, tma_out, rs);
@@ -1160,18 +1171,7 @@ double half_value(uint16_t u) {
 
 bool scatter_split_supported(int na, int ncls) {
   if ((na != 48 && na != 192) || ncls > kMaxClasses) return false;
-  if (g_split_sms == 0) {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        configure_mode<kStep>() != cudaSuccess || configure_mode<kBuffers>() != cudaSuccess ||
-        configure_mode<kAdjoint>() != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    g_split_sms = sms;
-  }
-  return true;
+  return split_sms() > 0;
 }
 
 // Off-diagonal part of the FP64 phase matrix P split as (Ph + Pl + Pm) unit, in the kernel's

@@ -796,7 +796,7 @@ __global__ void __launch_bounds__(TcThreads<NA>::kThreads, 1)
   }
 }
 
-int g_num_sms = 0;
+PerDevice g_tc;
 
 template <int NA>
 cudaError_t configure() {
@@ -809,20 +809,18 @@ cudaError_t configure() {
                               Tc<NA>::SMEM);
 }
 
+// SM count of the current device, its kernels configured; 0 if they cannot be.
+int tc_sms() {
+  return configured_sms(g_tc, [] {
+    const cudaError_t e = configure<48>();
+    return e == cudaSuccess ? configure<192>() : e;
+  });
+}
+
 }  // namespace
 
 bool scatter_bf16_supported(int na) {
-  if (na != 48 && na != 192) return false;
-  if (g_num_sms == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    if (cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
-    if (configure<48>() != cudaSuccess || configure<192>() != cudaSuccess) {
-      g_num_sms = 0;
-      return false;
-    }
-  }
-  return true;
+  return (na == 48 || na == 192) && tc_sms() > 0;
 }
 
 static PFN_cuTensorMapEncodeTiled_v12000 g_encode_out = nullptr;
@@ -869,7 +867,9 @@ cudaError_t launch_scatter_bf16(const GridParams& g, const BfTables& t, const ui
   // 48 directions: two CTAs per SM (one waits while the other computes: 0.185 against 0.234 ms
   // at 56^3, 0.457 against 0.611 at 80^3), but from 2.5 tiles per SM on; with fewer, CTAs
   // that share an SM finish later than tiles taken in turn (0.083 against 0.063 ms at 32^3)
-  const int cap = g_num_sms * (g.na == 48 && 2 * ntiles > 5 * g_num_sms ? TcThreads<48>::kPerSm : 1);
+  const int sms = tc_sms();
+  if (sms == 0) return cudaErrorInvalidValue;
+  const int cap = sms * (g.na == 48 && 2 * ntiles > 5 * sms ? TcThreads<48>::kPerSm : 1);
   const int grid = ntiles < cap ? ntiles : cap;
   const bool uni = g.mut_u >= 0.0f;
   if (g.na == 48) {

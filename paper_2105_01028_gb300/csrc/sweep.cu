@@ -394,7 +394,9 @@ cudaError_t launch_sweep(const GridParams& g, const DirInfo* dirs, const int8_t*
   if (!g.periodic && !g.mirror) {
     // fewer row groups per block where the grid would otherwise not fill the chip (16^3 at 48
     // directions: 60 blocks of eight row groups take 19 us, 480 of one row group 14)
-    int rs_n = groups * ngroups / (152 * 8);
+    const int sms = device_sms();
+    if (sms == 0) return cudaErrorUnknown;
+    int rs_n = groups * ngroups / (sms * 8);
     rs_n = rs_n < 1 ? 1 : (rs_n > kRowSweepsG ? kRowSweepsG : rs_n);
     const dim3 gg((groups + rs_n - 1) / rs_n, ngroups);
     auto k = un ? (um ? sweep_group_kernel<true, true> : sweep_group_kernel<true, false>)

@@ -396,13 +396,8 @@ cudaError_t launch_class(const GridParams& g, const DirInfo* dirs, const int* dl
 cudaError_t launch_sweep_tma(const GridParams& g, const DirInfo* dirs, const int* const dlist[3],
                              const int ndir[3], const int8_t* offs, const int8_t* hsh, const SweepMaps& maps,
                              float* Q, RunState rs, const cudaStream_t st[3]) {
-  static int nsm = 0;
-  if (nsm == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return cudaErrorUnknown;
-  }
+  const int nsm = device_sms();
+  if (nsm == 0) return cudaErrorUnknown;
   // the first class launched (with directions) also clears this step's max |S| and work counter
   const int f2 = ndir[2] > 0, f1 = !f2 && ndir[1] > 0, f0 = !f2 && !f1;
   // the classes write disjoint planes of Q and only read the rings: st[k] may run them
