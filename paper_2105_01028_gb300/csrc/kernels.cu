@@ -1,6 +1,7 @@
 // FP32 kernels of one time step: the per-voxel source iteration on CUDA cores (Eq. 12,
 // Section 2.4 steps 5-6), the detector / escape tallies (Section 3.1), the interface
 // split and the step counter.
+#include <algorithm>
 #include <cfloat>
 #include <cstdint>
 
@@ -345,11 +346,13 @@ __global__ void __launch_bounds__(ScatterCfg<NA>::kThreads, 2)
 // ----------------------------------------------------------------------------------------
 // Tallies of level n (Section 3.1): detector curves (FP64 bins) and the energy leaving
 // through all faces.
-// Work items are (face, 256 face voxels, 16 directions): a thread loads its voxel's 16
-// values together, so a step's face values (16 MB on the 96x96x64 slab at 192 directions)
-// are in flight at once.  A thread that walked all directions of its voxel in one chain left
-// the kernel bound by that chain's latency: 35 us at 32^3, 572 us at 3072 directions on
-// 32x32x24 voxels; now 8 and 62 us.
+// Work items are 256 entries of the detector list, then (face, 256 face voxels, 16 directions):
+// there a thread loads its voxel's 16 values together, so a step's face values (16 MB on the
+// 96x96x64 slab at 192 directions) are in flight at once.  A thread that walked all directions
+// of its voxel in one chain left the kernel bound by that chain's latency: 35 us at 32^3,
+// 572 us at 3072 directions on 32x32x24 voxels; now 8 and 62 us.  The entry list in one block
+// cost a step 96 us with eight detectors of 5 mm radius at 32^3 and 192 directions (291 us, now
+// 195; 188 with one-voxel detectors).
 // ----------------------------------------------------------------------------------------
 constexpr int kTallyDirs = 16;
 
@@ -364,71 +367,73 @@ __global__ void __launch_bounds__(256) tally_kernel(GridParams g, const DirInfo*
   const int n = *rs.step;
   const size_t plane = static_cast<size_t>(g.nv);
   const float* Icur = Iring + static_cast<size_t>(ring_slot(n)) * g.na * plane;
-  if (blockIdx.x == gridDim.x - 1) {
-    // detector entries: weight already holds alpha * Omega_cap * cos * h^2 * dt
-    const int b = rs.bins[n];
-    if (b >= 0 && b < nbins)
-      for (int e = threadIdx.x; e < n_entries; e += blockDim.x) {
+  const int ndet = (n_entries + 255) >> 8;
+  const int ngrp = (g.na + kTallyDirs - 1) / kTallyDirs;
+  // chunks of 256 voxels per face of each axis
+  const int cx = (g.ny * g.nz + 255) >> 8, cy = (g.nx * g.nz + 255) >> 8, cz = (g.nx * g.ny + 255) >> 8;
+  const bool open = !g.periodic && !g.mirror;  // a closed box lets nothing out
+  const int nitems = ndet + (open ? 2 * (cx + cy + cz) * ngrp : 0);
+  double acc = 0.0;
+  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+    if (it < ndet) {
+      // the weight already holds alpha * Omega_cap * cos * h^2 * dt
+      const int b = rs.bins[n], e = (it << 8) + threadIdx.x;
+      if (b >= 0 && b < nbins && e < n_entries) {
         const double val = static_cast<double>(det_w[e]) *
                            static_cast<double>(Icur[static_cast<size_t>(det_dir[e]) * plane + det_vox[e]]);
         atomicAdd(det + static_cast<size_t>(det_id[e]) * nbins + b, val);
       }
+      continue;
+    }
+    const int item = it - ndet;
+    const int grp = item % ngrp;
+    int c = item / ngrp, face, nc;
+    if (c < 2 * cx) {
+      face = 0;
+      nc = cx;
+    } else if ((c -= 2 * cx) < 2 * cy) {
+      face = 2;
+      nc = cy;
+    } else {
+      c -= 2 * cy;
+      face = 4;
+      nc = cz;
+    }
+    if (c >= nc) {
+      c -= nc;
+      face += 1;
+    }
+    const int ax = face >> 1;
+    const int nu = ax == 0 ? g.ny : g.nx, nw = ax == 2 ? g.ny : g.nz;
+    const int t = (c << 8) + threadIdx.x;
+    if (t >= nu * nw) continue;
+    const int iu = t % nu, iw = t / nu;
+    const int pa = (face & 1) ? pick(ax, g.nx, g.ny, g.nz) - 1 : 0;
+    const int x = ax == 0 ? pa : iu, y = ax == 0 ? iu : (ax == 1 ? pa : iw), z = ax == 2 ? pa : iw;
+    const float* col = Icur + (static_cast<size_t>(z) * g.ny + y) * g.nx + x;
+    float val[kTallyDirs], wc[kTallyDirs];
+#pragma unroll
+    for (int k = 0; k < kTallyDirs; ++k) {
+      const int d = grp * kTallyDirs + k;
+      wc[k] = d < g.na ? dirs[d].wcos_out[face] : 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < kTallyDirs; ++k)
+      val[k] = wc[k] != 0.0f ? __ldg(col + static_cast<size_t>(grp * kTallyDirs + k) * plane) : 0.0f;
+    float s = 0.0f;
+#pragma unroll
+    for (int k = 0; k < kTallyDirs; ++k) s = fmaf(wc[k], val[k], s);
+    acc += static_cast<double>(s);
   }
-  if (!g.periodic && !g.mirror) {  // a closed box lets nothing out
-    const int ngrp = (g.na + kTallyDirs - 1) / kTallyDirs;
-    // chunks of 256 voxels per face of each axis
-    const int cx = (g.ny * g.nz + 255) >> 8, cy = (g.nx * g.nz + 255) >> 8, cz = (g.nx * g.ny + 255) >> 8;
-    const int nitems = 2 * (cx + cy + cz) * ngrp;
-    double acc = 0.0;
-    for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
-      const int grp = item % ngrp;
-      int c = item / ngrp, face, nc;
-      if (c < 2 * cx) {
-        face = 0;
-        nc = cx;
-      } else if ((c -= 2 * cx) < 2 * cy) {
-        face = 2;
-        nc = cy;
-      } else {
-        c -= 2 * cy;
-        face = 4;
-        nc = cz;
-      }
-      if (c >= nc) {
-        c -= nc;
-        face += 1;
-      }
-      const int ax = face >> 1;
-      const int nu = ax == 0 ? g.ny : g.nx, nw = ax == 2 ? g.ny : g.nz;
-      const int t = (c << 8) + threadIdx.x;
-      if (t >= nu * nw) continue;
-      const int iu = t % nu, iw = t / nu;
-      const int pa = (face & 1) ? pick(ax, g.nx, g.ny, g.nz) - 1 : 0;
-      const int x = ax == 0 ? pa : iu, y = ax == 0 ? iu : (ax == 1 ? pa : iw), z = ax == 2 ? pa : iw;
-      const float* col = Icur + (static_cast<size_t>(z) * g.ny + y) * g.nx + x;
-      float val[kTallyDirs], wc[kTallyDirs];
+  if (!open) return;
 #pragma unroll
-      for (int k = 0; k < kTallyDirs; ++k) {
-        const int d = grp * kTallyDirs + k;
-        wc[k] = d < g.na ? dirs[d].wcos_out[face] : 0.0f;
-      }
-#pragma unroll
-      for (int k = 0; k < kTallyDirs; ++k)
-        val[k] = wc[k] != 0.0f ? __ldg(col + static_cast<size_t>(grp * kTallyDirs + k) * plane) : 0.0f;
-      float s = 0.0f;
-#pragma unroll
-      for (int k = 0; k < kTallyDirs; ++k) s = fmaf(wc[k], val[k], s);
-      acc += static_cast<double>(s);
-    }
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double s = 0.0;
-      for (int w = 0; w < 8; ++w) s += red[w];
-      atomicAdd(rs.escaped + n, s);
-    }
+  for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int w = 0; w < 8; ++w) s += red[w];
+    atomicAdd(rs.escaped + n, s);
   }
 }
 
@@ -505,8 +510,9 @@ cudaError_t launch_tally(const GridParams& g, const DirInfo* dirs, const float* 
                          const int* det_id, int n_det_entries, double* det, int nbins,
                          RunState rs, cudaStream_t st) {
   const auto chunks = [](int n) { return (n + 255) / 256; };
-  const long items = 2L * (chunks(g.ny * g.nz) + chunks(g.nx * g.nz) + chunks(g.nx * g.ny)) *
+  const long faces = 2L * (chunks(g.ny * g.nz) + chunks(g.nx * g.nz) + chunks(g.nx * g.ny)) *
                      ((g.na + kTallyDirs - 1) / kTallyDirs);
+  const long items = std::max(1L, chunks(n_det_entries) + (g.periodic || g.mirror ? 0L : faces));
   const int sms = device_sms();
   if (sms == 0) return cudaErrorUnknown;
   const int grid = items > 4 * sms ? 4 * sms : static_cast<int>(items);
