@@ -227,6 +227,11 @@ bool desc_valid(const trinity_grid_desc* d, std::string* why) {
   return true;
 }
 
+// Device bytes of the split phase matrix: the three operand images, diagonals and roots.
+size_t split_bytes(size_t na) {
+  return 3 * ((na + 63) / 64) * na * 128 + 3 * na * 4 + 64 * 4;
+}
+
 size_t footprint(const trinity_grid_desc* d) {
   const size_t nv = static_cast<size_t>(d->nx) * d->ny * d->nz;
   const size_t na = 12u * d->nside * d->nside;
@@ -239,6 +244,11 @@ size_t footprint(const trinity_grid_desc* d) {
   if (na_s != na) b += (kRing + 1) * na_s * nv * sizeof(float);  // coarse I history, Qbar
   b += 3 * nv * sizeof(float);                 // optics
   b += na_s * na_s * (sizeof(float) + sizeof(uint16_t));
+  if (na_s >= 48) b += split_bytes(na_s);  // (BF16 contexts: with their first gradient)
+  const size_t nmax = std::max(d->nx, std::max(d->ny, d->nz));
+  b += 2 * na * nmax * sizeof(int8_t);         // lattice offsets
+  if (na_s == na && d->boundary == TRINITY_BOUNDARY_VACUUM)
+    b += na * nmax * sizeof(int2) + kSweepGroup * na * sizeof(int);  // plain-load sweep: displacements, groups
   return b;
 }
 
@@ -405,11 +415,6 @@ int lock_inputs(trinity_ctx* ctx) {
   CK(cudaMemcpy(ctx->d_balance, &ctx->energy_init, sizeof(double), cudaMemcpyHostToDevice));
   ctx->locked = true;
   return TRINITY_OK;
-}
-
-// Device bytes of the split phase matrix: the three operand images, diagonals and roots.
-size_t split_bytes(int na) {
-  return 3 * static_cast<size_t>((na + 63) / 64) * na * 128 + 3 * static_cast<size_t>(na) * 4 + 64 * 4;
 }
 
 // Build the split of the phase matrix for the tensor-core iteration and upload it.
