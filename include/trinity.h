@@ -41,7 +41,7 @@ typedef struct trinity_ctx trinity_ctx;
 
 typedef enum {
   TRINITY_OK = 0,
-  TRINITY_W_NOT_CONVERGED = 1, /* completed, but some voxel hit max_iters in a step */
+  TRINITY_W_NOT_CONVERGED = 1, /* completed, but some voxel did not converge (trinity_step) */
   TRINITY_E_INVALID = -1,      /* bad argument or unsupported combination */
   TRINITY_E_OOM = -2,          /* device allocation failed */
   TRINITY_E_CUDA = -3,         /* a CUDA call failed (message has the CUDA error) */
@@ -199,10 +199,12 @@ int trinity_set_initial_state(trinity_ctx* ctx, const float* I0, const float* S0
  * floor of the mode's arithmetic: FP32 mode (12 directions), the change has not reached a new
  * minimum for three iterations (from 48 directions on the bound is taken at tol / 4 on
  * residuals formed with FP32 accuracy, corrected by Chebyshev iterations, until a residual
- * is no longer halved); BF16 mode, |S^k - S^(k-1)|_inf <= 2^-17 scale (the resolution of X
- * carried as two BF16 terms) or no new minimum for two iterations.  Then the detector and
- * energy tallies.  iters_out (may be NULL) receives the largest iteration count of each step.  Returns
- * TRINITY_W_NOT_CONVERGED if any voxel hit max_iters. */
+ * below 2^-21 of the voxel's largest Q + b1 S is no longer halved); BF16 mode,
+ * |S^k - S^(k-1)|_inf <= 2^-17 scale (the resolution of X carried as two BF16 terms) or no new
+ * minimum for two iterations.  Then the detector and energy tallies.  iters_out (may be NULL)
+ * receives the largest iteration count of each step.  Returns TRINITY_W_NOT_CONVERGED if any
+ * voxel hit max_iters (FP32 mode from 48 directions on: or was given up above that floor, or
+ * overflowed). */
 int trinity_step(trinity_ctx* ctx, int nsteps, int* iters_out);
 
 /* Same as trinity_step without per-step read-back: the steps are replayed from a
@@ -263,7 +265,8 @@ int trinity_kernels_per_step(const trinity_ctx* ctx, int* n);
 
 /* Form of the ray sweep a step runs: 0 plain loads (one kernel), 1 upwind planes staged
  * through TMA tile loads (one kernel per dominant-axis class, run concurrently: vacuum
- * faces, uniform refractive index and mu_t, nx a multiple of 4), 2 the fused two-level sweep. */
+ * faces, uniform refractive index and mu_t, nx a multiple of 4, at least 2^19 voxel-directions),
+ * 2 the fused two-level sweep. */
 int trinity_sweep_form(const trinity_ctx* ctx, int* form);
 
 /* on = 0: the plain-load sweep even where the TMA-staged one applies (both perform the
@@ -409,8 +412,8 @@ void trinity_serve_destroy(trinity_server* srv);
  * S = (1 - eps) P (Q + b1 o S) of the FP32 mode (same arithmetic and stop rule as
  * trinity_step) on caller-owned device buffers and allocates no device memory: its
  * scratch (per-voxel contraction bounds, a max-reduction cell, iteration counters, the
- * phase matrix split for the tensor cores) is a static device array of 4.2 MiB that every GPU loading the library holds until the
- * process exits.
+ * phase matrix split for the tensor cores) is a static device array of 4.2 MiB that every GPU
+ * loading the library holds until the process exits.
  *   na       12, 48 or 192 directions; nvox voxels, 1 <= nvox <= 1048576 (the scratch
  *            limit: larger sizes return TRINITY_E_INVALID without running).
  *   P        [na][na] FP32, symmetric with unit row sums up to rounding (e.g. the matrix of
@@ -422,7 +425,7 @@ void trinity_serve_destroy(trinity_server* srv);
  *   tol, max_iters as in trinity_grid_desc; *iters_max (may be NULL) gets the largest
  *   iteration count.  All pointers except iters_max are device pointers of the current
  *   device; the work runs on ``stream`` (a cudaStream_t or NULL) and the call returns
- *   after it finishes.  TRINITY_W_NOT_CONVERGED if a voxel reached max_iters.
+ *   after it finishes.  TRINITY_W_NOT_CONVERGED as for trinity_step.
  * The first call on a device looks up the scratch array's device address (a host-side
  * step, once per device); make that first call before any stream capture.  Every call
  * shares the one array and clears the parts that must start at zero, so calls whose GPU

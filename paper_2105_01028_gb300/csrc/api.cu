@@ -608,9 +608,12 @@ int restore_checkpoint(trinity_ctx* ctx, int k, int c, bool store) {
 // refractive index (one retarded delay per direction), not switched off, and a uniform mu_t
 // (0.445 ms on the 96x96x64 slab, the plain-load form 0.476).  Where mu_t varies the plain-load
 // form is the faster one, as it shares a voxel's weights among directions: 0.230 against
-// 0.261 ms at 64^3, 0.181 against 0.213 at 56^3 (192 directions, the same bits).  On the
-// smallest boxes its one launch beats three with a fork and a join: 9 against 14 us at 16^3 and
-// 48 directions (2^17.6 updates; from 2^19 on the TMA form is kept).
+// 0.261 ms at 64^3, 0.181 against 0.213 at 56^3 (192 directions, the same bits).  On small
+// boxes its one launch beats three with a fork and a join: 9 against 14 us at 16^3 and 48
+// directions (2^17.6 updates).  With uniform optics the two cross between 2^21 and 2^22.3
+// updates: the plain form is 3 to 5 us a step faster at 24^3 to 32^3 and 48 directions (of 52 to
+// 94 us), even at 40^3, and 1 to 7 us slower from 48^3 on.  The line at 2^19 is lower than that
+// and keeps the staged form on boxes that it has always run on.
 bool sweep_uses_tma(const trinity_ctx* ctx) {
   return !ctx->two_level && ctx->tma && !ctx->tma_off && ctx->g.n_u >= 1.0f && ctx->g.mut_u >= 0.0f &&
          static_cast<long>(ctx->g.nv) * ctx->g.na >= (1L << 19);
