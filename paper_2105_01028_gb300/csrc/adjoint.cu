@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(AdjCfg<NA>::kThreads, 2)
 #pragma unroll
     for (int v = 0; v < kTile; ++v) acc[v] = 0.0f;
     if (live) {
-      constexpr int kBlk = (NA % 8 == 0) ? 8 : 4;
+      constexpr int kBlk = 4;
       const float* pcol = P + i;
 #pragma unroll 1
       for (int j0 = 0; j0 < NA; j0 += kBlk) {

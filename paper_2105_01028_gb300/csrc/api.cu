@@ -638,8 +638,8 @@ int enqueue_transport(trinity_ctx* ctx, const RunState& rs) {
       CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_join[k], 0));
     }
   } else {
-    CK(launch_sweep(g, ctx->d_dirs, ctx->d_offs, ctx->d_group, ctx->n_group, ctx->d_disp, ctx->I, ctx->S, ctx->mut, ctx->nidx, ctx->d_refl, ctx->Q, rs,
-                    ctx->stream));
+    CK(launch_sweep(g, ctx->d_dirs, ctx->d_offs, ctx->d_group, ctx->n_group, ctx->d_disp, ctx->I, ctx->S, ctx->mut,
+                    ctx->nidx, ctx->d_refl, ctx->Q, rs, ctx->stream));
   }
   CK(launch_interface(ctx->n_iface, g.na, ctx->d_if_vox, ctx->d_if_rowptr, ctx->d_if_src, ctx->d_if_w,
                       ctx->d_if_keep, ctx->Q, g.nv, ctx->stream));

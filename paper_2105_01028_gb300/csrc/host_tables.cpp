@@ -134,8 +134,8 @@ std::vector<double> cosines(const std::vector<double>& dirs) {
 
 // K_ij = w * HG(Omega_i . Omega_j; g), scaled to unit row (= column) sums by a symmetric
 // diagonal D (damped Sinkhorn: d <- sqrt(d / (K d)) from the given d, which receives the
-// result, until every sum is within tol of one), then returned as D K D.  K is symmetric: it is filled by halves and K d is summed
-// by columns, which the compiler turns into vector code.
+// result, until every sum is within tol of one), then returned as D K D.  K is symmetric: it
+// is filled by halves and K d is summed by columns, which the compiler turns into vector code.
 std::vector<double> scaled_kernel(const std::vector<double>& mu, int n, double g, std::vector<double>& d,
                                   double tol) {
   const double w = 4.0 * kPi / n;

@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(ScatterCfg<NA>::kThreads, 2)
       // to the total, which keeps the rounding noise of the ~200-term sum close to that of
       // a pairwise sum.  The iteration's attainable accuracy is set by that noise, divided
       // by (1 - rho) ~ 0.07 at the workloads' optics.
-      constexpr int kBlk = (NA % 8 == 0) ? 8 : 4;
+      constexpr int kBlk = 4;
       const float* pcol = P + i;
 #pragma unroll 1
       for (int j0 = 0; j0 < NA; j0 += kBlk) {

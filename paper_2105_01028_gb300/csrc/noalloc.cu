@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(((NA + 31) / 32) * 32)
                       const float* __restrict__ S_prev, float* __restrict__ S_out, float* __restrict__ I_out,
                       float tol, int max_iters, NoAllocScratch* sc) {
   constexpr int W = ((NA + 31) / 32);
-  constexpr int kBlk = (NA % 8 == 0) ? 8 : 4;
+  constexpr int kBlk = 4;
   __shared__ __align__(16) float Xs[2][NA][kNaTile + 4];
   __shared__ float red_d[W][kNaTile], red_s[W][kNaTile];
   __shared__ float e_s[kNaTile], rho_s[kNaTile], best_s[kNaTile];

@@ -312,8 +312,8 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
   bool first_tile = true;
   int claimed = (kMode == kStep && tid == 0) ? atomicAdd(rs.tile_ctr + (n & 1), 1) : 0;
 
-  // Weight of 8 columns from c0 on, as b1_of and form_x read it (volatile or asm loads: hoisted out of the iterations these
-  // tables would cost more registers than there are)
+  // Weight of 8 columns from c0 on, as b1_of and form_x read it (volatile or asm loads: hoisted
+  // out of the iterations these tables would cost more registers than there are)
   // (kBuffers: b1 from the caller's array; in the inner iterations u = 1 - b1 as FP16, kept where
   // Xl was.  b1 itself in FP16 is one in thick voxels, and the corrections then diverge.)
   int v = 0;
@@ -741,7 +741,8 @@ __global__ void __launch_bounds__(Sp<NA>::kThreads, kPer)
         aborted = true;
         break;
       }
-      bool inner = false, fin = !live || (kMode == kAdjoint && al == 0.0f);  // fin: S has taken its last r of this outer
+      bool inner = false;
+      bool fin = !live || (kMode == kAdjoint && al == 0.0f);  // S has taken its last r of this outer
       bool stalled = false, lost = false;  // no further outers; ... and the residual is above its noise floor
       float target = 0.0f, es = 0.0f, crow = 0.0f, xb = 0.0f;  // xb: bound of the operand's elements / 2
       rm = row_max(red_d);

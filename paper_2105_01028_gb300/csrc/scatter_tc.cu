@@ -489,8 +489,9 @@ __global__ void __launch_bounds__(TcThreads<NA>::kThreads, TcThreads<NA>::kPerSm
               so[j + 1] = n1;
               split_bf16x2(fma2(b1, sn, q2), hi[jj / 2], lo[jj / 2]);          // X~ for the next MMA
             }
-            *reinterpret_cast<uint4*>(sAhi + sw128_chunk_off(kM, row, c0 + j8)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            *reinterpret_cast<uint4*>(sAlo + sw128_chunk_off(kM, row, c0 + j8)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            const uint32_t off = sw128_chunk_off(kM, row, c0 + j8);
+            *reinterpret_cast<uint4*>(sAhi + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<uint4*>(sAlo + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
           }
           tmem_st<CH>(t_row + C::SOFF + c0, so);
         }
