@@ -462,7 +462,7 @@ def run_adjoint(args):
             "status": status,
             "roofline": {"kernel": "scatter_split (adjoint mode)", "bound": "tensor", "achieved": solve_ach,
                          "peak": tc_peak, "unit": "TFLOP/s", "frac": solve_ach / tc_peak,
-                         "traffic": measured_traffic("scatter_split_kernel", nv * na),
+                         "traffic": measured_traffic("scatter_split_adjoint", nv * na),
                          "peak_source": pk["_source"]},
             "phases": phases,
             "forward_scatter_tflops": fwd_flops / (ms_fwd * 1e-3) / 1e12,

@@ -33,10 +33,10 @@
 // (3e-8 of it in the weak directions above).  Each row of
 // Ph + Pl + Pm + diag sums to one (the diagonal is a float pair; what the terms drop is 1e-10 of
 // the row), so photons are conserved.
-// Measured against FP64 on the 96x96x64 slab: 1.0e-7 in 2-norm of I and S after two steps;
-// the sum of 192 FP32 products on the CUDA cores that it replaces: 2.3e-7.  Two steps of that
-// slab at 192 directions: 5.8 ms (152 ms before); 100 steps of 16^3 at 48 directions: 5.7 ms
-// (14.0); 110592 voxels of 192 directions on the caller's buffers, cold: 1.19 ms (53.9).
+// Measured against FP64 on the 96x96x64 slab after two steps, in 2-norm: I 9.1e-8, S 8.7e-8;
+// the sums of 192 FP32 products on the CUDA cores that it replaces: 2.1e-7 and 2.3e-7.  Two steps
+// of that slab at 192 directions: 6.38 ms (155 before); 100 steps of 16^3 at 48 directions: 5.1 ms
+// (14.2); 110592 voxels of 192 directions on the caller's buffers, cold: 1.38 ms (54.2).
 //
 // Inner iteration.  Isotropic rebalance as in the other kernels: c = a sum_j b1_j r_j /
 // sum_j (1 - a b1_j) is added to every direction of r; the two-grid iteration that this
@@ -1135,9 +1135,10 @@ cudaError_t launch_split(const GridParams& g, const SplitTables& sp, const BfTab
   constexpr bool kU = kMode != kBuffers;
   const bool uni = kU && g.mut_u >= 0.0f;
   if (g.na == 48) {
-    // two CTAs per SM from 2.5 tiles per SM on (as scatter_tc.cu): 0.273 against 0.307 ms at
-    // 56^3 with varying mu_t, 0.683 against 0.809 at 80^3; one CTA otherwise (0.061 against
-    // 0.073 ms a step at 16^3)
+    // two CTAs per SM from 2.5 tiles per SM on (as scatter_tc.cu; varying mu_t): 0.157 against
+    // 0.170 ms at 40^3 (3.3 tiles per SM), 0.325 against 0.367 at 56^3, 0.809 against 0.945 at
+    // 80^3; one CTA otherwise: 0.093 against 0.101 ms at 32^3 (1.7 tiles per SM), 0.038 against
+    // 0.042 at 16^3 (uniform mu_t)
     const bool two = 2 * ntiles > 5 * sms;
     const int cap = two ? 2 * sms : sms, grid = ntiles < cap ? ntiles : cap;
     auto k = two ? (uni ? scatter_split_kernel<48, kU, kMode, 2> : scatter_split_kernel<48, false, kMode, 2>)
